@@ -847,7 +847,7 @@ __global__ void __launch_bounds__(256) mean_stress(GridInfo g, const T* __restri
 
 // ---------------------------------------------------------------------------
 // Gamma^p table (Def. gamma_tilde_fourier), FP64, one thread per stored
-// frequency of the half spectrum.
+// frequency of the half spectrum (or per set of mirror images).
 // ---------------------------------------------------------------------------
 struct GreenParams {
   int d, nv, ntri, nd;
@@ -864,7 +864,10 @@ struct GreenParams {
   int n_xi;
   double xi[3 * 16];
   int radius;
-  double C4[81];  // C0_ijkl, index ((i*3 + j)*3 + k)*3 + l
+  // acoustic tensor K_ik = C0_ijkl k_j k_l as a quadratic form in k (green_table):
+  // K_e = sum_f Kc[e * n + f] kk_f over the n = d (d + 1) / 2 index pairs
+  // (00, 01, 11 in 2-D; 00, 01, 02, 11, 12, 22 in 3-D)
+  double Kc[36];
   // closed-form path (green_table_iso): C0 isotropic with Lame constants
   // lam0, mu0, and a symbol that is a product of per-axis factors; for a box
   // spline whose directions are all +-e_i, xcount[i] is how often e_i occurs
@@ -907,6 +910,29 @@ __device__ double gen_symbol(const GreenParams& P, const long long* unum) {
   return g;
 }
 
+// per-axis factor g_i at u_i = un / D
+__device__ __forceinline__ double axis_symbol(const GreenParams& P, int i, long long un) {
+  if (P.kind == FH_GEN_BOXSPLINE) {
+    const int c = P.xcount[i];
+    if (c == 0) return 1.0;
+    double f;
+    if (un == 0) f = 1.0;
+    else if (un % P.D == 0) f = 0.0;  // sinc vanishes at the nonzero integers
+    else {
+      const double v = (double)un / (double)P.D;
+      f = sinpi(v) / (3.14159265358979323846 * v);
+    }
+    double g = 1.0;
+    for (int e = 0; e < c; ++e) g *= f;
+    return g;
+  }
+  const long long two = un < 0 ? -2 * un : 2 * un;
+  const double a = (P.kind == FH_GEN_DLVP) ? P.alpha[i] : 0.0;
+  if (a == 0.0) return two < P.D ? 1.0 : (two == P.D ? 0.5 : 0.0);
+  const double u = fabs((double)un / (double)P.D);
+  return fmin(1.0, fmax(0.0, (0.5 + a - u) / (2.0 * a)));
+}
+
 __device__ void mandel_pair(int d, int a, int& i, int& j) {
   if (d == 2) {
     const int I[3] = {0, 1, 0}, J[3] = {0, 1, 1};
@@ -942,109 +968,198 @@ __device__ __forceinline__ void reduce_frequency(const GreenParams& P, long long
   }
 }
 
-__global__ void green_table(GreenParams P, double* __restrict__ G64, float* __restrict__ G32, int* err) {
-  const long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (f >= P.nhalf) return;
-  const int d = P.d;
-  // storage frequency l -> h = V^-T l, reduced into G(M^T)
-  long long l[3] = {0, 0, 0};
-  long long rem = f;
-  l[P.nd - 1] = rem % P.H;
-  rem /= P.H;
-  for (int k = P.nd - 2; k >= 0; --k) { l[k] = rem % P.dims[k]; rem /= P.dims[k]; }
-  long long h[3] = {0, 0, 0}, u[3] = {0, 0, 0};
-  for (int i = 0; i < d; ++i)
-    for (int k = 0; k < P.nd; ++k) h[i] += l[k] * P.Fmap[k][i];
-  for (int i = 0; i < d; ++i) {
-    long long s = 0;
-    for (int c = 0; c < d; ++c) s += P.adjT[i][c] * h[c];
-    u[i] = P.sign * s;
+// storage frequencies of the mirror images of (l0, l1, l2), fm[0] = f itself
+// and -1 where there is no further one (see iso_emit); writes entry t = v to
+// each with the sign (-1)^(how often the reflected axes occur in i, j, p, q)
+template <int DIM>
+__device__ __forceinline__ void mirror_images(const GreenParams& P, long long f, long long l0, long long l1,
+                                              long long l2, int mirror, long long (&fm)[4]) {
+  fm[0] = f;
+  fm[1] = fm[2] = fm[3] = -1;
+  if (!mirror) return;
+  const long long m0 = (P.dims[0] - l0) % P.dims[0];
+  const long long m1 = DIM == 3 ? (P.dims[1] - l1) % P.dims[1] : 0;
+  const bool d0 = m0 != l0, d1 = DIM == 3 && m1 != l1;
+  if (DIM == 3) {
+    if (d0) fm[1] = (m0 * P.dims[1] + l1) * P.H + l2;
+    if (d1) fm[2] = (l0 * P.dims[1] + m1) * P.H + l2;
+    if (d0 && d1) fm[3] = (m0 * P.dims[1] + m1) * P.H + l2;
+  } else if (d0) {
+    fm[1] = m0 * P.H + l2;
   }
-  long long z0[3];
-  for (int i = 0; i < d; ++i) z0[i] = floordiv_ll(2 * u[i] + P.D, 2 * P.D);
-  for (int i = 0; i < d; ++i) {
-    for (int c = 0; c < d; ++c) h[i] -= P.M[c][i] * z0[c];
-    u[i] -= P.D * z0[i];
+}
+__device__ __forceinline__ void mirror_store(const GreenParams& P, int t, double v, int c0, int c1,
+                                             const long long (&fm)[4], double* __restrict__ G64,
+                                             float* __restrict__ G32) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    if (fm[r] < 0) continue;
+    const int flips = ((r & 1) ? c0 : 0) + ((r & 2) ? c1 : 0);
+    const double vr = (flips & 1) ? -v : v;
+    if (!FH_IN(CK_TABLE, (long long)t * P.nhalf + fm[r], (long long)P.ntri * P.nhalf)) continue;
+    G64[(size_t)t * P.nhalf + fm[r]] = vr;
+    G32[(size_t)t * P.nhalf + fm[r]] = (float)vr;
   }
+}
+// storage frequency of thread idx: all of them, or with `mirror` one of each
+// set of mirror images (l_k <= dims_k / 2 on the full axes); false past the end
+template <int DIM>
+__device__ __forceinline__ bool table_frequency(const GreenParams& P, long long idx, int mirror, long long& f,
+                                                long long& l0, long long& l1, long long& l2) {
+  f = idx;
+  l0 = l1 = l2 = 0;
+  if (!mirror) return idx < P.nhalf;
+  const long long n0 = P.dims[0] / 2 + 1, n1 = DIM == 3 ? P.dims[1] / 2 + 1 : 1;
+  if (idx >= n0 * n1 * P.H) return false;
+  l2 = idx % P.H;
+  const long long t = idx / P.H;
+  l1 = DIM == 3 ? t % n1 : 0;
+  l0 = DIM == 3 ? t / n1 : t;
+  f = DIM == 3 ? (l0 * P.dims[1] + l1) * P.H + l2 : l0 * P.H + l2;
+  return true;
+}
+
+// position of the index pair (i, k) in the order 00, 01, 11 or 00, 01, 02, 11, 12, 22
+template <int DIM>
+__device__ __forceinline__ constexpr int pair_index(int i, int k) {
+  const int lo = i < k ? i : k, hi = i < k ? k : i;
+  return lo * DIM - lo * (lo - 1) / 2 + (hi - lo);
+}
+
+constexpr int kMaxAxisAliases = 34;  // 2R + 2 per axis, R <= 16
+
+// Gamma^p for any C0.  With the acoustic tensor K(k) and N = K^-1 = adj K / det K,
+//   Gamma^0_ijpq(k) = (k_i k_q N_jp + k_i k_p N_jq + k_j k_q N_ip + k_j k_p N_iq) / 4,
+// so the alias sum needs only the moments A = sum_z w_z (k k) x N: 6 x 6 numbers in
+// 3-D (3 x 3 in 2-D), held in registers, one multiply-add each per alias; the Mandel
+// entries are formed from them once per frequency.
+//   ORTHO  C0 without normal-shear coupling and with a diagonal shear block: K_ii
+//          has the d squares and K_ik one product (12 of 36 terms in 3-D);
+//   SEP    the symbol is a product of per-axis factors: the orthonormalised weights
+//          factor as well and cost a few symbol evaluations per axis, aliases of zero
+//          weight are skipped (as in green_table_iso); else the symbol is evaluated
+//          per alias and the sum divided by the weights' sum;
+//   mirror (ORTHO and SEP only) M diagonal with the Smith axes M's own: reflecting an
+//          axis changes the signs of single entries, so one frequency of each set of
+//          mirror images is summed (1/4 of them in 3-D, 1/2 in 2-D).
+// Bound by the FP64 pipe: about 87 (ORTHO) or 111 FP64 instructions per alias in 3-D;
+// 64^3, radius 4 (729 aliases), orthotropic C0: 5.3 ms, where a loop over all aliases
+// with the 81-entry tensor and four-term entries in local memory took 180 ms.
+// K is evaluated per alias and not by differences along the alias axis, whose
+// rounding would be relative to the largest |k|^2, not to the one at hand.
+template <int DIM, bool ORTHO, bool SEP>
+__global__ void __launch_bounds__(64, 5) green_table(GreenParams P, double* __restrict__ G64, float* __restrict__ G32,
+                                                     int* err, int mirror, int mirror_geo0, int mirror_geo1) {
+  constexpr int NK = DIM * (DIM + 1) / 2, NV = NK;
+  long long f, l0, l1, l2;
+  if (!table_frequency<DIM>(P, blockIdx.x * (long long)blockDim.x + threadIdx.x, mirror, f, l0, l1, l2)) return;
+  long long h[3], u[3];
+  reduce_frequency(P, f, h, u);
   // aliases k = h + M^T z with |u_i + z_i| <= R + 1/2: z_i in {-R..R+1}, the
   // last one only where u_i = -1/2 (a cube symmetric in M^-T k, so that
   // Gamma^p_{-h} = Gamma^p_h).  Dirichlet and dlVP symbols vanish beyond
   // |u_i| = 1, so R = 1 covers them exactly.
   const int R = (P.kind == FH_GEN_BOXSPLINE) ? P.radius : 1;
-  const int span = 2 * R + 2;
-  int nal = 1;
-  for (int i = 0; i < d; ++i) nal *= span;
-  const double s2 = 1.41421356237309504880;
-  double acc[21];
-  for (int t = 0; t < P.ntri; ++t) acc[t] = 0.0;
-  double wsum = 0.0;
-  for (int ai = 0; ai < nal; ++ai) {
-    long long z[3] = {0, 0, 0};
-    int q = ai;
-    for (int i = 0; i < d; ++i) { z[i] = (q % span) - R; q /= span; }
-    long long un[3];
-    bool inside = true;
-    for (int i = 0; i < d; ++i) {
-      un[i] = u[i] + P.D * z[i];
-      const long long t = un[i] < 0 ? -2 * un[i] : 2 * un[i];
-      inside = inside && t <= (2 * R + 1) * P.D;
-    }
-    if (!inside) continue;
-    const double gv = gen_symbol(P, un);
-    if (gv == 0.0) continue;
-    const double w = gv * gv;
-    wsum += w;
-    double k[3] = {0, 0, 0};
-    bool nonzero = false;
-    for (int i = 0; i < d; ++i) {
-      long long s = h[i];
-      for (int c = 0; c < d; ++c) s += P.M[c][i] * z[c];
-      k[i] = (double)s;
-      nonzero = nonzero || (s != 0);
-    }
-    if (!nonzero) continue;  // Gamma^0(0) = 0
-    // acoustic tensor K_ik = C0_ijkl k_j k_l and its inverse N
-    double K[3][3];
-    for (int i = 0; i < d; ++i)
-      for (int kk = 0; kk < d; ++kk) {
-        double s = 0.0;
-        for (int j = 0; j < d; ++j)
-          for (int ll = 0; ll < d; ++ll) s += P.C4[((i * 3 + j) * 3 + kk) * 3 + ll] * k[j] * k[ll];
-        K[i][kk] = s;
+  int nal[3] = {1, 1, 1};
+  signed char zl[DIM][kMaxAxisAliases];
+  double wl[SEP ? DIM : 1][SEP ? kMaxAxisAliases : 1];
+  double wsum = SEP ? 1.0 : 0.0;
+  for (int i = 0; i < DIM; ++i) {
+    double sum = 0.0;
+    int n = 0;
+    for (int z = -R; z <= R + 1; ++z) {
+      const long long un = u[i] + P.D * z;
+      const long long t = un < 0 ? -2 * un : 2 * un;
+      if (t > (2 * R + 1) * P.D) continue;
+      if constexpr (SEP) {
+        const double g = axis_symbol(P, i, un);
+        if (g == 0.0) continue;
+        wl[i][n] = g * g;
+        sum += g * g;
       }
-    double N[3][3];
-    if (d == 2) {
-      const double det = K[0][0] * K[1][1] - K[0][1] * K[1][0];
-      N[0][0] = K[1][1] / det; N[0][1] = -K[0][1] / det;
-      N[1][0] = -K[1][0] / det; N[1][1] = K[0][0] / det;
-    } else {
-      const double c00 = K[1][1] * K[2][2] - K[1][2] * K[2][1];
-      const double c01 = K[1][2] * K[2][0] - K[1][0] * K[2][2];
-      const double c02 = K[1][0] * K[2][1] - K[1][1] * K[2][0];
-      const double det = K[0][0] * c00 + K[0][1] * c01 + K[0][2] * c02;
-      N[0][0] = c00 / det;
-      N[1][0] = c01 / det;
-      N[2][0] = c02 / det;
-      N[0][1] = (K[0][2] * K[2][1] - K[0][1] * K[2][2]) / det;
-      N[1][1] = (K[0][0] * K[2][2] - K[0][2] * K[2][0]) / det;
-      N[2][1] = (K[0][1] * K[2][0] - K[0][0] * K[2][1]) / det;
-      N[0][2] = (K[0][1] * K[1][2] - K[0][2] * K[1][1]) / det;
-      N[1][2] = (K[0][2] * K[1][0] - K[0][0] * K[1][2]) / det;
-      N[2][2] = (K[0][0] * K[1][1] - K[0][1] * K[1][0]) / det;
+      zl[i][n] = (signed char)z;
+      ++n;
     }
-    // Gamma^0 Mandel entry (a, b): s_a s_b / 4 (k_i N_jp k_q + k_i N_jq k_p + k_j N_ip k_q + k_j N_iq k_p)
-    int t = 0;
-    for (int a = 0; a < P.nv; ++a) {
-      int i, j;
-      mandel_pair(d, a, i, j);
-      const double sa = (i == j) ? 1.0 : s2;
-      for (int bb = a; bb < P.nv; ++bb) {
-        int p, qq;
-        mandel_pair(d, bb, p, qq);
-        const double sb = (p == qq) ? 1.0 : s2;
-        const double v = 0.25 * sa * sb *
-                         (k[i] * N[j][p] * k[qq] + k[i] * N[j][qq] * k[p] + k[j] * N[i][p] * k[qq] + k[j] * N[i][qq] * k[p]);
-        acc[t++] += w * v;
+    if constexpr (SEP) {
+      if (!(sum > 0.0)) wsum = 0.0;
+      for (int q = 0; q < n; ++q) wl[i][q] /= sum;
+    }
+    nal[i] = n;
+  }
+  double A[NK][NK];
+#pragma unroll
+  for (int e = 0; e < NK; ++e)
+#pragma unroll
+    for (int q = 0; q < NK; ++q) A[e][q] = 0.0;
+  for (int a = 0; a < nal[0]; ++a) {
+    for (int b = 0; b < nal[1]; ++b) {
+      const double za = (double)zl[0][a], zb = (double)zl[1][b];
+      double kb[DIM];
+#pragma unroll
+      for (int i = 0; i < DIM; ++i)
+        kb[i] = fma((double)P.M[1][i], zb, fma((double)P.M[0][i], za, (double)h[i]));  // integers: exact
+      double wab = 1.0;
+      if constexpr (SEP) wab = wl[0][a] * wl[1][b];
+      for (int c = 0; c < (DIM == 3 ? nal[2] : 1); ++c) {
+        double k[DIM];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i) k[i] = DIM == 3 ? fma((double)P.M[2][i], (double)zl[DIM - 1][c], kb[i]) : kb[i];
+        double w;
+        if constexpr (SEP) {
+          w = DIM == 3 ? wab * wl[DIM - 1][c] : wab;
+        } else {
+          const long long un[3] = {u[0] + P.D * zl[0][a], u[1] + P.D * zl[1][b],
+                                   DIM == 3 ? u[2] + P.D * zl[DIM - 1][c] : 0};
+          const double gv = gen_symbol(P, un);
+          if (gv == 0.0) continue;
+          w = gv * gv;
+          wsum += w;
+        }
+        double kk[NK], K[NK], N[NK];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i)
+#pragma unroll
+          for (int j = i; j < DIM; ++j) kk[pair_index<DIM>(i, j)] = k[i] * k[j];
+#pragma unroll
+        for (int i = 0; i < DIM; ++i)
+#pragma unroll
+          for (int j = i; j < DIM; ++j) {
+            const int e = pair_index<DIM>(i, j);
+            double s = 0.0;
+            if (ORTHO && i != j) {
+              s = P.Kc[e * NK + e] * kk[e];
+            } else {
+#pragma unroll
+              for (int p = 0; p < DIM; ++p)
+#pragma unroll
+                for (int q = p; q < DIM; ++q)
+                  if (!ORTHO || p == q) s = fma(P.Kc[e * NK + pair_index<DIM>(p, q)], kk[pair_index<DIM>(p, q)], s);
+            }
+            K[e] = s;
+          }
+        double det;
+        if constexpr (DIM == 2) {
+          N[0] = K[2];
+          N[1] = -K[1];
+          N[2] = K[0];
+          det = fma(K[0], K[2], -K[1] * K[1]);
+        } else {
+          N[0] = fma(K[3], K[5], -K[4] * K[4]);
+          N[1] = fma(K[2], K[4], -K[1] * K[5]);
+          N[2] = fma(K[1], K[4], -K[2] * K[3]);
+          N[3] = fma(K[0], K[5], -K[2] * K[2]);
+          N[4] = fma(K[1], K[2], -K[0] * K[4]);
+          N[5] = fma(K[0], K[3], -K[1] * K[1]);
+          det = fma(K[0], N[0], fma(K[1], N[1], K[2] * N[2]));
+        }
+        if (!(det > 0.0)) continue;  // only k = 0 (C0 is positive definite): Gamma^0(0) = 0
+        const double s = w * __drcp_rn(det);
+#pragma unroll
+        for (int q = 0; q < NK; ++q) N[q] *= s;
+#pragma unroll
+        for (int e = 0; e < NK; ++e)
+#pragma unroll
+          for (int q = 0; q < NK; ++q) A[e][q] = fma(kk[e], N[q], A[e][q]);
       }
     }
   }
@@ -1052,12 +1167,25 @@ __global__ void green_table(GreenParams P, double* __restrict__ G64, float* __re
     atomicExch(err, (int)FH_ERR_NO_ONB);
     wsum = 1.0;
   }
-  for (int t = 0; t < P.ntri; ++t) {
-    const double v = acc[t] / wsum;
-    if (!FH_IN(CK_TABLE, (long long)t * P.nhalf + f, (long long)P.ntri * P.nhalf)) continue;
-    G64[(size_t)t * P.nhalf + f] = v;
-    G32[(size_t)t * P.nhalf + f] = (float)v;
-  }
+  const double winv = SEP ? 1.0 : 1.0 / wsum;
+  long long fm[4];
+  mirror_images<DIM>(P, f, l0, l1, l2, mirror, fm);
+  constexpr int I2[3] = {0, 1, 0}, J2[3] = {0, 1, 1}, I3[6] = {0, 1, 2, 1, 0, 0}, J3[6] = {0, 1, 2, 2, 2, 1};
+  int t = 0;
+#pragma unroll
+  for (int a = 0; a < NV; ++a)
+#pragma unroll
+    for (int b = a; b < NV; ++b, ++t) {
+      const int i = DIM == 2 ? I2[a % 3] : I3[a], j = DIM == 2 ? J2[a % 3] : J3[a];
+      const int p = DIM == 2 ? I2[b % 3] : I3[b], q = DIM == 2 ? J2[b % 3] : J3[b];
+      const double sc = 0.25 * ((i == j) ? 1.0 : 1.41421356237309504880) * ((p == q) ? 1.0 : 1.41421356237309504880);
+      const double v = sc * winv *
+                       ((A[pair_index<DIM>(i, q)][pair_index<DIM>(j, p)] + A[pair_index<DIM>(i, p)][pair_index<DIM>(j, q)]) +
+                        (A[pair_index<DIM>(j, q)][pair_index<DIM>(i, p)] + A[pair_index<DIM>(j, p)][pair_index<DIM>(i, q)]));
+      const int c0 = (i == mirror_geo0) + (j == mirror_geo0) + (p == mirror_geo0) + (q == mirror_geo0);
+      const int c1 = (i == mirror_geo1) + (j == mirror_geo1) + (p == mirror_geo1) + (q == mirror_geo1);
+      mirror_store(P, t, v, c0, c1, fm, G64, G32);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1079,31 +1207,6 @@ __global__ void green_table(GreenParams P, double* __restrict__ G64, float* __re
 // aliases of zero weight are skipped.  One thread per stored frequency, aliases
 // in a fixed order (deterministic).
 // ---------------------------------------------------------------------------
-constexpr int kMaxAxisAliases = 34;  // 2R + 2 per axis, R <= 16
-
-// per-axis factor g_i at u_i = un / D
-__device__ __forceinline__ double axis_symbol(const GreenParams& P, int i, long long un) {
-  if (P.kind == FH_GEN_BOXSPLINE) {
-    const int c = P.xcount[i];
-    if (c == 0) return 1.0;
-    double f;
-    if (un == 0) f = 1.0;
-    else if (un % P.D == 0) f = 0.0;  // sinc vanishes at the nonzero integers
-    else {
-      const double v = (double)un / (double)P.D;
-      f = sinpi(v) / (3.14159265358979323846 * v);
-    }
-    double g = 1.0;
-    for (int e = 0; e < c; ++e) g *= f;
-    return g;
-  }
-  const long long two = un < 0 ? -2 * un : 2 * un;
-  const double a = (P.kind == FH_GEN_DLVP) ? P.alpha[i] : 0.0;
-  if (a == 0.0) return two < P.D ? 1.0 : (two == P.D ? 0.5 : 0.0);
-  const double u = fabs((double)un / (double)P.D);
-  return fmin(1.0, fmax(0.0, (0.5 + a - u) / (2.0 * a)));
-}
-
 // index of the fourth moment with exponents (e0, e1, e2) of n_0, n_1, n_2 in
 // the accumulation order of green_table_iso<3>
 __device__ __forceinline__ int moment_index3(int e1, int e2) {
@@ -1145,22 +1248,8 @@ __device__ void iso_emit(const GreenParams& P, const double* Bm, long long f, lo
   const double c4 = 0.25 / P.mu0;
   const double cb = (P.lam0 + P.mu0) / (P.mu0 * (P.lam0 + 2.0 * P.mu0));
   const double s2 = 1.41421356237309504880;
-  // mirror images (s0, s1) of the storage frequency; (0, 0) is f itself
   long long fm[4];
-  fm[0] = f;
-  fm[1] = fm[2] = fm[3] = -1;
-  if (mirror) {
-    const long long m0 = (P.dims[0] - l0) % P.dims[0];
-    const long long m1 = DIM == 3 ? (P.dims[1] - l1) % P.dims[1] : 0;
-    const bool d0 = m0 != l0, d1 = DIM == 3 && m1 != l1;
-    if (DIM == 3) {
-      if (d0) fm[1] = (m0 * P.dims[1] + l1) * P.H + l2;
-      if (d1) fm[2] = (l0 * P.dims[1] + m1) * P.H + l2;
-      if (d0 && d1) fm[3] = (m0 * P.dims[1] + m1) * P.H + l2;
-    } else if (d0) {
-      fm[1] = m0 * P.H + l2;
-    }
-  }
+  mirror_images<DIM>(P, f, l0, l1, l2, mirror, fm);
   int t = 0;
   for (int a = 0; a < P.nv; ++a) {
     int i, j;
@@ -1175,14 +1264,7 @@ __device__ void iso_emit(const GreenParams& P, const double* Bm, long long f, lo
       const double v = sa * sb * (c4 * lin - cb * moment(i, j, p, q));
       const int c0 = (i == mirror_geo0) + (j == mirror_geo0) + (p == mirror_geo0) + (q == mirror_geo0);
       const int c1 = (i == mirror_geo1) + (j == mirror_geo1) + (p == mirror_geo1) + (q == mirror_geo1);
-      for (int r = 0; r < 4; ++r) {
-        if (fm[r] < 0) continue;
-        const int flips = ((r & 1) ? c0 : 0) + ((r & 2) ? c1 : 0);
-        const double vr = (flips & 1) ? -v : v;
-        if (!FH_IN(CK_TABLE, (long long)t * P.nhalf + fm[r], (long long)P.ntri * P.nhalf)) continue;
-        G64[(size_t)t * P.nhalf + fm[r]] = vr;
-        G32[(size_t)t * P.nhalf + fm[r]] = (float)vr;
-      }
+      mirror_store(P, t, v, c0, c1, fm, G64, G32);
       ++t;
     }
   }
@@ -1237,15 +1319,7 @@ __global__ void __launch_bounds__(128) green_table_iso(GreenParams P, double* __
     if (idx >= tet3(n)) return;
     cubic_triple(idx, l0, l1, l2);
     f = (l0 * P.dims[1] + l1) * P.H + l2;
-  } else if (mirror) {
-    const long long n0 = P.dims[0] / 2 + 1, n1 = DIM == 3 ? P.dims[1] / 2 + 1 : 1;
-    if (idx >= n0 * n1 * P.H) return;
-    l2 = idx % P.H;
-    const long long t = idx / P.H;
-    l1 = DIM == 3 ? t % n1 : 0;
-    l0 = DIM == 3 ? t / n1 : t;
-    f = DIM == 3 ? (l0 * P.dims[1] + l1) * P.H + l2 : l0 * P.H + l2;
-  } else if (f >= P.nhalf) {
+  } else if (!table_frequency<DIM>(P, idx, mirror, f, l0, l1, l2)) {
     return;
   }
   long long h[3], u[3];

@@ -1161,14 +1161,11 @@ bool cholesky_ok(const double* A, int n) {
   return true;
 }
 
-// Mandel matrix -> fourth-order tensor C_ijkl (3x3x3x3 storage)
 // The closed-form table kernel (green_table_iso) applies when C0 is isotropic
 // (Mandel: lam0 + 2 mu0 on the normal diagonal, lam0 off it, 2 mu0 on the shear
 // diagonal, zero elsewhere; compared to 1e-15 of its largest entry) and the
-// symbol is a product of per-axis factors: Dirichlet, dlVP, or a box spline
-// whose directions are all +-e_i.  Fills lam0, mu0 and the per-axis direction
-// counts of GP.
-bool closed_form_table(const fh_solver* s, const double* c0, fh::GreenParams* GP) {
+// symbol is a product of per-axis factors.  Fills lam0, mu0 of GP.
+bool isotropic_reference(const fh_solver* s, const double* c0, fh::GreenParams* GP) {
   const int nv = s->g.nv, d = s->g.d;
   const double lam0 = c0[1], mu0 = 0.5 * c0[(nv - 1) * nv + nv - 1];
   double big = 0.0;
@@ -1181,6 +1178,15 @@ bool closed_form_table(const fh_solver* s, const double* c0, fh::GreenParams* GP
       if (std::fabs(c0[a * nv + b] - want) > 1e-15 * big) return false;
     }
   if (!(mu0 > 0.0) || !(lam0 + 2.0 * mu0 > 0.0)) return false;
+  GP->lam0 = lam0;
+  GP->mu0 = mu0;
+  return true;
+}
+
+// The symbol is a product of per-axis factors: Dirichlet, dlVP, or a box
+// spline whose directions are all +-e_i.  Fills the per-axis direction counts.
+bool separable_symbol(const fh_solver* s, fh::GreenParams* GP) {
+  const int d = s->g.d;
   for (int i = 0; i < 3; ++i) GP->xcount[i] = 0;
   if (s->gen.kind == FH_GEN_BOXSPLINE) {
     for (int q = 0; q < s->gen.n_xi; ++q) {
@@ -1194,12 +1200,11 @@ bool closed_form_table(const fh_solver* s, const double* c0, fh::GreenParams* GP
       GP->xcount[axis] += 1;
     }
   }
-  GP->lam0 = lam0;
-  GP->mu0 = mu0;
   return true;
 }
 
-// Mirror symmetry of the table (green_table_iso): M diagonal and every Smith
+// Mirror symmetry of the table (C0 isotropic or orthotropic in the grid axes,
+// separable symbol): M diagonal and every Smith
 // axis one of M's axes (each row of Fmap a single +-1), all d axes non-trivial.
 // geo[k] receives the geometric axis of the full storage axes k = 0 .. d-2.
 bool mirror_axes(const fh_solver* s, int* geo) {
@@ -1221,13 +1226,14 @@ bool mirror_axes(const fh_solver* s, int* geo) {
   return true;
 }
 
-// A 6 x 6 Mandel matrix whose normal-shear blocks are zero and whose shear
-// block is diagonal (isotropic, cubic or orthotropic in the grid axes)
-bool decoupled6(const double* c) {
-  for (int a = 0; a < 6; ++a)
-    for (int b = 0; b < 6; ++b) {
-      const bool structural_zero = ((a < 3) != (b < 3)) || (a >= 3 && b >= 3 && a != b);
-      if (structural_zero && c[a * 6 + b] != 0.0) return false;
+// A Mandel matrix whose normal-shear blocks are zero and whose shear block is
+// diagonal (isotropic, cubic or orthotropic in the grid axes)
+bool decoupled(const double* c, int d) {
+  const int nv = mandel_nv(d);
+  for (int a = 0; a < nv; ++a)
+    for (int b = 0; b < nv; ++b) {
+      const bool structural_zero = ((a < d) != (b < d)) || (a >= d && b >= d && a != b);
+      if (structural_zero && c[a * nv + b] != 0.0) return false;
     }
   return true;
 }
@@ -1248,13 +1254,15 @@ bool cubic_axes(const fh_solver* s, const fh::GreenParams& GP) {
   return true;
 }
 
-void mandel_to_c4(const double* Cm, int d, double* C4) {
+// Coefficients of the acoustic tensor K_ik = C_ijkl k_j k_l as a quadratic
+// form (GreenParams::Kc), from the fourth-order tensor of a Mandel matrix
+void acoustic_form(const double* Cm, int d, double* Kc) {
   const int I2[3] = {0, 1, 0}, J2[3] = {0, 1, 1};
   const int I3[6] = {0, 1, 2, 1, 0, 0}, J3[6] = {0, 1, 2, 2, 2, 1};
   const int* I = d == 2 ? I2 : I3;
   const int* J = d == 2 ? J2 : J3;
   const int nv = mandel_nv(d);
-  for (int q = 0; q < 81; ++q) C4[q] = 0.0;
+  double C4[3][3][3][3] = {};
   for (int a = 0; a < nv; ++a)
     for (int b = 0; b < nv; ++b) {
       const double sa = I[a] == J[a] ? 1.0 : std::sqrt(2.0);
@@ -1263,8 +1271,35 @@ void mandel_to_c4(const double* Cm, int d, double* C4) {
       const int ij[2][2] = {{I[a], J[a]}, {J[a], I[a]}};
       const int kl[2][2] = {{I[b], J[b]}, {J[b], I[b]}};
       for (auto& p : ij)
-        for (auto& q : kl) C4[((p[0] * 3 + p[1]) * 3 + q[0]) * 3 + q[1]] = v;
+        for (auto& q : kl) C4[p[0]][p[1]][q[0]][q[1]] = v;
     }
+  int e = 0;
+  for (int i = 0; i < d; ++i)
+    for (int k = i; k < d; ++k, ++e) {
+      int f = 0;
+      for (int j = 0; j < d; ++j)
+        for (int l = j; l < d; ++l, ++f) {
+          // K is symmetric for a symmetric C0: both orders of (i, k) averaged
+          double v = 0.5 * (C4[i][j][k][l] + C4[k][j][i][l]);
+          if (j != l) v += 0.5 * (C4[i][l][k][j] + C4[k][l][i][j]);
+          Kc[e * nv + f] = v;
+        }
+    }
+}
+
+// the table kernel for any C0 (green_table); mirror images only where C0 has
+// the reflections' symmetry as well
+template <int DIM>
+void launch_green_table(fh_solver* s, const fh::GreenParams& GP, bool ortho, bool separable, bool mirror, const int* geo) {
+  mirror = mirror && ortho && separable;
+  long long n = s->g.nhalf;
+  if (mirror) n = (long long)(s->g.dims[0] / 2 + 1) * (DIM == 3 ? s->g.dims[1] / 2 + 1 : 1) * s->g.H;
+  const unsigned blocks = (unsigned)((n + 63) / 64);
+  auto launch = [&](auto kern) { kern<<<blocks, 64, 0, s->work>>>(GP, s->G64, s->G32, s->err, mirror, geo[0], geo[1]); };
+  if (ortho && separable) launch(fh::green_table<DIM, true, true>);
+  else if (ortho) launch(fh::green_table<DIM, true, false>);
+  else if (separable) launch(fh::green_table<DIM, false, true>);
+  else launch(fh::green_table<DIM, false, false>);
 }
 
 }  // namespace
@@ -1771,14 +1806,14 @@ static fh_status fh_set_reference_impl(fh_solver* s, const double* C0) {
   GP.n_xi = s->gen.n_xi;
   for (int q = 0; q < 3 * 16; ++q) GP.xi[q] = s->gen.xi[q];
   GP.radius = s->gen.alias_radius;
-  mandel_to_c4(c0, d, GP.C4);
+  acoustic_form(c0, d, GP.Kc);
   fh_status rc = join_user(s);
   if (rc != FH_OK) return rc;
   CK(cudaMemsetAsync(s->err, 0, sizeof(int), s->work));
-  const int blocks = (int)((s->g.nhalf + 127) / 128);
-  if (closed_form_table(s, c0, &GP)) {
-    int geo[2] = {-1, -1};
-    const bool mirror = mirror_axes(s, geo);
+  int geo[2] = {-1, -1};
+  const bool separable = separable_symbol(s, &GP);
+  const bool mirror = separable && mirror_axes(s, geo);
+  if (separable && isotropic_reference(s, c0, &GP)) {
     const bool cubic = mirror && cubic_axes(s, GP);
     long long nthreads = s->g.nhalf;
     if (mirror) nthreads = (long long)(s->g.dims[0] / 2 + 1) * (d == 3 ? s->g.dims[1] / 2 + 1 : 1) * s->g.H;
@@ -1795,13 +1830,15 @@ static fh_status fh_set_reference_impl(fh_solver* s, const double* C0) {
       fh::green_table_iso<3><<<mblocks, tpb, 0, s->work>>>(GP, s->G64, s->G32, s->err, mirror, geo[0], geo[1],
                                                            cubic ? 1 : 0);
   } else {
-    fh::green_table<<<blocks, 128, 0, s->work>>>(GP, s->G64, s->G32, s->err);
+    const bool ortho = decoupled(c0, d);
+    if (d == 2) launch_green_table<2>(s, GP, ortho, separable, mirror, geo);
+    else launch_green_table<3>(s, GP, ortho, separable, mirror, geo);
   }
   CK(cudaGetLastError());
   // the constitutive stage of the 3-D row passes skips structural zeros when
   // every phase matrix and C0 have them (then C_p - C0 has them too)
-  s->dc_decoupled = nv == 6 && !s->field && decoupled6(c0);
-  for (int q = 0; q < s->nphase && s->dc_decoupled; ++q) s->dc_decoupled = decoupled6(s->Cp + q * 36);
+  s->dc_decoupled = nv == 6 && !s->field && decoupled(c0, 3);
+  for (int q = 0; q < s->nphase && s->dc_decoupled; ++q) s->dc_decoupled = decoupled(s->Cp + q * 36, 3);
   // stiffness differences C_p - C0
   double dc[kMaxPhases * 36];
   float dcf[kMaxPhases * 36];
