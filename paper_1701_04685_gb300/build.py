@@ -21,7 +21,9 @@ LIB = os.path.join(OUT_DIR, "libffthomog.so")
 LIB_CHECKED = os.path.join(OUT_DIR, "libffthomog_checked.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-SOURCES = ["solver.cu", "lattice.cpp", "noalloc.cu", "fno.cu"]
+SOURCES = ["solver.cu", "cluster64.cu", "cluster32.cu", "genpass64.cu", "genpass32.cu", "lattice.cpp", "noalloc.cu", "fno.cu"]
+# the units whose kernels carry the index checks of the checked build
+CHECKED = ["solver.cu", "cluster64.cu", "cluster32.cu", "genpass64.cu", "genpass32.cu"]
 HEADERS = ["internal.hpp", "kernels.cuh", "fft.cuh", "cluster.cuh", "warprow.cuh", "linewarp.cuh", "colpass2.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -49,25 +51,29 @@ def _compile_cuda(nvcc, src, obj, extra=()):
 
 
 def build_checked(force: bool = False, verbose: bool = False) -> str:
-    """The checked library: solver.cu with -DFH_CHECKED, the other objects
-    from the normal build."""
+    """The checked library: the solver's units with -DFH_CHECKED, the other
+    objects from the normal build."""
     if not force and not _stale(LIB_CHECKED) and not _stale():
         return LIB_CHECKED
     os.makedirs(OUT_DIR, exist_ok=True)
     nvcc = _nvcc()
-    obj = os.path.join(OUT_DIR, "solver_checked.o")
-    cmd = _compile_cuda(nvcc, "solver.cu", obj, ("-DFH_CHECKED",))
-    if verbose:
-        print(" ".join(cmd), file=sys.stderr)
-    # compiled alongside the normal build's objects
-    proc = subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    procs, objs = [], []
+    for src in CHECKED:
+        obj = os.path.join(OUT_DIR, os.path.splitext(src)[0] + "_checked.o")
+        cmd = _compile_cuda(nvcc, src, obj, ("-DFH_CHECKED",))
+        if verbose:
+            print(" ".join(cmd), file=sys.stderr)
+        # compiled alongside the normal build's objects
+        procs.append(subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True))
+        objs.append(obj)
     try:
         build(force=force, verbose=verbose)
     finally:
-        out, _ = proc.communicate()
-    if proc.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + out)
-    objs = [obj] + [os.path.join(OUT_DIR, os.path.splitext(f)[0] + ".o") for f in SOURCES if f != "solver.cu"]
+        outs = [p.communicate()[0] for p in procs]
+    for p, out in zip(procs, outs):
+        if p.returncode != 0:
+            raise RuntimeError("nvcc failed:\n" + out)
+    objs += [os.path.join(OUT_DIR, os.path.splitext(f)[0] + ".o") for f in SOURCES if f not in CHECKED]
     tmp = LIB_CHECKED + ".tmp"
     r = subprocess.run([nvcc, "-shared", *ARCH, "-o", tmp, *objs, "-lcudart"], stdout=subprocess.PIPE,
                        stderr=subprocess.STDOUT, text=True)

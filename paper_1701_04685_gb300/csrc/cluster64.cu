@@ -1,0 +1,30 @@
+// The cluster kernel's FP64 variants (cluster.cuh).
+#include "clusterkern.hpp"
+#include "cluster.cuh"
+
+namespace fh {
+
+template <int NV>
+static const void* variant(int cs, bool pow2) {
+  if (cs == 16)
+    return pow2 ? (const void*)cluster_solve_2d<double, NV, 16, true> : (const void*)cluster_solve_2d<double, NV, 16, false>;
+  return pow2 ? (const void*)cluster_solve_2d<double, NV, 8, true> : (const void*)cluster_solve_2d<double, NV, 8, false>;
+}
+
+const void* cluster_kernel(double, int nv, int cs, bool pow2) { return nv == 3 ? variant<3>(cs, pow2) : variant<6>(cs, pow2); }
+
+cudaError_t cluster_take_check64(CheckRecord* rec) {
+  *rec = CheckRecord{};
+#ifdef FH_CHECKED
+  cudaError_t e = cudaMemcpyFromSymbol(rec, g_check, sizeof(*rec));
+  if (e == cudaSuccess && rec->count != 0ull) {
+    const CheckRecord zero{};
+    e = cudaMemcpyToSymbol(g_check, &zero, sizeof(zero));
+  }
+  return e;
+#else
+  return cudaSuccess;
+#endif
+}
+
+}  // namespace fh

@@ -1,0 +1,35 @@
+// Host side of the two-step passes of general lengths (genpass.cuh), one
+// translation unit per precision so that they compile beside the solver.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "internal.hpp"
+#include "kernels.cuh"
+
+namespace fh {
+
+
+// rows per block of the row pass for rows of L points (L = R1 R2, see gen_length)
+int gen_rows_per_block(double, int L);
+int gen_rows_per_block(float, int L);
+
+// pass along an axis of N points with element stride `stride` (modes as line_pass)
+cudaError_t gen_col(int mode, const GridInfo& g, int N, const double2* tw, double2* S, const double* G,
+                    const LoadState* st, long long stride, int nload, cudaStream_t stream);
+cudaError_t gen_col(int mode, const GridInfo& g, int N, const float2* tw, float2* S, const float* G,
+                    const LoadState* st, long long stride, int nload, cudaStream_t stream);
+
+// row pass (first: no inverse; kinv: the Krylov operator's inverse half)
+cudaError_t gen_row(bool first, bool kinv, const GridInfo& g, const double2* tw, double* E, double2* S,
+                    const uint8_t* phase, const double* dC, Control* ctl, LoadState* st, double* partials, double* hist,
+                    int nload, double* Wout, const double* Yaux, cudaStream_t stream);
+cudaError_t gen_row(bool first, bool kinv, const GridInfo& g, const float2* tw, float* E, float2* S,
+                    const uint8_t* phase, const float* dC, Control* ctl, LoadState* st, double* partials, double* hist,
+                    int nload, float* Wout, const float* Yaux, cudaStream_t stream);
+
+// checked build: the units' violation records (cleared when taken)
+cudaError_t gen_take_check64(CheckRecord* rec);
+cudaError_t gen_take_check32(CheckRecord* rec);
+
+}  // namespace fh

@@ -53,7 +53,7 @@ struct CheckRecord {
 
 #ifdef FH_CHECKED
 static __device__ CheckRecord g_check;
-__device__ __noinline__ bool check_fail(int site, long long i, long long n) {
+static __device__ __noinline__ bool check_fail(int site, long long i, long long n) {
   if (atomicAdd(&g_check.count, 1ull) == 0ull) {
     g_check.site = site;
     g_check.index = i;
@@ -319,7 +319,7 @@ __device__ __forceinline__ void update_state(LoadState& s, double d2, double n2,
   else if (s.iter >= max_iter) { s.status = FH_NOT_CONVERGED; s.done = 1; }
 }
 
-__device__ void advance_state(LoadState& s, Control* ctl, double* hist, int load, double d2, double n2) {
+static __device__ void advance_state(LoadState& s, Control* ctl, double* hist, int load, double d2, double n2) {
   update_state(s, d2, n2, ctl->tol, ctl->max_iter, ctl->stall_window);
   if (s.iter <= ctl->hist_cap) hist[(size_t)load * ctl->hist_cap + (s.iter - 1)] = s.r;
 }
@@ -882,7 +882,7 @@ __device__ __forceinline__ long long floordiv_ll(long long a, long long b) {
 }
 
 // symbol g at u = unum / D  (see fh_generator)
-__device__ double gen_symbol(const GreenParams& P, const long long* unum) {
+static __device__ double gen_symbol(const GreenParams& P, const long long* unum) {
   double g = 1.0;
   if (P.kind == FH_GEN_BOXSPLINE) {
     for (int s = 0; s < P.n_xi; ++s) {
@@ -933,7 +933,7 @@ __device__ __forceinline__ double axis_symbol(const GreenParams& P, int i, long 
   return fmin(1.0, fmax(0.0, (0.5 + a - u) / (2.0 * a)));
 }
 
-__device__ void mandel_pair(int d, int a, int& i, int& j) {
+static __device__ void mandel_pair(int d, int a, int& i, int& j) {
   if (d == 2) {
     const int I[3] = {0, 1, 0}, J[3] = {0, 1, 1};
     i = I[a]; j = J[a];
@@ -1228,7 +1228,7 @@ __device__ __forceinline__ int moment_index3(int e1, int e2) {
 // storage frequencies with l_k <= dims_k / 2 on the full (non-half) axes and
 // write every mirror image: 1/2 (2-D) or 1/4 (3-D) of the alias sums.
 template <int DIM>
-__device__ void iso_emit(const GreenParams& P, const double* Bm, long long f, long long l0, long long l1, long long l2,
+static __device__ void iso_emit(const GreenParams& P, const double* Bm, long long f, long long l0, long long l1, long long l2,
                          int mirror, int mirror_geo0, int mirror_geo1, double* __restrict__ G64,
                          float* __restrict__ G32) {
   auto moment = [&](int i, int j, int p, int q) -> double {
@@ -1482,7 +1482,7 @@ __global__ void __launch_bounds__(128) green_table_iso(GreenParams P, double* __
 struct Tri21 {
   double v[21];
 };
-__global__ void field_prepare(const double* __restrict__ C, Tri21 c0, int ntri, long long m,
+static __global__ void field_prepare(const double* __restrict__ C, Tri21 c0, int ntri, long long m,
                               double* __restrict__ dC64, float* __restrict__ dC32, float* __restrict__ C32) {
   const long long n = (long long)ntri * m;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -1495,7 +1495,7 @@ __global__ void field_prepare(const double* __restrict__ C, Tri21 c0, int ntri, 
 }
 
 // phase ids must index the phase table
-__global__ void check_phases(const uint8_t* __restrict__ phase, long long m, int nphase, int* err) {
+static __global__ void check_phases(const uint8_t* __restrict__ phase, long long m, int nphase, int* err) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x)
     if (phase[i] >= nphase) atomicExch(err, (int)FH_ERR_ARG);
 }

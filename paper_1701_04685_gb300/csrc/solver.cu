@@ -25,6 +25,9 @@
 #include "colpass2.cuh"
 #include "rowpass2.cuh"
 #include "krylov.cuh"
+#include "genpass.hpp"
+#include "gensplit.hpp"
+#include "clusterkern.hpp"
 #include "planewarp.cuh"
 
 namespace fh {
@@ -137,6 +140,7 @@ struct fh_solver {
   bool col2s = true;         // rows and columns of 32, 64 or 128 points: the two-step passes (else the earlier forms)
   int row2[2] = {0, 0};      // 3-D fields with rows of 32, 64 or 128 points: the two-step row pass applies (L), else 0
   int row2_bpl[2] = {1, 1};  // its blocks per load
+  int rowg_bpl[2] = {0, 0};  // > 0: blocks per load of the two-step row pass of general lengths (genpass.cuh)
   bool skip_mean = false;   // the phase in progress is followed by another (mixed mode): its mean stress is not used
   int warp_res[2] = {0, 0};  // resident blocks per SM of that pass
   int sms = 0;               // multiprocessors of the device
@@ -232,6 +236,14 @@ void choose_shapes(fh_solver* s, int prec) {
     const int rb = g.L == 32 ? fh::Row2<4, 8>::RB : fh::Row2<8, 8>::RB;
     s->row2[prec] = g.L;
     s->row2_bpl[prec] = (int)((g.nrows + rb - 1) / rb);
+  }
+  // other 3-D rows of L = R1 R2 points (16 .. 256): the two-step row pass of
+  // general lengths, where neither of the passes above applies
+  s->rowg_bpl[prec] = 0;
+  int r1, r2;
+  if (g.nv == 6 && s->row_warp[prec] == 0 && s->row2[prec] == 0 && fh::gen_split(g.L, &r1, &r2)) {
+    const int rb = prec == FH_PREC_FP64 ? fh::gen_rows_per_block(0.0, g.L) : fh::gen_rows_per_block(0.f, g.L);
+    s->rowg_bpl[prec] = (int)((g.nrows + rb - 1) / rb);
   }
   // FP32 3-D grids whose axis-1 and axis-2 lengths are 32, 64 or 128 points
   // (and whose plane fits in a CTA's shared memory): the fused plane pass
@@ -367,6 +379,15 @@ int col2_len(const fh_solver* s, int prec, int a) {
   return (N == 32 || N == 64 || N == 128) ? N : 0;
 }
 
+// The two-step column pass of general lengths (genpass.cuh) applies to the
+// other axes of R1 R2 points, 16 .. 256, of 3-D fields that neither the
+// compile-time lengths above nor the warp column pass take.
+bool col_gen(const fh_solver* s, int prec, int a) {
+  int r1, r2;
+  return s->col2s && s->g.nv == 6 && col2_len(s, prec, a) == 0 && col_warp_p(s, prec, a) == 0 &&
+         fh::gen_split(s->g.dims[a], &r1, &r2);
+}
+
 // columns per block and resident blocks per SM of the two-step column pass:
 // 8 in FP32, 4 in FP64 (whose tile of 8 would leave one block per SM)
 template <typename T>
@@ -418,6 +439,11 @@ void launch_axis(fh_solver* s, int prec, int a, int mode, int nload) {
   long long n_outer = 1, n_inner = 1;
   for (int k = 0; k < a; ++k) n_outer *= g.dims[k];
   for (int k = a + 1; k + 1 < g.nd; ++k) n_inner *= g.dims[k];
+  if (col_gen(s, prec, a)) {
+    fh::gen_col(mode, g, g.dims[a], twp<T>(s->ax[a]), reinterpret_cast<typename fh::cplx_t<T>::type*>(s->S), Gptr<T>(s), s->st,
+                n_inner * g.H, nload, s->work);
+    return;
+  }
   const long long blocks = (long long)nload * n_outer * n_inner * s->ntiles[prec][a];
   launch_line<T>(s, prec, a, mode, (unsigned)blocks, (int)n_outer, (int)n_inner);
 }
@@ -534,6 +560,17 @@ void launch_row2(fh_solver* s, int prec, int nload, T* X, const T* dC, Control* 
       Wout, Yaux);
 }
 
+// the two-step row pass of general lengths applies (phase-wise stiffness, not
+// switched off by the autotuner's candidate 5)
+bool use_rowg(const fh_solver* s, int prec) { return s->col2s && s->rowg_bpl[prec] > 0 && !s->field; }
+
+template <typename T, bool FIRST, bool KINV>
+int enqueue_rowg(fh_solver* s, int prec, int nload, T* X, const T* dC, Control* ctl, T* Wout, const T* Yaux) {
+  fh::gen_row(FIRST, KINV, s->g, twp<T>(s->ax[s->g.nd - 1]), X, reinterpret_cast<typename fh::cplx_t<T>::type*>(s->S), s->phase,
+              dC, ctl, s->st, s->partials, s->hist, nload, Wout, Yaux, s->work);
+  return s->rowg_bpl[prec];
+}
+
 // returns the blocks per load (the partial sums' layout)
 template <typename T, bool FIRST, bool KINV>
 int enqueue_row2(fh_solver* s, int prec, int nload, T* X, const T* dC, Control* ctl, T* Wout, const T* Yaux) {
@@ -549,6 +586,10 @@ template <typename T, bool FIRST>
 void enqueue_row_pass(fh_solver* s, int prec, int nload) {
   if (use_row2(s, prec) && !(sizeof(T) == 4 && use_plane(s, prec))) {
     enqueue_row2<T, FIRST, false>(s, prec, nload, Eptr<T>(s), dCptr<T>(s), s->ctl, nullptr, nullptr);
+    return;
+  }
+  if (use_rowg(s, prec)) {
+    enqueue_rowg<T, FIRST, false>(s, prec, nload, Eptr<T>(s), dCptr<T>(s), s->ctl, nullptr, nullptr);
     return;
   }
   if constexpr (sizeof(T) == 4) {
@@ -689,6 +730,7 @@ fh_status set_smem_attrs_nv(fh_solver* s, int prec) {
       case 128: CK((set_col2_attrs<T, 8, 16>())); continue;
       default: break;
     }
+    if (col_gen(s, prec, a)) continue;   // sets its own attributes
     if constexpr (sizeof(T) == 4) {
       switch (col_warp_p(s, prec, a)) {
         case 1: CK((set_col_attrs<1>())); continue;
@@ -759,7 +801,7 @@ fh_status run_solve(fh_solver* s, int prec, int nload, int chunk, int max_iter, 
   CK(cudaGetLastError());
   long long launched = 0, extra = 0;
   bool finished = false;
-  if (s->polish && prec == FH_PREC_FP64 && use_row2(s, prec) && !s->plane_on) {
+  if (s->polish && prec == FH_PREC_FP64 && (use_row2(s, prec) || use_rowg(s, prec)) && !s->plane_on) {
     // The FP64 phase of a mixed solve usually stops after its first
     // iteration: that iteration's row pass ends after the E update and the
     // residual (the two-step row pass skips tau and the forward transform).
@@ -830,6 +872,7 @@ int enqueue_row_x(fh_solver* s, int prec, int nload, T* X, Control* ctl, T* Wout
   C* S = reinterpret_cast<C*>(s->S);
   const int last = g.nd - 1;
   if (use_row2(s, prec)) return enqueue_row2<T, FIRST, KINV>(s, prec, nload, X, dC_form0<T>(s), ctl, Wout, Yaux);
+  if (use_rowg(s, prec)) return enqueue_rowg<T, FIRST, KINV>(s, prec, nload, X, dC_form0<T>(s), ctl, Wout, Yaux);
   if constexpr (sizeof(T) == 4) {
     const int P = s->field ? 0 : s->row_warp[prec];
     if (P > 0) {
@@ -978,7 +1021,7 @@ fh_status cluster_fits_nv(fh_solver* s, bool* ok) {
   }
   if (lay.total + 1024 > kMaxSmem) return FH_OK;
   s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0] = gs;
-  auto kern = fh::cluster_solve_2d<T, NV, CS, POW2>;
+  const void* kern = fh::cluster_kernel(T(0), NV, CS, POW2);
   CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
@@ -1061,7 +1104,8 @@ fh_status launch_cluster_nv(fh_solver* s, int nload) {
   cudaLaunchConfig_t cfg = cluster_config<T, NV, CS, POW2>(lay.total, nload, s->work, attr);
   const fh::ClusterTask* tp = s->qtasks;
   unsigned int* np = s->qnext;
-  CK(cudaLaunchKernelEx(&cfg, fh::cluster_solve_2d<T, NV, CS, POW2>, tp, nload, np));
+  void* args[] = {&tp, &nload, &np};
+  CK(cudaLaunchKernelExC(&cfg, fh::cluster_kernel(T(0), NV, CS, POW2), args));
   return FH_OK;
 }
 
@@ -1384,6 +1428,11 @@ fh_status checked(fh_status rc) {
   if (rec.count != 0ull) {
     const fh::CheckRecord zero{};
     CK(cudaMemcpyToSymbol(fh::g_check, &zero, sizeof(zero)));
+  }
+  // the units of the cluster kernel and of the general two-step passes keep records of their own
+  for (auto take : {fh::cluster_take_check64, fh::cluster_take_check32, fh::gen_take_check64, fh::gen_take_check32})
+    if (rec.count == 0ull) CK(take(&rec));
+  if (rec.count != 0ull) {
     fh::set_error(std::string("index check failed (") + std::to_string(rec.count) + " accesses): " +
                   check_site_name(rec.site) + ", index " + std::to_string(rec.index) + " outside [0, " +
                   std::to_string(rec.extent) + ")");
@@ -1583,7 +1632,7 @@ fh_status fh_solver_create(const fh_pattern* p, const fh_generator* gen, int nlo
   CKS(cudaMalloc(&s->ctl, sizeof(Control)));
   CKS(cudaMalloc(&s->st, FH_MAX_LOADS * sizeof(LoadState)));
   const size_t nblk = (size_t)nload_max * std::max({s->row_bpl[0], s->row_bpl[1], s->row_bpl_gen[0], s->row_bpl_gen[1],
-                                                    s->row2_bpl[0], s->row2_bpl[1],
+                                                    s->row2_bpl[0], s->row2_bpl[1], s->rowg_bpl[0], s->rowg_bpl[1],
                                                     2 * g.dims[0]});
   CKS(cudaMalloc(&s->partials, 2 * nblk * sizeof(double)));
   CKS(cudaMalloc(&s->partials2, (size_t)nload_max * kMeanBlocks * fh::MAXV * sizeof(double)));
@@ -2104,7 +2153,7 @@ bool apply_variant(fh_solver* s, int prec, int var) {
   if (var == 0) return true;
   if (var == 4) {
     if (s->row_warp[prec] > 0 && !s->field) return false;   // the warp row pass runs instead
-    if (s->row2[prec] > 0 && !s->field) return false;       // the two-step row pass runs instead
+    if ((s->row2[prec] > 0 || s->rowg_bpl[prec] > 0) && !s->field) return false;   // a two-step row pass runs instead
     const int rpb = 2 * d.rpb_gen;
     if (rpb > g.nrows) return false;
     const int Lp = prec == FH_PREC_FP64 ? fh::padded_len<3>(g.L) : fh::padded_len<4>(g.L);
@@ -2117,12 +2166,12 @@ bool apply_variant(fh_solver* s, int prec, int var) {
   }
   if (var == 5) {
     bool any = false;
-    if (s->row2[prec] > 0 && !s->field) {
+    if ((s->row2[prec] > 0 || s->rowg_bpl[prec] > 0) && !s->field) {
       s->col2s = false;
       any = true;
     }
     for (int a = 0; a + 1 < g.nd; ++a) {
-      if (col2_len(s, prec, a) > 0) {
+      if (col2_len(s, prec, a) > 0 || col_gen(s, prec, a)) {
         s->col2s = false;
         any = true;
       }
@@ -2255,7 +2304,7 @@ fh_status launch_queue(fh_solver* const* solvers, const std::vector<int>& member
   }
   std::stable_sort(tasks.begin(), tasks.end(),
                    [](const fh::ClusterTask& a, const fh::ClusterTask& b) { return a.g.m > b.g.m; });
-  auto kern = fh::cluster_solve_2d<T, NV, CS, POW2>;
+  const void* kern = fh::cluster_kernel(T(0), NV, CS, POW2);
   CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchAttribute attr[1];
@@ -2269,9 +2318,10 @@ fh_status launch_queue(fh_solver* const* solvers, const std::vector<int>& member
   CK(cudaMemcpyAsync(*dtasks, tasks.data(), tasks.size() * sizeof(fh::ClusterTask), cudaMemcpyHostToDevice, stream));
   CK(cudaMemsetAsync(*dnext, 0, sizeof(unsigned int), stream));
   const fh::ClusterTask* tp = *dtasks;
-  const int nt = (int)tasks.size();
+  int nt = (int)tasks.size();
   unsigned int* np = *dnext;
-  CK(cudaLaunchKernelEx(&cfg, kern, tp, nt, np));
+  void* args[] = {&tp, &nt, &np};
+  CK(cudaLaunchKernelExC(&cfg, kern, args));
   return FH_OK;
 }
 
