@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
   __shared__ __align__(16) T dcs[16 * NV * NV];
   __shared__ __align__(16) T dcp[16 * 12];   // the 12 nonzeros of decoupled phase matrices
   __shared__ double red[32];
+  if (!FIRST && !KINV && ctl->all_done) return;   // replays after the last iteration
   const bool decoupled = ctl->decoupled != 0;
   const bool no_fwd = !FIRST && !KINV && ctl->no_forward != 0;
   const int load = blockIdx.x / blocks_per_load;
@@ -221,6 +222,7 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
   const long long row0 = (long long)qb * RB;
   const int nrow = (int)min((long long)RB, g.nrows - row0);
   const bool skip = st[load].done != 0;
+  if ((FIRST || KINV) && skip) return;
   ResAcc<T> acc_d, acc_n;
   const size_t cstrS = (size_t)g.nrows * H, cstrE = (size_t)g.m;
   const long long nS = (long long)ctl->nload * NV * g.nhalf, nE = (long long)ctl->nload * NV * g.m;
@@ -438,24 +440,7 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
   __syncthreads();
   if (s_ticket != gridDim.x - 1) return;
   __threadfence();
-  for (int load2 = 0; load2 < ctl->nload; ++load2) {
-    double a = 0.0, b = 0.0;
-    for (int q = tid; q < blocks_per_load; q += NT) {
-      const size_t blk = (size_t)load2 * blocks_per_load + q;
-      a += __ldcg(&partials[2 * blk]);
-      b += __ldcg(&partials[2 * blk + 1]);
-    }
-    a = block_sum(a, red);
-    b = block_sum(b, red);
-    if (tid == 0 && !st[load2].done) advance_state(st[load2], ctl, hist, load2, a, b);
-  }
-  if (tid == 0) {
-    int all = 1;
-    for (int l = 0; l < ctl->nload; ++l) all &= st[l].done;
-    ctl->all_done = all;
-    ctl->ticket = 0u;
-    __threadfence();
-  }
+  finish_row_pass(ctl, st, partials, hist, blocks_per_load);
 }
 
 inline GenShape gen_shape(int N, bool rows, int H) {

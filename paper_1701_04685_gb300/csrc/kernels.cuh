@@ -324,6 +324,35 @@ static __device__ void advance_state(LoadState& s, Control* ctl, double* hist, i
   if (s.iter <= ctl->hist_cap) hist[(size_t)load * ctl->hist_cap + (s.iter - 1)] = s.r;
 }
 
+// The last block of a row pass: the residual sums of every load in a fixed order,
+// the per-load states, the all-done flag.  One warp per load, so that the loads'
+// reductions run side by side (one load after the other with block reductions took
+// about 2 us a load at the end of every pass).
+__device__ __forceinline__ void finish_row_pass(Control* ctl, LoadState* st, const double* partials, double* hist, int bpl) {
+  const int lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
+  const double2* part = reinterpret_cast<const double2*>(partials);
+  for (int l = (int)(threadIdx.x >> 5); l < ctl->nload; l += nw) {
+    double a = 0.0, b = 0.0;
+#pragma unroll 4
+    for (int q = lane; q < bpl; q += 32) {
+      const double2 v = __ldcg(part + (size_t)l * bpl + q);
+      a += v.x;
+      b += v.y;
+    }
+    a = warp_sum(a);
+    b = warp_sum(b);
+    if (lane == 0 && !st[l].done) advance_state(st[l], ctl, hist, l, a, b);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int all = 1;
+    for (int l = 0; l < ctl->nload; ++l) all &= st[l].done;
+    ctl->all_done = all;
+    ctl->ticket = 0u;
+    __threadfence();
+  }
+}
+
 // ---------------------------------------------------------------------------
 // row pass along the contiguous axis (length L), fused with the pointwise
 // constitutive stage and the residual.
@@ -352,8 +381,10 @@ __global__ void __launch_bounds__(256, PassOcc<T>::value) row_pass(GridInfo g, D
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32];
   __shared__ int s_skip;
+  if (!FIRST && !KINV && ctl->all_done) return;   // replays after the last iteration
   const int load = blockIdx.x / blocks_per_load;
   const int rb = blockIdx.x - load * blocks_per_load;
+  if ((FIRST || KINV) && st[load].done) return;
   const long long row0 = (long long)rb * rpb;
   const int nrow = (int)min((long long)rpb, g.nrows - row0);
   const int L = g.L, H = g.H;
@@ -562,24 +593,7 @@ partial_sums:
   if (s_ticket != gridDim.x - 1) return;
   // 7. last block: fixed-order reduction per load, state update
   __threadfence();
-  for (int load2 = 0; load2 < ctl->nload; ++load2) {
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < blocks_per_load; q += blockDim.x) {
-      const size_t blk = (size_t)load2 * blocks_per_load + q;
-      a += __ldcg(&partials[2 * blk]);
-      b += __ldcg(&partials[2 * blk + 1]);
-    }
-    a = block_sum(a, red);
-    b = block_sum(b, red);
-    if (threadIdx.x == 0 && !st[load2].done) advance_state(st[load2], ctl, hist, load2, a, b);
-  }
-  if (threadIdx.x == 0) {
-    int all = 1;
-    for (int l = 0; l < ctl->nload; ++l) all &= st[l].done;
-    ctl->all_done = all;
-    ctl->ticket = 0u;
-    __threadfence();
-  }
+  finish_row_pass(ctl, st, partials, hist, blocks_per_load);
 }
 
 // ---------------------------------------------------------------------------
@@ -736,6 +750,12 @@ __global__ void green_1d(GridInfo g, cplx<T>* __restrict__ S, const T* __restric
 // each phase, so the block sums E + eps0 over the points of every phase
 // (additions only) and applies the phase matrices to those sums:
 // sum_x C(x):(E(x) + eps0) = sum_p C_p : sum_{x in phase p} (E(x) + eps0).
+// Bound by the FP64 pipe (one conversion and one addition per value): a phase
+// that does not occur in a warp's 32 points costs it nothing, which changes no
+// bit (the additions left out are of zeros).  The block's 28 sums are taken by
+// one warp reduction each and one barrier, and the last block's by one warp per
+// result; the grid is a few blocks per SM (512 blocks a load with a block reduction
+// per sum took 0.49 ms at 64^3 x 6 loads FP32 and 1.13 ms at 128^3 x 6 loads FP64).
 // ---------------------------------------------------------------------------
 constexpr int kMeanPhaseSums = 4;
 
@@ -746,12 +766,14 @@ __global__ void __launch_bounds__(256) mean_stress(GridInfo g, const T* __restri
                                                    double* __restrict__ partials, double* __restrict__ out,
                                                    int blocks_per_load, const double* __restrict__ Cfld = nullptr,
                                                    int nphase = 16) {
-  __shared__ double red[32];
+  constexpr int NSUM = kMeanPhaseSums * (MAXV + 1);
+  __shared__ double red[8][NSUM];
+  __shared__ double tot[NSUM];
   __shared__ unsigned int s_ticket;
   const int load = blockIdx.x / blocks_per_load;
   const int q = blockIdx.x - load * blocks_per_load;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nv = g.nv;
-  double acc[MAXV] = {0, 0, 0, 0, 0, 0};
   double e0[MAXV];
   for (int c = 0; c < nv; ++c) e0[c] = ctl->eps0[load][c];
   const size_t Ebase = (size_t)load * nv * g.m;
@@ -762,86 +784,113 @@ __global__ void __launch_bounds__(256) mean_stress(GridInfo g, const T* __restri
     // contributions are added last, so relabelling two phases (a stiffness
     // field reduced to its distinct matrices) gives the same bits.
     double sp[kMeanPhaseSums][MAXV];
-    long long cnt[kMeanPhaseSums] = {0, 0, 0, 0};
+    int cnt[kMeanPhaseSums] = {0, 0, 0, 0};
 #pragma unroll
     for (int c = 0; c < MAXV; ++c)
 #pragma unroll
       for (int p = 0; p < kMeanPhaseSums; ++p) sp[p][c] = 0.0;
-    for (long long i = (long long)q * blockDim.x + threadIdx.x; i < g.m; i += (long long)blocks_per_load * blockDim.x) {
-      if (!FH_IN(CK_MEAN, (long long)Ebase + (long long)(nv - 1) * g.m + i, (long long)ctl->nload * nv * g.m)) continue;
-      const int ph = phase[i];
+    // whole warps run the loop together (i counts from the warp's first point)
+    const long long step = (long long)blocks_per_load * blockDim.x;
+    for (long long i0 = (long long)q * blockDim.x + 32 * warp; i0 < g.m; i0 += step) {
+      const long long i = i0 + lane;
+      const bool in = i < g.m && FH_IN(CK_MEAN, (long long)Ebase + (long long)(nv - 1) * g.m + i, (long long)ctl->nload * nv * g.m);
+      const int ph = in ? phase[i] : -1;
+      T e[MAXV];
 #pragma unroll
-      for (int p = 0; p < kMeanPhaseSums; ++p) cnt[p] += (ph == p);
+      for (int c = 0; c < MAXV; ++c) e[c] = in && c < nv ? E[Ebase + (size_t)c * g.m + i] : T(0);
+#pragma unroll
+      for (int p = 0; p < kMeanPhaseSums; ++p) {
+        const bool mine = ph == p;
+        if (!__any_sync(0xffffffffu, mine)) continue;
+        if (mine) {
+          ++cnt[p];
+#pragma unroll
+          for (int c = 0; c < MAXV; ++c) sp[p][c] += (double)e[c];
+        }
+      }
+    }
+    // block sums; sum_p C_p : (sum over phase p of E + n_p eps0)
+    for (int p = 0; p < nphase; ++p) {
+      const double n = warp_sum((double)cnt[p]);
+      if (lane == 0) red[warp][p * (MAXV + 1) + MAXV] = n;
+    }
+#pragma unroll
+    for (int p = 0; p < kMeanPhaseSums; ++p) {
+      if (p >= nphase) break;
 #pragma unroll
       for (int c = 0; c < MAXV; ++c) {
-        if (c >= nv) break;
-        const double e = (double)E[Ebase + (size_t)c * g.m + i];
-        // the phase selects the addend, not the addition (FP64 additions are
-        // the scarce resource here: one per phase and component)
-#pragma unroll
-        for (int p = 0; p < kMeanPhaseSums; ++p)
-          if (p < nphase) sp[p][c] += (ph == p) ? e : 0.0;
+        const double v = warp_sum(sp[p][c]);
+        if (lane == 0) red[warp][p * (MAXV + 1) + c] = v;
       }
     }
-    // block sums; thread 0 forms sum_p C_p : (sum over phase p of E + n_p eps0)
-    double n[kMeanPhaseSums], S[kMeanPhaseSums][MAXV];
-    for (int p = 0; p < nphase; ++p) {
-      n[p] = block_sum((double)cnt[p], red);
-      for (int c = 0; c < nv; ++c) S[p][c] = block_sum(sp[p][c], red);
+    __syncthreads();
+    if (threadIdx.x < nphase * (MAXV + 1)) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+      tot[threadIdx.x] = t;
     }
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    if (threadIdx.x < nv) {
+      const int a = threadIdx.x;
+      double acc = 0.0;
       for (int p = 0; p < nphase; ++p) {
-        double v[MAXV];
+        const double* S = tot + p * (MAXV + 1);
+        double t = 0.0;
+        for (int c = 0; c < nv; ++c) t += Cp[((size_t)p * nv + a) * nv + c] * (S[c] + S[MAXV] * e0[c]);
+        acc += t;
+      }
+      partials[(size_t)blockIdx.x * MAXV + a] = acc;
+    }
+  } else {
+    double acc[MAXV] = {0, 0, 0, 0, 0, 0};
+    for (long long i = (long long)q * blockDim.x + threadIdx.x; i < g.m; i += (long long)blocks_per_load * blockDim.x) {
+      double e[MAXV];
+      if (!FH_IN(CK_MEAN, (long long)Ebase + (long long)(nv - 1) * g.m + i, (long long)ctl->nload * nv * g.m)) continue;
+      if (!Cfld && !FH_IN(CK_MEAN, phase[i], 16)) continue;
+      for (int c = 0; c < nv; ++c) e[c] = (double)E[Ebase + (size_t)c * g.m + i] + e0[c];
+      if (Cfld) {   // point-by-point stiffness, upper triangle [tri][m]
+        int t = 0;
+        for (int a = 0; a < nv; ++a)
+          for (int b = a; b < nv; ++b, ++t) {
+            const double cab = Cfld[(size_t)t * g.m + i];
+            acc[a] += cab * e[b];
+            if (b != a) acc[b] += cab * e[a];
+          }
+      } else {
+        const double* C = Cp + (size_t)phase[i] * nv * nv;
         for (int a = 0; a < nv; ++a) {
-          double t = 0.0;
-          for (int c = 0; c < nv; ++c) t += Cp[((size_t)p * nv + a) * nv + c] * (S[p][c] + n[p] * e0[c]);
-          v[a] = t;
+          double s = 0.0;
+          for (int b = 0; b < nv; ++b) s += C[a * nv + b] * e[b];
+          acc[a] += s;
         }
-        for (int a = 0; a < nv; ++a) acc[a] += v[a];
       }
     }
-  } else
-  for (long long i = (long long)q * blockDim.x + threadIdx.x; i < g.m; i += (long long)blocks_per_load * blockDim.x) {
-    double e[MAXV];
-    if (!FH_IN(CK_MEAN, (long long)Ebase + (long long)(nv - 1) * g.m + i, (long long)ctl->nload * nv * g.m)) continue;
-    if (!Cfld && !FH_IN(CK_MEAN, phase[i], 16)) continue;
-    for (int c = 0; c < nv; ++c) e[c] = (double)E[Ebase + (size_t)c * g.m + i] + e0[c];
-    if (Cfld) {   // point-by-point stiffness, upper triangle [tri][m]
-      int t = 0;
-      for (int a = 0; a < nv; ++a)
-        for (int b = a; b < nv; ++b, ++t) {
-          const double cab = Cfld[(size_t)t * g.m + i];
-          acc[a] += cab * e[b];
-          if (b != a) acc[b] += cab * e[a];
-        }
-    } else {
-      const double* C = Cp + (size_t)phase[i] * nv * nv;
-      for (int a = 0; a < nv; ++a) {
-        double s = 0.0;
-        for (int b = 0; b < nv; ++b) s += C[a * nv + b] * e[b];
-        acc[a] += s;
-      }
+#pragma unroll
+    for (int a = 0; a < MAXV; ++a) {
+      const double v = warp_sum(acc[a]);
+      if (lane == 0) red[warp][a] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < nv) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += red[w][threadIdx.x];
+      partials[(size_t)blockIdx.x * MAXV + threadIdx.x] = t;
     }
   }
-  for (int a = 0; a < nv; ++a) {
-    const double v = block_sum(acc[a], red);
-    if (threadIdx.x == 0) partials[(size_t)blockIdx.x * MAXV + a] = v;
-  }
-  if (threadIdx.x == 0) {
-    __threadfence();
-    s_ticket = atomicAdd(&ctl->ticket2, 1u);
-  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_ticket = atomicAdd(&ctl->ticket2, 1u);
   __syncthreads();
   if (s_ticket != gridDim.x - 1) return;
   __threadfence();
-  for (int l = 0; l < ctl->nload; ++l)
-    for (int a = 0; a < nv; ++a) {
-      double s = 0.0;
-      for (int qq = threadIdx.x; qq < blocks_per_load; qq += blockDim.x)
-        s += __ldcg(&partials[((size_t)l * blocks_per_load + qq) * MAXV + a]);
-      s = block_sum(s, red);
-      if (threadIdx.x == 0) out[l * MAXV + a] = s * g.inv_m;
-    }
+  for (int la = warp; la < ctl->nload * nv; la += 8) {
+    const int l = la / nv, a = la - l * nv;
+    double s = 0.0;
+#pragma unroll 4
+    for (int qq = lane; qq < blocks_per_load; qq += 32) s += __ldcg(&partials[((size_t)l * blocks_per_load + qq) * MAXV + a]);
+    s = warp_sum(s);
+    if (lane == 0) out[l * MAXV + a] = s * g.inv_m;
+  }
   if (threadIdx.x == 0) ctl->ticket2 = 0u;
 }
 

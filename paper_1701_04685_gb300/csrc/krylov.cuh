@@ -98,8 +98,9 @@ __global__ void __launch_bounds__(kKryThreads) kry_update_xr(T* __restrict__ x, 
                                                              const Control* ctl, long long m, int nv, int bpl,
                                                              double* __restrict__ part) {
   const int load = blockIdx.x / bpl, q = blockIdx.x - load * bpl;
+  if (st[load].done) return;   // kry_scalars reads no sums of a load that has stopped
   ResAcc<T> arr, arh, axx;
-  if (FH_IN(CK_KRY, load, ctl->nload) && !st[load].done) {
+  if (FH_IN(CK_KRY, load, ctl->nload)) {
     const T alpha = (T)sc[load].alpha, omega = (T)sc[load].omega;
     const size_t base = (size_t)load * nv * m;
     for (int c = 0; c < nv; ++c) {
@@ -159,17 +160,21 @@ template <int STEP>
 __global__ void __launch_bounds__(kKryThreads) kry_scalars(KrylovScal* sc, LoadState* st, Control* ctl,
                                                            double* __restrict__ hist,
                                                            const double* __restrict__ part, int nsum, int bpl) {
-  __shared__ double red[32];
-  for (int l = 0; l < ctl->nload; ++l) {
+  // one warp per load: the loads' reductions run side by side
+  const int lane = threadIdx.x & 31;
+  for (int l = (int)(threadIdx.x >> 5); l < ctl->nload; l += kKryThreads / 32) {
     if (st[l].done) continue;
     double v[3] = {0.0, 0.0, 0.0};
-    for (int j = 0; j < nsum; ++j) {
-      double a = 0.0;
-      for (int qq = threadIdx.x; qq < bpl; qq += blockDim.x) a += part[(size_t)nsum * ((size_t)l * bpl + qq) + j];
-      v[j] = block_sum(a, red);
-      __syncthreads();
+#pragma unroll 2
+    for (int qq = lane; qq < bpl; qq += 32) {
+      const double* pq = part + (size_t)nsum * ((size_t)l * bpl + qq);
+      v[0] += pq[0];
+      v[1] += pq[1];
+      if (nsum > 2) v[2] += pq[2];
     }
-    if (threadIdx.x == 0) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) v[j] = warp_sum(v[j]);
+    if (lane == 0) {
       KrylovScal& k = sc[l];
       if (STEP == 0) {
         k.rho = v[0];
@@ -192,8 +197,8 @@ __global__ void __launch_bounds__(kKryThreads) kry_scalars(KrylovScal* sc, LoadS
         advance_state(st[l], ctl, hist, l, v[0], v[2]);
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
   if (STEP == 3 && threadIdx.x == 0) {
     int all = 1;
     for (int l = 0; l < ctl->nload; ++l) all &= st[l].done;

@@ -341,24 +341,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1) plane_pass_warp6(GridInfo g,
   if (s_ticket != gridDim.x - 1) return;
   __threadfence();
   const int bpl = 2 * N0;
-  for (int load2 = 0; load2 < ctl->nload; ++load2) {
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < bpl; q += blockDim.x) {
-      const size_t blk = (size_t)load2 * bpl + q;
-      a += __ldcg(&partials[2 * blk]);
-      b += __ldcg(&partials[2 * blk + 1]);
-    }
-    a = block_sum(a, red);
-    b = block_sum(b, red);
-    if (threadIdx.x == 0 && !st[load2].done) advance_state(st[load2], ctl, hist, load2, a, b);
-  }
-  if (threadIdx.x == 0) {
-    int all = 1;
-    for (int l = 0; l < ctl->nload; ++l) all &= st[l].done;
-    ctl->all_done = all;
-    ctl->ticket = 0u;
-    __threadfence();
-  }
+  finish_row_pass(ctl, st, partials, hist, bpl);
 }
 
 }  // namespace fh

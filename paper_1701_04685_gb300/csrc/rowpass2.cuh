@@ -71,11 +71,13 @@ __global__ void __launch_bounds__(Row2<R1, R2>::THREADS, sizeof(T) == 4 ? 3 : 1)
   __shared__ __align__(16) T dcp[16 * 12];   // the 12 nonzeros of decoupled phase matrices
   __shared__ double red[32];
   __shared__ int s_skip;
+  if (!FIRST && !KINV && ctl->all_done) return;   // replays after the last iteration
   const bool decoupled = ctl->decoupled != 0;
   const bool no_fwd = !FIRST && !KINV && ctl->no_forward != 0;
   const int load = blockIdx.x / blocks_per_load;
   const int qb = blockIdx.x - load * blocks_per_load;
   const long long row0 = (long long)qb * RB;
+  if ((FIRST || KINV) && st[load].done) return;
   for (int i = threadIdx.x; i < L; i += NT) tw[i] = twg[i];
   if (!KINV) {
     for (int i = threadIdx.x; i < 16 * NV * NV; i += NT) dcs[i] = dC[i];
@@ -337,24 +339,7 @@ __global__ void __launch_bounds__(Row2<R1, R2>::THREADS, sizeof(T) == 4 ? 3 : 1)
   __syncthreads();
   if (s_ticket != gridDim.x - 1) return;
   __threadfence();
-  for (int load2 = 0; load2 < ctl->nload; ++load2) {
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < blocks_per_load; q += blockDim.x) {
-      const size_t blk = (size_t)load2 * blocks_per_load + q;
-      a += __ldcg(&partials[2 * blk]);
-      b += __ldcg(&partials[2 * blk + 1]);
-    }
-    a = block_sum(a, red);
-    b = block_sum(b, red);
-    if (threadIdx.x == 0 && !st[load2].done) advance_state(st[load2], ctl, hist, load2, a, b);
-  }
-  if (threadIdx.x == 0) {
-    int all = 1;
-    for (int l = 0; l < ctl->nload; ++l) all &= st[l].done;
-    ctl->all_done = all;
-    ctl->ticket = 0u;
-    __threadfence();
-  }
+  finish_row_pass(ctl, st, partials, hist, blocks_per_load);
 }
 
 }  // namespace fh

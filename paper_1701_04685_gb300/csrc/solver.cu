@@ -62,7 +62,7 @@ struct NvtxRange {
 };
 
 constexpr int kThreads = 256;
-constexpr int kMeanBlocks = 512;   // blocks per load of the mean-stress reduction
+constexpr int kMeanBlocks = 512;   // most blocks per load of the mean-stress reduction
 constexpr int kHistCap = 65536;
 constexpr size_t kMaxSmem = 227 * 1024;
 constexpr int kMaxPhases = 16;
@@ -119,7 +119,6 @@ struct fh_solver {
   double* mstress = nullptr;
   int* err = nullptr;
   double* scratch64 = nullptr;  // nv*m doubles, for strain copies
-  int* h_flag = nullptr;        // pinned
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev_user = nullptr;
   // host state
   int nphase = 0;
@@ -786,15 +785,76 @@ fh_status get_graph(fh_solver* s, int prec, int nload, int chunk, cudaGraphExec_
   return FH_OK;
 }
 
+// mean stresses of the field X: about four blocks per SM over all loads
+template <typename T>
+void enqueue_mean_stress(fh_solver* s, int nload, const T* X) {
+  const long long most = std::min<long long>((s->g.m + kThreads - 1) / kThreads, kMeanBlocks);
+  const int bpl = (int)std::max<long long>(1, std::min<long long>(most, 4 * std::max(1, s->sms) / nload));
+  fh::mean_stress<T><<<nload * bpl, kThreads, 0, s->work>>>(s->g, X, s->phase, s->Cp64, s->ctl, s->partials2, s->mstress, bpl,
+                                                            s->field ? s->Cf64 : nullptr, s->nphase);
+}
+
+// Iterations until the host looks again: a whole graph replay, or fewer where the
+// loads' residuals (geometric from the last look to this one) or max_iter say that
+// the solve ends sooner: every iteration past the end still launches its passes.
+int next_iterations(const fh_solver* s, int nload, int chunk, int max_iter, double tol, int ran, const double* r_before) {
+  int left = 1;
+  double expect = 1.0;
+  bool known = ran > 0 && tol > 0.0;
+  for (int l = 0; l < nload; ++l) {
+    const LoadState& st = s->h_states[l];
+    if (st.done) continue;
+    left = std::max(left, max_iter - st.iter);
+    if (!known) continue;
+    const double rate = r_before[l] > 0.0 ? std::log(st.r / r_before[l]) / ran : 0.0;
+    if (!(rate < 0.0) || !(st.r > tol)) known = false;
+    else expect = std::max(expect, std::log(tol / st.r) / rate);
+  }
+  int n = std::min(chunk, left);
+  if (known) n = std::min(n, std::max(4, (int)std::ceil(std::min(expect, 1e6)) + 1));
+  return n;
+}
+
+// The iterations of a solve on the passes: graph replays of `chunk` iterations,
+// single launches for a shorter run, until every load has stopped.  `replay` gives
+// the graph, `iterate` launches one iteration.  Returns the iterations launched.
+template <typename Replay, typename Iterate>
+fh_status run_iterations(fh_solver* s, int nload, int chunk, int max_iter, double tol, long long* launched, Replay replay,
+                         Iterate iterate) {
+  double r_before[FH_MAX_LOADS] = {};
+  int ran = 0;
+  for (;;) {
+    const int n = next_iterations(s, nload, chunk, max_iter, tol, ran, r_before);
+    for (int l = 0; l < nload; ++l) r_before[l] = s->h_states[l].r;
+    if (n == chunk) {
+      cudaGraphExec_t exec;
+      fh_status rc = replay(&exec);
+      if (rc != FH_OK) return rc;
+      CK(cudaGraphLaunch(exec, s->work));
+    } else {
+      for (int i = 0; i < n; ++i) iterate();
+      CK(cudaGetLastError());
+    }
+    *launched += n;
+    ran = n;
+    CK(cudaMemcpyAsync(s->h_states, s->st, sizeof(LoadState) * nload, cudaMemcpyDeviceToHost, s->work));
+    CK(cudaStreamSynchronize(s->work));
+    bool all = true;
+    for (int l = 0; l < nload; ++l) all = all && s->h_states[l].done;
+    if (all) return FH_OK;
+    if (*launched > (long long)max_iter + chunk) {
+      fh::set_error("iteration state did not terminate");
+      return FH_ERR_INTERNAL;
+    }
+  }
+}
+
 int line_launches_per_iter(const GridInfo& g) { return g.nd == 1 ? 1 : 1 + 2 * (g.nd - 2); }
 int line_launches_per_iter(const fh_solver* s, int prec) { return use_plane(s, prec) ? 1 : line_launches_per_iter(s->g); }
 
 template <typename T>
-fh_status run_solve(fh_solver* s, int prec, int nload, int chunk, int max_iter, long long* launches) {
+fh_status run_solve(fh_solver* s, int prec, int nload, int chunk, int max_iter, double tol, long long* launches) {
   fh_status rc = set_smem_attrs<T>(s, prec);
-  if (rc != FH_OK) return rc;
-  cudaGraphExec_t exec;
-  rc = get_graph<T>(s, prec, nload, chunk, &exec);
   if (rc != FH_OK) return rc;
   CK(cudaEventRecord(s->ev0, s->work));
   enqueue_row_pass<T, true>(s, prec, nload);
@@ -814,30 +874,26 @@ fh_status run_solve(fh_solver* s, int prec, int nload, int chunk, int max_iter, 
     CK(cudaMemsetAsync(&s->ctl->no_forward, 0, sizeof(int), s->work));
     CK(cudaGetLastError());
     launched = 1;
-    CK(cudaMemcpyAsync(s->h_flag, &s->ctl->all_done, sizeof(int), cudaMemcpyDeviceToHost, s->work));
+    CK(cudaMemcpyAsync(s->h_states, s->st, sizeof(LoadState) * nload, cudaMemcpyDeviceToHost, s->work));
     CK(cudaStreamSynchronize(s->work));
-    finished = *s->h_flag != 0;
+    finished = true;
+    for (int l = 0; l < nload; ++l) finished = finished && s->h_states[l].done;
     if (!finished) {
       enqueue_row_pass<T, true>(s, prec, nload);
       CK(cudaGetLastError());
       extra = 1;
     }
   }
-  while (!finished) {
-    CK(cudaGraphLaunch(exec, s->work));
-    launched += chunk;
-    CK(cudaMemcpyAsync(s->h_flag, &s->ctl->all_done, sizeof(int), cudaMemcpyDeviceToHost, s->work));
-    CK(cudaStreamSynchronize(s->work));
-    if (*s->h_flag) break;
-    if (launched > (long long)max_iter + chunk) {
-      fh::set_error("iteration state did not terminate");
-      return FH_ERR_INTERNAL;
-    }
+  if (!finished) {
+    rc = run_iterations(s, nload, chunk, max_iter, tol, &launched,
+                        [&](cudaGraphExec_t* exec) { return get_graph<T>(s, prec, nload, chunk, exec); },
+                        [&] {
+                          enqueue_line_passes<T>(s, prec, nload);
+                          enqueue_row_pass<T, false>(s, prec, nload);
+                        });
+    if (rc != FH_OK) return rc;
   }
-  const int bpl = std::max(1, (int)std::min<long long>((s->g.m + kThreads - 1) / kThreads, kMeanBlocks));
-  if (!s->skip_mean)
-    fh::mean_stress<T><<<nload * bpl, kThreads, 0, s->work>>>(s->g, Eptr<T>(s), s->phase, s->Cp64, s->ctl, s->partials2,
-                                                              s->mstress, bpl, s->field ? s->Cf64 : nullptr, s->nphase);
+  if (!s->skip_mean) enqueue_mean_stress<T>(s, nload, Eptr<T>(s));
   CK(cudaGetLastError());
   CK(cudaEventRecord(s->ev1, s->work));
   *launches = (s->skip_mean ? 1 : 2) + extra + launched * (1 + line_launches_per_iter(s, prec));
@@ -935,7 +991,7 @@ void enqueue_bicgstab_iteration(fh_solver* s, int prec, int nload) {
 int kry_launches_per_iter(const GridInfo& g) { return 4 + 2 * (2 + line_launches_per_iter(g)) + 3; }
 
 template <typename T>
-fh_status run_bicgstab(fh_solver* s, int prec, int nload, int chunk, int max_iter, long long* launches) {
+fh_status run_bicgstab(fh_solver* s, int prec, int nload, int chunk, int max_iter, double tol, long long* launches) {
   fh_status rc = set_smem_attrs<T>(s, prec);
   if (rc != FH_OK) return rc;
   const int slot = prec == FH_PREC_FP64 ? 0 : 1;
@@ -949,22 +1005,6 @@ fh_status run_bicgstab(fh_solver* s, int prec, int nload, int chunk, int max_ite
   // control block of the operator applications: the solve's, with eps0 = 0
   CK(cudaMemcpyAsync(s->ctl0, s->ctl, sizeof(Control), cudaMemcpyDeviceToDevice, s->work));
   CK(cudaMemsetAsync(s->ctl0->eps0, 0, sizeof(s->ctl0->eps0), s->work));
-  cudaGraphExec_t exec = nullptr;
-  for (auto& e : s->graphs)
-    if (e.prec == prec && e.nload == nload && e.chunk == chunk && e.method == 1) exec = e.exec;
-  if (!exec) {
-    CK(cudaStreamBeginCapture(s->work, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < chunk; ++i) enqueue_bicgstab_iteration<T>(s, prec, nload);
-    cudaGraph_t graph;
-    CK(cudaStreamEndCapture(s->work, &graph));
-    cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-      fh::set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e));
-      return FH_ERR_CUDA;
-    }
-    s->graphs.push_back({prec, nload, chunk, 1, exec});
-  }
   CK(cudaEventRecord(s->ev0, s->work));
   // start: r = b - A E0 (the stress of E0 + eps0 through the passes), rhat = r
   T* x = Eptr<T>(s);
@@ -975,21 +1015,28 @@ fh_status run_bicgstab(fh_solver* s, int prec, int nload, int chunk, int max_ite
   fh::kry_scalars<0><<<1, fh::kKryThreads, 0, s->work>>>(s->ksc, s->st, s->ctl, s->hist, s->kpart, 3, kKryBpl);
   CK(cudaGetLastError());
   long long launched = 0;
-  for (;;) {
-    CK(cudaGraphLaunch(exec, s->work));
-    launched += chunk;
-    CK(cudaMemcpyAsync(s->h_flag, &s->ctl->all_done, sizeof(int), cudaMemcpyDeviceToHost, s->work));
-    CK(cudaStreamSynchronize(s->work));
-    if (*s->h_flag) break;
-    if (launched > (long long)max_iter + chunk) {
-      fh::set_error("iteration state did not terminate");
-      return FH_ERR_INTERNAL;
+  auto graph = [&](cudaGraphExec_t* out) -> fh_status {
+    for (auto& e : s->graphs)
+      if (e.prec == prec && e.nload == nload && e.chunk == chunk && e.method == 1) {
+        *out = e.exec;
+        return FH_OK;
+      }
+    CK(cudaStreamBeginCapture(s->work, cudaStreamCaptureModeThreadLocal));
+    for (int i = 0; i < chunk; ++i) enqueue_bicgstab_iteration<T>(s, prec, nload);
+    cudaGraph_t graph;
+    CK(cudaStreamEndCapture(s->work, &graph));
+    cudaError_t e = cudaGraphInstantiate(out, graph, 0);
+    cudaGraphDestroy(graph);
+    if (e != cudaSuccess) {
+      fh::set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e));
+      return FH_ERR_CUDA;
     }
-  }
-  const int bpl = std::max(1, (int)std::min<long long>((s->g.m + kThreads - 1) / kThreads, kMeanBlocks));
-  if (!s->skip_mean)
-    fh::mean_stress<T><<<nload * bpl, kThreads, 0, s->work>>>(s->g, x, s->phase, s->Cp64, s->ctl, s->partials2,
-                                                              s->mstress, bpl, s->field ? s->Cf64 : nullptr, s->nphase);
+    s->graphs.push_back({prec, nload, chunk, 1, *out});
+    return FH_OK;
+  };
+  rc = run_iterations(s, nload, chunk, max_iter, tol, &launched, graph, [&] { enqueue_bicgstab_iteration<T>(s, prec, nload); });
+  if (rc != FH_OK) return rc;
+  if (!s->skip_mean) enqueue_mean_stress<T>(s, nload, x);
   CK(cudaGetLastError());
   CK(cudaEventRecord(s->ev1, s->work));
   *launches = (2 + line_launches_per_iter(s->g)) + 2 + (s->skip_mean ? 0 : 1) + launched * kry_launches_per_iter(s->g);
@@ -1150,10 +1197,7 @@ fh_status run_solve_cluster(fh_solver* s, int nload, int cs, long long* launches
   CK(cudaEventRecord(s->ev0, s->work));
   fh_status rc = cs == 16 ? launch_cluster<T, 16>(s, nload) : launch_cluster<T, 8>(s, nload);
   if (rc != FH_OK) return rc;
-  const int bpl = std::max(1, (int)std::min<long long>((s->g.m + kThreads - 1) / kThreads, kMeanBlocks));
-  if (!s->skip_mean)
-    fh::mean_stress<T><<<nload * bpl, kThreads, 0, s->work>>>(s->g, Eptr<T>(s), s->phase, s->Cp64, s->ctl, s->partials2,
-                                                              s->mstress, bpl, s->field ? s->Cf64 : nullptr, s->nphase);
+  if (!s->skip_mean) enqueue_mean_stress<T>(s, nload, Eptr<T>(s));
   CK(cudaGetLastError());
   CK(cudaEventRecord(s->ev1, s->work));
   *launches = s->skip_mean ? 1 : 2;
@@ -1172,7 +1216,6 @@ void free_all(fh_solver* s) {
     if (a.tw64) cudaFree(a.tw64);
     if (a.tw32) cudaFree(a.tw32);
   }
-  if (s->h_flag) cudaFreeHost(s->h_flag);
   if (s->h_states) cudaFreeHost(s->h_states);
   if (s->h_ms) cudaFreeHost(s->h_ms);
   if (s->h_tasks) cudaFreeHost(s->h_tasks);
@@ -1357,6 +1400,7 @@ fh_status profile_passes(fh_solver* s, int prec, int nload, int reps, double* ms
   int big = 0x7fffffff;
   double zero = 0.0;
   CK(cudaMemsetAsync(s->st, 0, FH_MAX_LOADS * sizeof(LoadState), s->work));
+  CK(cudaMemsetAsync(&s->ctl->all_done, 0, sizeof(int), s->work));
   CK(cudaMemcpyAsync(&s->ctl->tol, &zero, sizeof(double), cudaMemcpyHostToDevice, s->work));
   CK(cudaMemcpyAsync(&s->ctl->max_iter, &big, sizeof(int), cudaMemcpyHostToDevice, s->work));
   CK(cudaMemcpyAsync(&s->ctl->nload, &nload, sizeof(int), cudaMemcpyHostToDevice, s->work));
@@ -1639,7 +1683,6 @@ fh_status fh_solver_create(const fh_pattern* p, const fh_generator* gen, int nlo
   CKS(cudaMalloc(&s->hist, (size_t)nload_max * kHistCap * sizeof(double)));
   CKS(cudaMalloc(&s->mstress, FH_MAX_LOADS * fh::MAXV * sizeof(double)));
   CKS(cudaMalloc(&s->err, sizeof(int)));
-  CKS(cudaMallocHost(&s->h_flag, sizeof(int)));
   CKS(cudaMallocHost(&s->h_states, FH_MAX_LOADS * sizeof(LoadState)));
   CKS(cudaMallocHost(&s->h_ms, FH_MAX_LOADS * fh::MAXV * sizeof(double)));
   CKS(cudaMalloc(&s->qtasks, FH_MAX_LOADS * sizeof(fh::ClusterTask)));
@@ -1958,6 +2001,8 @@ fh_status begin_phase(fh_solver* s, int nload, const double* eps0, double tol, i
   CK(cudaMemcpyAsync(s->ctl, &h, sizeof(Control), cudaMemcpyHostToDevice, s->work));
   if (start) CK(cudaMemcpyAsync(s->st, start, nload * sizeof(LoadState), cudaMemcpyHostToDevice, s->work));
   else CK(cudaMemsetAsync(s->st, 0, FH_MAX_LOADS * sizeof(LoadState), s->work));
+  // the host's copy, from which run_iterations sizes its replays
+  for (int l = 0; l < nload; ++l) s->h_states[l] = start ? start[l] : LoadState{};
   const size_t nfield = (size_t)nload * nv * s->g.m;
   const unsigned conv_blocks = 1024;
   if (init == 0) {
@@ -1982,11 +2027,11 @@ fh_status begin_phase(fh_solver* s, int nload, const double* eps0, double tol, i
     rc = prec == FH_PREC_FP64 ? run_solve_cluster<double>(s, nload, out->cs, &out->launches)
                               : run_solve_cluster<float>(s, nload, out->cs, &out->launches);
   else if (s->method == 1)
-    rc = prec == FH_PREC_FP64 ? run_bicgstab<double>(s, prec, nload, chunk, max_iter, &out->launches)
-                              : run_bicgstab<float>(s, prec, nload, chunk, max_iter, &out->launches);
+    rc = prec == FH_PREC_FP64 ? run_bicgstab<double>(s, prec, nload, chunk, max_iter, tol, &out->launches)
+                              : run_bicgstab<float>(s, prec, nload, chunk, max_iter, tol, &out->launches);
   else
-    rc = prec == FH_PREC_FP64 ? run_solve<double>(s, prec, nload, chunk, max_iter, &out->launches)
-                              : run_solve<float>(s, prec, nload, chunk, max_iter, &out->launches);
+    rc = prec == FH_PREC_FP64 ? run_solve<double>(s, prec, nload, chunk, max_iter, tol, &out->launches)
+                              : run_solve<float>(s, prec, nload, chunk, max_iter, tol, &out->launches);
   if (rc != FH_OK) return rc;
   CK(cudaMemcpyAsync(s->h_states, s->st, sizeof(LoadState) * nload, cudaMemcpyDeviceToHost, s->work));
   CK(cudaMemcpyAsync(s->h_ms, s->mstress, sizeof(double) * nload * fh::MAXV, cudaMemcpyDeviceToHost, s->work));
@@ -2270,10 +2315,7 @@ namespace {
 // begin_phase does for a solve it runs itself.
 template <typename T>
 fh_status finish_deferred(fh_solver* s, int nload, PhaseOut* out) {
-  const int bpl = std::max(1, (int)std::min<long long>((s->g.m + kThreads - 1) / kThreads, kMeanBlocks));
-  if (!s->skip_mean)
-    fh::mean_stress<T><<<nload * bpl, kThreads, 0, s->work>>>(s->g, Eptr<T>(s), s->phase, s->Cp64, s->ctl, s->partials2,
-                                                              s->mstress, bpl, s->field ? s->Cf64 : nullptr, s->nphase);
+  if (!s->skip_mean) enqueue_mean_stress<T>(s, nload, Eptr<T>(s));
   CK(cudaGetLastError());
   CK(cudaEventRecord(s->ev1, s->work));
   CK(cudaMemcpyAsync(s->h_states, s->st, sizeof(LoadState) * nload, cudaMemcpyDeviceToHost, s->work));

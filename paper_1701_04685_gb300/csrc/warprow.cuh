@@ -523,8 +523,10 @@ __global__ void __launch_bounds__(kWarpRowThreads, (P <= 4 ? 2 : 1)) row_pass_wa
   __shared__ __align__(16) T dcp[16 * 12];   // the 12 nonzeros of decoupled phase matrices
   __shared__ double red[32];
   __shared__ int s_skip;
+  if (!FIRST && !KINV && ctl->all_done) return;   // replays after the last iteration
   const int load = blockIdx.x / blocks_per_load;
   const int qb = blockIdx.x - load * blocks_per_load;
+  if ((FIRST || KINV) && st[load].done) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const bool decoupled = ctl->decoupled != 0;
   for (int i = threadIdx.x; i < L; i += blockDim.x) tw[i] = twg[i];
@@ -719,24 +721,7 @@ __global__ void __launch_bounds__(kWarpRowThreads, (P <= 4 ? 2 : 1)) row_pass_wa
   __syncthreads();
   if (s_ticket != gridDim.x - 1) return;
   __threadfence();
-  for (int load2 = 0; load2 < ctl->nload; ++load2) {
-    double a = 0.0, b = 0.0;
-    for (int q = threadIdx.x; q < blocks_per_load; q += blockDim.x) {
-      const size_t blk = (size_t)load2 * blocks_per_load + q;
-      a += __ldcg(&partials[2 * blk]);
-      b += __ldcg(&partials[2 * blk + 1]);
-    }
-    a = block_sum(a, red);
-    b = block_sum(b, red);
-    if (threadIdx.x == 0 && !st[load2].done) advance_state(st[load2], ctl, hist, load2, a, b);
-  }
-  if (threadIdx.x == 0) {
-    int all = 1;
-    for (int l = 0; l < ctl->nload; ++l) all &= st[l].done;
-    ctl->all_done = all;
-    ctl->ticket = 0u;
-    __threadfence();
-  }
+  finish_row_pass(ctl, st, partials, hist, blocks_per_load);
 }
 
 template <typename T>
