@@ -1,4 +1,4 @@
-// Small DFTs of 4 to 16 points in registers, X_k = sum_t v_t w^{kt},
+// Small DFTs of 4 to 16, 18, 20, 24 and 32 points in registers, X_k = sum_t v_t w^{kt},
 // w = exp(DIR 2 pi i / R), for the two-step passes of any length R1 R2.
 // Lengths with coprime factors take the prime-factor map (no twiddles between
 // the factors), 9 and 16 the Cooley-Tukey split, 7, 11 and 13 the real-pair sums
@@ -112,6 +112,42 @@ __device__ __forceinline__ void dft9(cplx<T>* v) {
 template <int R, int DIR, typename T>
 __device__ __forceinline__ void dft_n(cplx<T>* v);
 
+// 32 = 4 x 8: n = 8 n1 + n2, k = k1 + 4 k2
+template <int DIR, typename T>
+__device__ __forceinline__ void dft32(cplx<T>* v) {
+  auto root = [](int e) {   // exp(DIR 2 pi i e / 32), 0 <= e <= 21
+    const double c[9] = {1.0, 0.9807852804032304491, 0.9238795325112867561, 0.8314696123025452371, 0.7071067811865475244,
+                         0.5555702330196022247, 0.3826834323650897717, 0.1950903220161282678, 0.0};
+    cplx<T> w;
+    const int q = e & 7, s = e >> 3;   // e = 8 s + q: quarter turns
+    const T a = (T)c[q], b = (T)c[8 - q];
+    w.x = s == 0 ? a : s == 1 ? -b : -a;
+    w.y = s == 0 ? b : s == 1 ? a : -b;
+    if (DIR < 0) w.y = -w.y;
+    return w;
+  };
+  cplx<T> y[8][4];
+#pragma unroll
+  for (int n2 = 0; n2 < 8; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < 4; ++n1) y[n2][n1] = v[8 * n1 + n2];
+    dft4<DIR, T>(y[n2]);
+  }
+#pragma unroll
+  for (int n2 = 1; n2 < 8; ++n2)
+#pragma unroll
+    for (int k1 = 1; k1 < 4; ++k1) y[n2][k1] = cmul(y[n2][k1], root(n2 * k1));
+#pragma unroll
+  for (int k1 = 0; k1 < 4; ++k1) {
+    cplx<T> a[8];
+#pragma unroll
+    for (int n2 = 0; n2 < 8; ++n2) a[n2] = y[n2][k1];
+    dft8<DIR, T>(a);
+#pragma unroll
+    for (int k2 = 0; k2 < 8; ++k2) v[k1 + 4 * k2] = a[k2];
+  }
+}
+
 // R = RA RB, coprime: v[(RB n1 + RA n2) mod R] -> X[k] = Z[k mod RA][k mod RB]
 template <int RA, int RB, int DIR, typename T>
 __device__ __forceinline__ void dft_pfa(cplx<T>* v) {
@@ -146,13 +182,26 @@ __device__ __forceinline__ void dft_n(cplx<T>* v) {
   else if constexpr (R == 14) dft_pfa<2, 7, DIR, T>(v);
   else if constexpr (R == 15) dft_pfa<3, 5, DIR, T>(v);
   else if constexpr (R == 16) dft16<DIR, T>(v);
+  else if constexpr (R == 18) dft_pfa<2, 9, DIR, T>(v);
+  else if constexpr (R == 20) dft_pfa<4, 5, DIR, T>(v);
+  else if constexpr (R == 24) dft_pfa<3, 8, DIR, T>(v);
+  else if constexpr (R == 32) dft32<DIR, T>(v);
   else dft_odd<R, DIR, T>(v);
 }
 
-// f(integral_constant R) for a run-time radix 4 .. 16 (the branch is uniform in a block)
+// f(integral_constant R) for a run-time radix, up to RM (the branch is uniform in a block)
 template <int R> struct RadixC { static constexpr int value = R; };
-template <typename F>
+template <int RM, typename F>
 __device__ __forceinline__ void with_radix(int r, F f) {
+  if constexpr (RM > 16) {
+    switch (r) {
+      case 18: f(RadixC<18>{}); return;
+      case 20: f(RadixC<20>{}); return;
+      case 24: f(RadixC<24>{}); return;
+      case 32: f(RadixC<32>{}); return;
+      default: break;
+    }
+  }
   switch (r) {
     case 4: f(RadixC<4>{}); break;
     case 5: f(RadixC<5>{}); break;

@@ -1,6 +1,6 @@
-// Two-step passes for 3-D grids (n_v = 6) and axes of any length N = R1 R2 with
-// 4 <= R1 <= R2 <= 16 (from 16 to 256 points: 100 = 10 x 10, 96 = 8 x 12,
-// 84 = 7 x 12, ...), FP32 and FP64.
+// Two-step passes for axes of any length N = R1 R2 with radices 4 to 16 (and 18,
+// 20, 24, 32 in FP32): 100 = 10 x 10, 96 = 8 x 12, 84 = 7 x 12, 512 = 16 x 32, ...,
+// 2-D and 3-D grids, FP32 and FP64, phase-wise or point-by-point stiffness.
 //
 // The same two steps as line_pass_2s and row_pass_2s (colpass2.cuh,
 // rowpass2.cuh, whose compile-time lengths 32, 64 and 128 stay there), with the
@@ -13,10 +13,12 @@
 // 0.6 ms an iteration against 2.6 ms (a solve of 20 iterations 13.6 against 53.6 ms).
 //
 // Line layout: row k1 at offset (R2 | 1) k1, so that its stride is odd.  Column
-// tiles: CT = 8 (FP32) or 4 (FP64) columns a block and line stride 2 mod 16:
-// the lanes of an access phase (CT columns x 2 entries) fall on distinct banks.
-// Row lines: stride R2 mod 16, so that consecutive entries of consecutive lines
-// follow one another.
+// tiles: CT = 8 columns a block in FP32 3-D, else 4 (FP64: shared memory; 2-D: a
+// 512^2 grid with 3 loads has only 771 columns), line stride 16 / CT mod 16 (FP64:
+// 2): the lanes of an access phase fall on distinct banks.  Row lines: stride R2
+// mod 16, so that consecutive entries of consecutive lines follow one another.
+// 512^2 x 3 loads FP32 with point-by-point stiffness: 63 us an iteration against
+// 132 us (block row pass 79, block line pass 53).
 #pragma once
 
 #include "genpass.hpp"
@@ -24,9 +26,9 @@
 
 namespace fh {
 
-constexpr int kGenThreads32 = 384, kGenThreads64 = 256;
-template <typename T> __host__ __device__ constexpr int gen_ct() { return sizeof(T) == 4 ? 8 : 4; }
-template <typename T> __host__ __device__ constexpr int gen_threads() { return sizeof(T) == 4 ? kGenThreads32 : kGenThreads64; }
+template <typename T, int NV> __host__ __device__ constexpr int gen_ct() { return sizeof(T) == 4 && NV == 6 ? 8 : 4; }
+template <typename T, int NV> __host__ __device__ constexpr int gen_threads() { return sizeof(T) == 4 && NV == 6 ? 384 : 256; }
+template <typename T> __host__ __device__ constexpr int gen_rmax() { return sizeof(T) == 4 ? 32 : 16; }
 
 // q = n / d for n < 2^16, d < 2^16
 struct MulDiv {
@@ -50,12 +52,12 @@ __device__ __forceinline__ C twiddle(const C* tw, int t) {
 }
 
 // MODE 0 forward, 1 inverse, 2 forward + Green step + inverse (axis 0), as line_pass_2s
-template <typename T, int MODE>
-__global__ void __launch_bounds__(gen_threads<T>(), 2)
+template <typename T, int NV, int MODE>
+__global__ void __launch_bounds__(gen_threads<T, NV>(), 2)
     line_pass_gen(GridInfo g, GenShape K, const cplx<T>* __restrict__ twg, cplx<T>* __restrict__ S,
                   const T* __restrict__ Gt, const LoadState* st, long long stride, long long ncols, int nload) {
   using C = cplx<T>;
-  constexpr int NV = 6, NTRI = 21, CT = gen_ct<T>();
+  constexpr int NTRI = NV * (NV + 1) / 2, CT = gen_ct<T, NV>(), RM = gen_rmax<T>();
   constexpr int DIR = MODE == 1 ? 1 : -1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);   // tw[t] = exp(-2 pi i t / N)
@@ -78,7 +80,7 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
   (void)sl0; (void)nS; (void)nT;
 
   // stage A: column w, entry j2, component c: points j2 + R2 j1 from global memory
-  with_radix(K.R1, [&](auto rc) {
+  with_radix<RM>(K.R1, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     for (int a = threadIdx.x; a < NV * CT * K.R2; a += nthr) {
       const int w = a % CT, t = a / CT, c = qdiv(t, K.dR2), j2 = t - c * K.R2;
@@ -101,7 +103,7 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
   __syncthreads();
 
   // stage B: row k1; MODE 0 and 1: frequencies k1 + R1 k2 to global memory, MODE 2: in place
-  with_radix(K.R2, [&](auto rc) {
+  with_radix<RM>(K.R2, [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     for (int b = threadIdx.x; b < NV * CT * K.R1; b += nthr) {
       const int w = b % CT, t = b / CT, c = qdiv(t, K.dR1), k1 = t - c * K.R1;
@@ -158,7 +160,7 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
     }
     __syncthreads();
     // inverse, stage B: row k1, sum over k2, then the twiddles w_N^{+j2 k1}
-    with_radix(K.R2, [&](auto rc) {
+    with_radix<RM>(K.R2, [&](auto rc) {
       constexpr int R = decltype(rc)::value;
       for (int b = threadIdx.x; b < NV * CT * K.R1; b += nthr) {
         const int w = b % CT, t = b / CT, c = qdiv(t, K.dR1), k1 = t - c * K.R1;
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
     });
     __syncthreads();
     // inverse, stage A: entry j2, sum over k1, points j2 + R2 j1 to global memory
-    with_radix(K.R1, [&](auto rc) {
+    with_radix<RM>(K.R1, [&](auto rc) {
       constexpr int R = decltype(rc)::value;
       for (int a = threadIdx.x; a < NV * CT * K.R2; a += nthr) {
         const int w = a % CT, t = a / CT, c = qdiv(t, K.dR2), j2 = t - c * K.R2;
@@ -195,44 +197,47 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
   }
 }
 
-// The row pass (row_pass_2s): a block owns RB rows of one load, 3 RB complex
-// lines; one task per thread and stage (3 RB max(R1, R2) <= threads), so that a
-// stage's results wait in registers for the barrier before they are written.
-template <typename T, bool FIRST, bool KINV>
-__global__ void __launch_bounds__(gen_threads<T>(), 2)
+// The row pass (row_pass_2s): a block owns RB rows of one load, their RB n_v real
+// lines taken in pairs as complex lines (real line f = n_v r + c is component c of
+// row r); one task per thread and stage, so that a stage's results wait in registers
+// for the barrier before they are written.  Cfld (not null): the stiffness point by
+// point, upper triangle [tri][m], instead of the phase table.
+template <typename T, int NV, bool FIRST, bool KINV>
+__global__ void __launch_bounds__(gen_threads<T, NV>(), 2)
     row_pass_gen(GridInfo g, GenShape K, int RB, const cplx<T>* __restrict__ twg, T* __restrict__ E, cplx<T>* __restrict__ S,
                  const uint8_t* __restrict__ phase, const T* __restrict__ dC, Control* ctl, LoadState* st,
                  double* __restrict__ partials, double* __restrict__ hist, int blocks_per_load, T* __restrict__ Wout,
-                 const T* __restrict__ Yaux) {
+                 const T* __restrict__ Yaux, const T* __restrict__ Cfld) {
   static_assert(!(FIRST && KINV), "the inverse-only pass follows a transform");
   using C = cplx<T>;
-  constexpr int NV = 6;
+  constexpr int RM = gen_rmax<T>();
   const int L = K.N, H = g.H, NT = blockDim.x, tid = threadIdx.x;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);
-  C* buf = tw + L;                           // [3 RB][LS]: line 3 r + p = row r, components 2p, 2p + 1
+  C* buf = tw + L;                           // [ceil(RB NV / 2)][LS]
   __shared__ __align__(16) T dcs[16 * NV * NV];
-  __shared__ __align__(16) T dcp[16 * 12];   // the 12 nonzeros of decoupled phase matrices
+  __shared__ __align__(16) T dcp[NV == 6 ? 16 * 12 : 1];   // the 12 nonzeros of decoupled phase matrices
   __shared__ double red[32];
   if (!FIRST && !KINV && ctl->all_done) return;   // replays after the last iteration
-  const bool decoupled = ctl->decoupled != 0;
+  const bool decoupled = NV == 6 && ctl->decoupled != 0;
   const bool no_fwd = !FIRST && !KINV && ctl->no_forward != 0;
   const int load = blockIdx.x / blocks_per_load;
   const int qb = blockIdx.x - load * blocks_per_load;
   const long long row0 = (long long)qb * RB;
   const int nrow = (int)min((long long)RB, g.nrows - row0);
+  const int nreal = nrow * NV, npair = (nreal + 1) >> 1;
   const bool skip = st[load].done != 0;
   if ((FIRST || KINV) && skip) return;
   ResAcc<T> acc_d, acc_n;
   const size_t cstrS = (size_t)g.nrows * H, cstrE = (size_t)g.m;
   const long long nS = (long long)ctl->nload * NV * g.nhalf, nE = (long long)ctl->nload * NV * g.m;
-  const int nB = 3 * RB * K.LS;
+  const int nB = ((RB * NV + 1) >> 1) * K.LS;
   (void)nS; (void)nE; (void)nB;
   if (!skip) {
     for (int i = tid; i < L; i += NT) tw[i] = twg[i];
-    if (!KINV) {
+    if (!KINV && !Cfld) {
       if (decoupled) {
-        for (int i = tid; i < 16 * 12; i += NT) dcp[i] = decoupled_entry(dC + (i / 12) * NV * NV, i % 12);
+        for (int i = tid; i < 16 * 12; i += NT) dcp[i % (NV == 6 ? 192 : 1)] = decoupled_entry(dC + (i / 12) * NV * NV, i % 12);
       } else {
         for (int i = tid; i < 16 * NV * NV; i += NT) dcs[i] = dC[i];
       }
@@ -248,14 +253,19 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
     // stage A and B tasks of this thread
     const int la = qdiv(tid, K.dR2), j2 = tid - la * K.R2;
     const int lb = qdiv(tid, K.dR1), k1 = tid - lb * K.R1;
-    const bool onA = la < 3 * nrow, onB = lb < 3 * nrow;
+    const bool onA = la < npair, onB = lb < npair;
     C* lineA = buf + la * K.LS;
     C* lineB = buf + lb * K.LS;
+    // half spectrum of real line f of this block (row row0 + f / NV, component f % NV)
+    auto spec = [&](int f) -> long long {
+      const int r = f / NV;
+      return (long long)(f - r * NV) * (long long)cstrS + (row0 + r) * H;
+    };
 
     // one stage with its barrier: values to registers, then to the other layout
     auto stageB = [&](auto dir) {   // row k1 -> points or frequencies k1 + R1 k2 in natural order
       constexpr int DIR = decltype(dir)::value;
-      with_radix(K.R2, [&](auto rc) {
+      with_radix<RM>(K.R2, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         C v[R];
         if (onB && FH_IN(CK_ROW_SMEM, lb * K.LS + k1 * K.RS + R - 1, nB)) {
@@ -274,25 +284,24 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
 
     if (!FIRST) {
       // inverse, stage A: Z[j2 + R2 j1] = A + i B from the half spectra (conjugate mirror for k > L / 2)
-      with_radix(K.R1, [&](auto rc) {
+      with_radix<RM>(K.R1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
-        const int r = la / 3, p = la - 3 * r;
-        if (onA && FH_IN(CK_ROW_S, ((long long)load * NV + 2 * p + 1) * (long long)cstrS + (row0 + r) * H + H - 1, nS) &&
+        if (onA && FH_IN(CK_ROW_S, (long long)load * NV * (long long)cstrS + spec(2 * la) + H - 1, nS) &&
             FH_IN(CK_ROW_SMEM, la * K.LS + (R - 1) * K.RS + j2, nB)) {
-          const C* SA = Sl + (size_t)(2 * p) * cstrS + (row0 + r) * H;
-          const C* SB = SA + cstrS;
-          C v[R], vb[R];
+          const C* SA = Sl + spec(2 * la);
+          const bool two = NV == 6 || 2 * la + 1 < nreal;   // an odd number of real lines: the last pair has one
+          const C* SB = two ? Sl + spec(2 * la + 1) : SA;
+          const T tb = two ? T(1) : T(0);
+          C v[R];
 #pragma unroll
           for (int j = 0; j < R; ++j) {
             const int k = j2 + K.R2 * j;
-            const int kk = 2 * k <= L ? k : L - k;
-            v[j] = SA[kk];
-            vb[j] = SB[kk];
-          }
-#pragma unroll
-          for (int j = 0; j < R; ++j) {
-            const T s = 2 * (j2 + K.R2 * j) <= L ? T(1) : T(-1);
-            const C A = v[j], B = vb[j];
+            const bool lo = 2 * k <= L;
+            const int kk = lo ? k : L - k;
+            const T s = lo ? T(1) : T(-1);
+            const C A = SA[kk];
+            C B = SB[kk];
+            if (NV != 6) { B.x *= tb; B.y *= tb; }
             v[j].x = A.x - s * B.y;
             v[j].y = s * A.y + B.x;
           }
@@ -311,9 +320,11 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
       const int r = qdiv(idx, K.dN), x = idx - r * L;
       const size_t pt = (size_t)(row0 + r) * L + x;
       if (!(FH_IN(CK_ROW_E, (long long)load * NV * (long long)cstrE + (NV - 1) * (long long)cstrE + (long long)pt, nE) &&
-            FH_IN(CK_ROW_PHASE, (long long)pt, g.m) && FH_IN(CK_ROW_SMEM, (3 * r + 2) * K.LS + x, nB)))
+            FH_IN(CK_ROW_PHASE, (long long)pt, g.m) && FH_IN(CK_ROW_SMEM, ((r * NV + NV - 1) >> 1) * K.LS + x, nB)))
         continue;
-      C* ln = buf + (3 * r) * K.LS + x;
+      const int f0 = r * NV;
+      T* ln = reinterpret_cast<T*>(buf + x);   // real line f at ln[(f >> 1) 2 LS + (f & 1)]
+      auto at = [&](int c) -> T& { return ln[(size_t)((f0 + c) >> 1) * 2 * K.LS + ((f0 + c) & 1)]; };
       T ev[NV];
 #pragma unroll
       for (int c = 0; c < NV; ++c) ev[c] = El[c * cstrE + pt];
@@ -321,16 +332,11 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
         const T* Yl = Yaux ? Yaux + (size_t)load * NV * cstrE : El;
         T* Wl = Wout + (size_t)load * NV * cstrE;
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-          const C z = ln[p * K.LS];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int c = 2 * p + h;
-            const T wv = ev[c] - (h ? z.y : z.x) * scale;
-            Wl[c * cstrE + pt] = wv;
-            acc_d.add_prod(wv, Yaux ? Yl[c * cstrE + pt] : ev[c]);
-            acc_n.add_sq(wv);
-          }
+        for (int c = 0; c < NV; ++c) {
+          const T wv = ev[c] - at(c) * scale;
+          Wl[c * cstrE + pt] = wv;
+          acc_d.add_prod(wv, Yaux ? Yl[c * cstrE + pt] : ev[c]);
+          acc_n.add_sq(wv);
         }
         continue;
       }
@@ -341,13 +347,8 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
       } else {
         T rd = T(0), rn = T(0);
 #pragma unroll
-        for (int p = 0; p < 3; ++p) {
-          const C z = ln[p * K.LS];
-          en[2 * p] = z.x * scale;
-          en[2 * p + 1] = z.y * scale;
-        }
-#pragma unroll
         for (int c = 0; c < NV; ++c) {
+          en[c] = at(c) * scale;
           if (incremental) en[c] += ev[c];
           const T dd = en[c] - ev[c], nn = en[c] + e0[c];
           rd = fma(dd, dd, rd);
@@ -358,36 +359,46 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
         acc_n.add(rn);
       }
       if (no_fwd) continue;
-      int ph = phase[pt];
-      if (!FH_IN(CK_ROW_PHASE, ph, 16)) ph = 0;
       T xv[NV], tau[NV];
 #pragma unroll
       for (int b = 0; b < NV; ++b) xv[b] = en[b] + e0[b];
-      if (decoupled) {
-        stress6_decoupled<T>(dcp + ph * 12, xv, tau);
+      if (Cfld) {
+#pragma unroll
+        for (int a = 0; a < NV; ++a) tau[a] = T(0);
+#pragma unroll
+        for (int a = 0; a < NV; ++a)
+#pragma unroll
+          for (int b = a; b < NV; ++b) {
+            const T cab = Cfld[(size_t)(a * NV - (a * (a - 1)) / 2 + (b - a)) * g.m + pt];
+            tau[a] = fma(cab, xv[b], tau[a]);
+            if (b != a) tau[b] = fma(cab, xv[a], tau[b]);
+          }
       } else {
-        const T* dc = dcs + ph * NV * NV;
+        int ph = phase[pt];
+        if (!FH_IN(CK_ROW_PHASE, ph, 16)) ph = 0;
+        if (NV == 6 && decoupled) {
+          if constexpr (NV == 6) stress6_decoupled<T>(dcp + ph * 12, xv, tau);
+        } else {
+          const T* dc = dcs + ph * NV * NV;
 #pragma unroll
-        for (int a = 0; a < NV; ++a) {
-          T t = T(0);
+          for (int a = 0; a < NV; ++a) {
+            T t = T(0);
 #pragma unroll
-          for (int b = 0; b < NV; ++b) t = fma(dc[a * NV + b], xv[b], t);
-          tau[a] = t;
+            for (int b = 0; b < NV; ++b) t = fma(dc[a * NV + b], xv[b], t);
+            tau[a] = t;
+          }
         }
       }
 #pragma unroll
-      for (int p = 0; p < 3; ++p) {
-        C z;
-        z.x = tau[2 * p];
-        z.y = tau[2 * p + 1];
-        ln[p * K.LS] = z;
-      }
+      for (int c = 0; c < NV; ++c) at(c) = tau[c];
     }
+    if (NV != 6 && !KINV && (nreal & 1))   // the imaginary part of the last pair
+      for (int x = tid; x < L; x += NT) buf[(npair - 1) * K.LS + x].y = T(0);
 
     if (!KINV && !no_fwd) {
       __syncthreads();
       // forward, stage A: points j2 + R2 j1 -> row layout with the twiddles
-      with_radix(K.R1, [&](auto rc) {
+      with_radix<RM>(K.R1, [&](auto rc) {
         constexpr int R = decltype(rc)::value;
         C v[R];
         if (onA && FH_IN(CK_ROW_SMEM, la * K.LS + j2 + K.R2 * (R - 1), nB)) {
@@ -405,11 +416,10 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
       });
       __syncthreads();
       stageB(RadixC<-1>{});
-      // split each line's spectrum into its two components' half spectra
-      for (int idx = tid; idx < 3 * nrow * H; idx += NT) {
+      // split each line's spectrum into the half spectra of its two real lines
+      for (int idx = tid; idx < npair * H; idx += NT) {
         const int line = qdiv(idx, K.dH), k = idx - line * H;
-        const int r = line / 3, p = line - 3 * r;
-        if (!FH_IN(CK_ROW_S, ((long long)load * NV + 2 * p + 1) * (long long)cstrS + (row0 + r) * H + k, nS)) continue;
+        if (!FH_IN(CK_ROW_S, (long long)load * NV * (long long)cstrS + spec(2 * line) + k, nS)) continue;
         const C* ln = buf + line * K.LS;
         const C zk = ln[k];
         const C zm = ln[k == 0 ? 0 : L - k];
@@ -418,9 +428,8 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
         A.y = T(0.5) * (zk.y - zm.y);
         B.x = T(0.5) * (zk.y + zm.y);
         B.y = T(-0.5) * (zk.x - zm.x);
-        C* SA = Sl + (size_t)(2 * p) * cstrS + (row0 + r) * H + k;
-        SA[0] = A;
-        SA[cstrS] = B;
+        Sl[spec(2 * line) + k] = A;
+        if (NV == 6 || 2 * line + 1 < nreal) Sl[spec(2 * line + 1) + k] = B;
       }
     }
   }
@@ -443,12 +452,12 @@ __global__ void __launch_bounds__(gen_threads<T>(), 2)
   finish_row_pass(ctl, st, partials, hist, blocks_per_load);
 }
 
-inline GenShape gen_shape(int N, bool rows, int H) {
+inline GenShape gen_shape(int N, bool fp32, bool rows, int ct, int H) {
   GenShape K{};
   K.N = N;
-  gen_split(N, &K.R1, &K.R2);
+  gen_split(N, fp32, &K.R1, &K.R2);
   K.RS = K.R2 | 1;
-  const int need = K.R1 * K.RS, mod = rows ? K.R2 % 16 : 2;
+  const int need = K.R1 * K.RS, mod = rows ? K.R2 % 16 : fp32 ? 16 / ct : 2;
   K.LS = need + ((mod - need) % 16 + 16) % 16;
   K.dR1 = make_muldiv(K.R1);
   K.dR2 = make_muldiv(K.R2);
@@ -457,24 +466,28 @@ inline GenShape gen_shape(int N, bool rows, int H) {
   return K;
 }
 
-// rows per block: one task per thread, and two blocks' lines in shared memory
-template <typename T>
-int gen_rb(int L) {
-  const GenShape K = gen_shape(L, true, 1);
-  int rb = std::max(1, gen_threads<T>() / (3 * K.R2));
-  while (rb > 1 && (size_t)(L + 3 * rb * K.LS) * 2 * sizeof(T) > 96 * 1024) --rb;
-  return rb;
+// rows per block: one task per thread, two blocks' lines in shared memory, and
+// (few rows) about two blocks per SM
+template <typename T, int NV>
+int gen_rb(int L, long long rows_of_all_loads) {
+  constexpr bool fp32 = sizeof(T) == 4;
+  const GenShape K = gen_shape(L, fp32, true, 1, 1);
+  int rb = std::max(1, 2 * (gen_threads<T, NV>() / K.R2) / NV);
+  auto lines = [](int r) { return (r * NV + 1) / 2; };
+  while (rb > 1 && (lines(rb) * K.R2 > gen_threads<T, NV>() || (size_t)(L + lines(rb) * K.LS) * 2 * sizeof(T) > 96 * 1024)) --rb;
+  const long long want = (rows_of_all_loads + 2 * 152 - 1) / (2 * 152);
+  return (int)std::max<long long>(1, std::min<long long>(rb, want));
 }
 
-template <typename T>
+template <typename T, int NV>
 cudaError_t gen_col_t(int mode, const GridInfo& g, int N, const cplx<T>* tw, cplx<T>* S, const T* G, const LoadState* st,
                       long long stride, int nload, cudaStream_t stream) {
-  constexpr int CT = gen_ct<T>();
-  const GenShape K = gen_shape(N, false, 1);
+  constexpr int CT = gen_ct<T, NV>(), TH = gen_threads<T, NV>();
+  const GenShape K = gen_shape(N, sizeof(T) == 4, false, CT, 1);
   const long long ncols = g.nhalf / N, tiles = (ncols + CT - 1) / CT;
-  const size_t sm = (size_t)(N + 6 * CT * K.LS) * 2 * sizeof(T);
-  // a stage's 6 CT R2 tasks in equal rounds
-  const int tasks = 6 * CT * K.R2, rounds = (tasks + gen_threads<T>() - 1) / gen_threads<T>();
+  const size_t sm = (size_t)(N + NV * CT * K.LS) * 2 * sizeof(T);
+  // a stage's NV CT R2 tasks in equal rounds
+  const int tasks = NV * CT * K.R2, rounds = (tasks + TH - 1) / TH;
   const int threads = ((tasks + rounds - 1) / rounds + 31) / 32 * 32;
   auto launch = [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
@@ -482,28 +495,31 @@ cudaError_t gen_col_t(int mode, const GridInfo& g, int N, const cplx<T>* tw, cpl
     kern<<<(unsigned)(tiles * nload), threads, sm, stream>>>(g, K, tw, S, G, st, stride, ncols, nload);
     return cudaGetLastError();
   };
-  if (mode == 0) return launch(line_pass_gen<T, 0>);
-  if (mode == 1) return launch(line_pass_gen<T, 1>);
-  return launch(line_pass_gen<T, 2>);
+  if constexpr (NV == 6) {   // 2-D grids have axis 0 only
+    if (mode == 0) return launch(line_pass_gen<T, NV, 0>);
+    if (mode == 1) return launch(line_pass_gen<T, NV, 1>);
+  }
+  return launch(line_pass_gen<T, NV, 2>);
 }
 
-template <typename T>
+template <typename T, int NV>
 cudaError_t gen_row_t(bool first, bool kinv, const GridInfo& g, const cplx<T>* tw, T* E, cplx<T>* S, const uint8_t* phase,
-                      const T* dC, Control* ctl, LoadState* st, double* partials, double* hist, int nload, T* Wout,
-                      const T* Yaux, cudaStream_t stream) {
-  const GenShape K = gen_shape(g.L, true, g.H);
-  const int rb = gen_rb<T>(g.L), bpl = (int)((g.nrows + rb - 1) / rb);
-  const size_t sm = (size_t)(g.L + 3 * rb * K.LS) * 2 * sizeof(T);
-  const int threads = (3 * rb * K.R2 + 31) / 32 * 32;
+                      const T* dC, Control* ctl, LoadState* st, double* partials, double* hist, int nload, int rb, T* Wout,
+                      const T* Yaux, const T* Cfld, cudaStream_t stream) {
+  const GenShape K = gen_shape(g.L, sizeof(T) == 4, true, 1, g.H);
+  const int bpl = (int)((g.nrows + rb - 1) / rb), lines = (rb * NV + 1) / 2;
+  const size_t sm = (size_t)(g.L + lines * K.LS) * 2 * sizeof(T);
+  const int threads = (lines * K.R2 + 31) / 32 * 32;
   auto launch = [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)(nload * bpl), threads, sm, stream>>>(g, K, rb, tw, E, S, phase, dC, ctl, st, partials, hist, bpl, Wout, Yaux);
+    kern<<<(unsigned)(nload * bpl), threads, sm, stream>>>(g, K, rb, tw, E, S, phase, dC, ctl, st, partials, hist, bpl, Wout, Yaux,
+                                                           Cfld);
     return cudaGetLastError();
   };
-  if (first) return launch(row_pass_gen<T, true, false>);
-  if (kinv) return launch(row_pass_gen<T, false, true>);
-  return launch(row_pass_gen<T, false, false>);
+  if (first) return launch(row_pass_gen<T, NV, true, false>);
+  if (kinv) return launch(row_pass_gen<T, NV, false, true>);
+  return launch(row_pass_gen<T, NV, false, false>);
 }
 
 }  // namespace fh

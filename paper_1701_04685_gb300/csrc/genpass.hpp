@@ -10,9 +10,10 @@
 namespace fh {
 
 
-// rows per block of the row pass for rows of L points (L = R1 R2, see gen_length)
-int gen_rows_per_block(double, int L);
-int gen_rows_per_block(float, int L);
+// rows per block of the row pass for rows of L points (gen_split), n_v components
+// and the given number of rows over all loads
+int gen_rows_per_block(double, int nv, int L, long long rows);
+int gen_rows_per_block(float, int nv, int L, long long rows);
 
 // pass along an axis of N points with element stride `stride` (modes as line_pass)
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const double2* tw, double2* S, const double* G,
@@ -20,13 +21,14 @@ cudaError_t gen_col(int mode, const GridInfo& g, int N, const double2* tw, doubl
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const float2* tw, float2* S, const float* G,
                     const LoadState* st, long long stride, int nload, cudaStream_t stream);
 
-// row pass (first: no inverse; kinv: the Krylov operator's inverse half)
+// row pass with rb rows per block (first: no inverse; kinv: the Krylov operator's
+// inverse half; Cfld: point-by-point stiffness or null)
 cudaError_t gen_row(bool first, bool kinv, const GridInfo& g, const double2* tw, double* E, double2* S,
                     const uint8_t* phase, const double* dC, Control* ctl, LoadState* st, double* partials, double* hist,
-                    int nload, double* Wout, const double* Yaux, cudaStream_t stream);
+                    int nload, int rb, double* Wout, const double* Yaux, const double* Cfld, cudaStream_t stream);
 cudaError_t gen_row(bool first, bool kinv, const GridInfo& g, const float2* tw, float* E, float2* S,
                     const uint8_t* phase, const float* dC, Control* ctl, LoadState* st, double* partials, double* hist,
-                    int nload, float* Wout, const float* Yaux, cudaStream_t stream);
+                    int nload, int rb, float* Wout, const float* Yaux, const float* Cfld, cudaStream_t stream);
 
 // checked build: the units' violation records (cleared when taken)
 cudaError_t gen_take_check64(CheckRecord* rec);

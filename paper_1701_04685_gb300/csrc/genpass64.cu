@@ -5,17 +5,23 @@
 
 namespace fh {
 
-int gen_rows_per_block(double, int L) { return gen_rb<double>(L); }
+int gen_rows_per_block(double, int nv, int L, long long rows) {
+  return nv == 3 ? gen_rb<double, 3>(L, rows) : gen_rb<double, 6>(L, rows);
+}
 
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const double2* tw, double2* S, const double* G, const LoadState* st,
                     long long stride, int nload, cudaStream_t stream) {
-  return gen_col_t<double>(mode, g, N, tw, S, G, st, stride, nload, stream);
+  return g.nv == 3 ? gen_col_t<double, 3>(mode, g, N, tw, S, G, st, stride, nload, stream)
+                   : gen_col_t<double, 6>(mode, g, N, tw, S, G, st, stride, nload, stream);
 }
 
 cudaError_t gen_row(bool first, bool kinv, const GridInfo& g, const double2* tw, double* E, double2* S, const uint8_t* phase,
-                    const double* dC, Control* ctl, LoadState* st, double* partials, double* hist, int nload, double* Wout,
-                    const double* Yaux, cudaStream_t stream) {
-  return gen_row_t<double>(first, kinv, g, tw, E, S, phase, dC, ctl, st, partials, hist, nload, Wout, Yaux, stream);
+                    const double* dC, Control* ctl, LoadState* st, double* partials, double* hist, int nload, int rb, double* Wout,
+                    const double* Yaux, const double* Cfld, cudaStream_t stream) {
+  return g.nv == 3 ? gen_row_t<double, 3>(first, kinv, g, tw, E, S, phase, dC, ctl, st, partials, hist, nload, rb, Wout, Yaux,
+                                       Cfld, stream)
+                   : gen_row_t<double, 6>(first, kinv, g, tw, E, S, phase, dC, ctl, st, partials, hist, nload, rb, Wout, Yaux,
+                                       Cfld, stream);
 }
 
 cudaError_t gen_take_check64(CheckRecord* rec) {

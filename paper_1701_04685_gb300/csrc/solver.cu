@@ -139,7 +139,9 @@ struct fh_solver {
   bool col2s = true;         // rows and columns of 32, 64 or 128 points: the two-step passes (else the earlier forms)
   int row2[2] = {0, 0};      // 3-D fields with rows of 32, 64 or 128 points: the two-step row pass applies (L), else 0
   int row2_bpl[2] = {1, 1};  // its blocks per load
-  int rowg_bpl[2] = {0, 0};  // > 0: blocks per load of the two-step row pass of general lengths (genpass.cuh)
+  int rowg_rb[2] = {0, 0};   // > 0: rows per block of the two-step row pass of general lengths (genpass.cuh)
+  int rowg_bpl[2] = {0, 0};  // its blocks per load
+  bool rowg_on[2] = {true, true};  // off for the autotuner's candidate 4 (block row pass with other shapes)
   bool skip_mean = false;   // the phase in progress is followed by another (mixed mode): its mean stress is not used
   int warp_res[2] = {0, 0};  // resident blocks per SM of that pass
   int sms = 0;               // multiprocessors of the device
@@ -236,12 +238,14 @@ void choose_shapes(fh_solver* s, int prec) {
     s->row2[prec] = g.L;
     s->row2_bpl[prec] = (int)((g.nrows + rb - 1) / rb);
   }
-  // other 3-D rows of L = R1 R2 points (16 .. 256): the two-step row pass of
-  // general lengths, where neither of the passes above applies
-  s->rowg_bpl[prec] = 0;
+  // rows of L = R1 R2 points: the two-step row pass of general lengths, where
+  // neither of the passes above applies or the stiffness is given point by point
+  s->rowg_rb[prec] = s->rowg_bpl[prec] = 0;
   int r1, r2;
-  if (g.nv == 6 && s->row_warp[prec] == 0 && s->row2[prec] == 0 && fh::gen_split(g.L, &r1, &r2)) {
-    const int rb = prec == FH_PREC_FP64 ? fh::gen_rows_per_block(0.0, g.L) : fh::gen_rows_per_block(0.f, g.L);
+  if (fh::gen_split(g.L, prec == FH_PREC_FP32, &r1, &r2)) {
+    const long long rows = g.nrows * nl;
+    const int rb = prec == FH_PREC_FP64 ? fh::gen_rows_per_block(0.0, g.nv, g.L, rows) : fh::gen_rows_per_block(0.f, g.nv, g.L, rows);
+    s->rowg_rb[prec] = rb;
     s->rowg_bpl[prec] = (int)((g.nrows + rb - 1) / rb);
   }
   // FP32 3-D grids whose axis-1 and axis-2 lengths are 32, 64 or 128 points
@@ -378,13 +382,13 @@ int col2_len(const fh_solver* s, int prec, int a) {
   return (N == 32 || N == 64 || N == 128) ? N : 0;
 }
 
-// The two-step column pass of general lengths (genpass.cuh) applies to the
-// other axes of R1 R2 points, 16 .. 256, of 3-D fields that neither the
-// compile-time lengths above nor the warp column pass take.
+// The two-step column pass of general lengths (genpass.cuh) applies to the other
+// axes of R1 R2 points that neither the compile-time lengths above nor the warp
+// column pass take.
 bool col_gen(const fh_solver* s, int prec, int a) {
   int r1, r2;
-  return s->col2s && s->g.nv == 6 && col2_len(s, prec, a) == 0 && col_warp_p(s, prec, a) == 0 &&
-         fh::gen_split(s->g.dims[a], &r1, &r2);
+  return s->col2s && col2_len(s, prec, a) == 0 && col_warp_p(s, prec, a) == 0 &&
+         fh::gen_split(s->g.dims[a], prec == FH_PREC_FP32, &r1, &r2);
 }
 
 // columns per block and resident blocks per SM of the two-step column pass:
@@ -559,14 +563,16 @@ void launch_row2(fh_solver* s, int prec, int nload, T* X, const T* dC, Control* 
       Wout, Yaux);
 }
 
-// the two-step row pass of general lengths applies (phase-wise stiffness, not
-// switched off by the autotuner's candidate 5)
-bool use_rowg(const fh_solver* s, int prec) { return s->col2s && s->rowg_bpl[prec] > 0 && !s->field; }
+// the two-step row pass of general lengths applies (not switched off by the
+// autotuner's candidates 4 and 5)
+bool use_rowg(const fh_solver* s, int prec) {
+  return s->col2s && s->rowg_on[prec] && s->rowg_rb[prec] > 0 && (s->field || (s->row_warp[prec] == 0 && s->row2[prec] == 0));
+}
 
 template <typename T, bool FIRST, bool KINV>
-int enqueue_rowg(fh_solver* s, int prec, int nload, T* X, const T* dC, Control* ctl, T* Wout, const T* Yaux) {
+int enqueue_rowg(fh_solver* s, int prec, int nload, T* X, const T* dC, Control* ctl, T* Wout, const T* Yaux, int form) {
   fh::gen_row(FIRST, KINV, s->g, twp<T>(s->ax[s->g.nd - 1]), X, reinterpret_cast<typename fh::cplx_t<T>::type*>(s->S), s->phase,
-              dC, ctl, s->st, s->partials, s->hist, nload, Wout, Yaux, s->work);
+              dC, ctl, s->st, s->partials, s->hist, nload, s->rowg_rb[prec], Wout, Yaux, field_ptr<T>(s, form), s->work);
   return s->rowg_bpl[prec];
 }
 
@@ -588,7 +594,7 @@ void enqueue_row_pass(fh_solver* s, int prec, int nload) {
     return;
   }
   if (use_rowg(s, prec)) {
-    enqueue_rowg<T, FIRST, false>(s, prec, nload, Eptr<T>(s), dCptr<T>(s), s->ctl, nullptr, nullptr);
+    enqueue_rowg<T, FIRST, false>(s, prec, nload, Eptr<T>(s), dCptr<T>(s), s->ctl, nullptr, nullptr, s->form);
     return;
   }
   if constexpr (sizeof(T) == 4) {
@@ -928,7 +934,7 @@ int enqueue_row_x(fh_solver* s, int prec, int nload, T* X, Control* ctl, T* Wout
   C* S = reinterpret_cast<C*>(s->S);
   const int last = g.nd - 1;
   if (use_row2(s, prec)) return enqueue_row2<T, FIRST, KINV>(s, prec, nload, X, dC_form0<T>(s), ctl, Wout, Yaux);
-  if (use_rowg(s, prec)) return enqueue_rowg<T, FIRST, KINV>(s, prec, nload, X, dC_form0<T>(s), ctl, Wout, Yaux);
+  if (use_rowg(s, prec)) return enqueue_rowg<T, FIRST, KINV>(s, prec, nload, X, dC_form0<T>(s), ctl, Wout, Yaux, 0);
   if constexpr (sizeof(T) == 4) {
     const int P = s->field ? 0 : s->row_warp[prec];
     if (P > 0) {
@@ -2195,10 +2201,11 @@ bool apply_variant(fh_solver* s, int prec, int var) {
     s->ax[a].planp[prec] = d.plans[a];
   }
   s->col2s = true;
+  s->rowg_on[prec] = true;
   if (var == 0) return true;
   if (var == 4) {
     if (s->row_warp[prec] > 0 && !s->field) return false;   // the warp row pass runs instead
-    if ((s->row2[prec] > 0 || s->rowg_bpl[prec] > 0) && !s->field) return false;   // a two-step row pass runs instead
+    if (s->row2[prec] > 0 && !s->field) return false;       // the two-step row pass runs instead
     const int rpb = 2 * d.rpb_gen;
     if (rpb > g.nrows) return false;
     const int Lp = prec == FH_PREC_FP64 ? fh::padded_len<3>(g.L) : fh::padded_len<4>(g.L);
@@ -2207,11 +2214,12 @@ bool apply_variant(fh_solver* s, int prec, int var) {
     s->rpb_gen[prec] = rpb;
     s->row_bpl_gen[prec] = (int)((g.nrows + rpb - 1) / rpb);
     s->row_smem_gen[prec] = sm;
+    s->rowg_on[prec] = false;   // the block row pass
     return true;
   }
   if (var == 5) {
     bool any = false;
-    if ((s->row2[prec] > 0 || s->rowg_bpl[prec] > 0) && !s->field) {
+    if ((s->row2[prec] > 0 && !s->field) || use_rowg(s, prec)) {
       s->col2s = false;
       any = true;
     }
