@@ -61,13 +61,20 @@ __host__ inline size_t col2_smem() {
 template <int R2>
 __device__ __forceinline__ int c2off(int k1, int j2) { return j2 + (R2 + 1) * k1; }
 
-// w[t] = w_N^{DIR base t} for t < R (R = 4, 8 or 16): the powers t = 1, 2, 4, 8
-// come from the table tw[t] = exp(-2 pi i t / N), every other one is the
-// product of two earlier ones (at most three roundings deep)
+// w[t] = w_N^{DIR base t} for t < R (R = 4, 8 or 16).  FP32: the powers t = 1, 2,
+// 4, 8 come from the table tw[t] = exp(-2 pi i t / N), every other one is the
+// product of two earlier ones (at most three roundings deep).  FP64: all come from
+// the table, since the products would be a tenth of a pass's FP64 instructions
+// (4 or 11 complex products per 8 or 16 points), which bound it
 template <int R, int DIR, typename T = float>
 __device__ __forceinline__ void twiddle_powers(const cplx<T>* tw, int base, cplx<T>* w) {
   w[0].x = T(1);
   w[0].y = T(0);
+  if constexpr (sizeof(T) == 8) {
+#pragma unroll
+    for (int t = 1; t < R; ++t) w[t] = twl<DIR, T>(tw, base * t);
+    return;
+  }
 #pragma unroll
   for (int p = 1; p < R; p <<= 1) w[p] = twl<DIR, T>(tw, base * p);
 #pragma unroll

@@ -235,11 +235,11 @@ __global__ void __launch_bounds__(gen_threads<T, NV>(), 2)
   (void)nS; (void)nE; (void)nB;
   if (!skip) {
     for (int i = tid; i < L; i += NT) tw[i] = twg[i];
-    if (!KINV && !Cfld) {
+    if (!KINV && !Cfld) {   // tau / 2, as in row_pass_2s
       if (decoupled) {
-        for (int i = tid; i < 16 * 12; i += NT) dcp[i % (NV == 6 ? 192 : 1)] = decoupled_entry(dC + (i / 12) * NV * NV, i % 12);
+        for (int i = tid; i < 16 * 12; i += NT) dcp[i % (NV == 6 ? 192 : 1)] = T(0.5) * decoupled_entry(dC + (i / 12) * NV * NV, i % 12);
       } else {
-        for (int i = tid; i < 16 * NV * NV; i += NT) dcs[i] = dC[i];
+        for (int i = tid; i < 16 * NV * NV; i += NT) dcs[i] = T(0.5) * dC[i];
       }
     }
     __syncthreads();
@@ -373,6 +373,8 @@ __global__ void __launch_bounds__(gen_threads<T, NV>(), 2)
             tau[a] = fma(cab, xv[b], tau[a]);
             if (b != a) tau[b] = fma(cab, xv[a], tau[b]);
           }
+#pragma unroll
+        for (int a = 0; a < NV; ++a) tau[a] *= T(0.5);
       } else {
         int ph = phase[pt];
         if (!FH_IN(CK_ROW_PHASE, ph, 16)) ph = 0;
@@ -424,10 +426,10 @@ __global__ void __launch_bounds__(gen_threads<T, NV>(), 2)
         const C zk = ln[k];
         const C zm = ln[k == 0 ? 0 : L - k];
         C A, B;
-        A.x = T(0.5) * (zk.x + zm.x);
-        A.y = T(0.5) * (zk.y - zm.y);
-        B.x = T(0.5) * (zk.y + zm.y);
-        B.y = T(-0.5) * (zk.x - zm.x);
+        A.x = zk.x + zm.x;
+        A.y = zk.y - zm.y;
+        B.x = zk.y + zm.y;
+        B.y = zm.x - zk.x;
         Sl[spec(2 * line) + k] = A;
         if (NV == 6 || 2 * line + 1 < nreal) Sl[spec(2 * line + 1) + k] = B;
       }

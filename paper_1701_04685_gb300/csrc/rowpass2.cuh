@@ -80,9 +80,11 @@ __global__ void __launch_bounds__(Row2<R1, R2>::THREADS, sizeof(T) == 4 ? 3 : 1)
   if ((FIRST || KINV) && st[load].done) return;
   for (int i = threadIdx.x; i < L; i += NT) tw[i] = twg[i];
   if (!KINV) {
-    for (int i = threadIdx.x; i < 16 * NV * NV; i += NT) dcs[i] = dC[i];
+    // tau / 2: the split of a line's spectrum into its two components then needs
+    // additions only (a power of two: the same bits)
+    for (int i = threadIdx.x; i < 16 * NV * NV; i += NT) dcs[i] = T(0.5) * dC[i];
     if (decoupled)
-      for (int i = threadIdx.x; i < 16 * 12; i += NT) dcp[i] = decoupled_entry(dC + (i / 12) * NV * NV, i % 12);
+      for (int i = threadIdx.x; i < 16 * 12; i += NT) dcp[i] = T(0.5) * decoupled_entry(dC + (i / 12) * NV * NV, i % 12);
   }
   if (threadIdx.x == 0) s_skip = st[load].done;
   __syncthreads();
@@ -310,10 +312,10 @@ __global__ void __launch_bounds__(Row2<R1, R2>::THREADS, sizeof(T) == 4 ? 3 : 1)
         const C zk = ln[k];
         const C zm = ln[k == 0 ? 0 : L - k];
         C A, B;
-        A.x = T(0.5) * (zk.x + zm.x);
-        A.y = T(0.5) * (zk.y - zm.y);
-        B.x = T(0.5) * (zk.y + zm.y);
-        B.y = T(-0.5) * (zk.x - zm.x);
+        A.x = zk.x + zm.x;
+        A.y = zk.y - zm.y;
+        B.x = zk.y + zm.y;
+        B.y = zm.x - zk.x;
         Sw[(size_t)(2 * p) * cstrS + row * H + k] = A;
         Sw[(size_t)(2 * p + 1) * cstrS + row * H + k] = B;
       }

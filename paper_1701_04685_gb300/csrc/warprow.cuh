@@ -45,13 +45,12 @@ __device__ __forceinline__ void dft16(cplx<T>* v) {
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) y[n2][k1] = a[k1];
   }
-  auto tw16 = [&](int m) {   // exp(DIR 2 pi i m / 16) for m in {1, 2, 3, 4, 6, 9}
+  auto tw16 = [&](int m) {   // exp(DIR 2 pi i m / 16) for m in {1, 2, 3, 6, 9}
     cplx<T> w;
     switch (m) {
       case 1: w.x = c1; w.y = s1; break;
       case 2: w.x = h; w.y = h; break;
       case 3: w.x = s1; w.y = c1; break;
-      case 4: w.x = T(0); w.y = T(1); break;
       case 6: w.x = -h; w.y = h; break;
       default: w.x = -c1; w.y = -s1; break;
     }
@@ -61,7 +60,8 @@ __device__ __forceinline__ void dft16(cplx<T>* v) {
 #pragma unroll
   for (int n2 = 1; n2 < 4; ++n2)
 #pragma unroll
-    for (int k1 = 1; k1 < 4; ++k1) y[n2][k1] = cmul(y[n2][k1], tw16(n2 * k1));
+    for (int k1 = 1; k1 < 4; ++k1)   // w^4 = DIR i costs nothing
+      y[n2][k1] = n2 * k1 == 4 ? mul_i<DIR>(y[n2][k1]) : cmul(y[n2][k1], tw16(n2 * k1));
 #pragma unroll
   for (int k1 = 0; k1 < 4; ++k1) {
     cplx<T> a[4] = {y[0][k1], y[1][k1], y[2][k1], y[3][k1]};
