@@ -26,6 +26,7 @@
 
 #include <cooperative_groups.h>
 
+#include "bigfft.cuh"
 #include "kernels.cuh"
 #include "warprow.cuh"
 
@@ -80,10 +81,9 @@ __host__ __device__ inline ClusterLayout cluster_layout(int N0, int L, int nv, i
   return c;
 }
 
-// threads per CTA: 8 warps for general radix plans (with the 11- and
-// 13-point stages compiled in, 16 warps would cap registers at 128 and
-// spill) and in FP64; 16 warps for FP32 plans of radices 2, 4, 8 only
-template <typename T, bool POW2> struct ClusterThreads { static constexpr int value = (POW2 && sizeof(T) == 4) ? 512 : 256; };
+// threads per CTA: 16 warps in FP32, 8 in FP64 (whose pipe they fill, and whose
+// larger line transforms need the registers)
+template <typename T> struct ClusterThreads { static constexpr int value = sizeof(T) == 4 ? 512 : 256; };
 
 // The whole solve of load `load` by the cluster this CTA belongs to.  Ends
 // with a cluster barrier, after which the cluster may start another solve.
@@ -163,6 +163,22 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
   const T scale = (T)g.inv_m;
   __syncthreads();
 
+  // line transform of buf (ping-pong with tmp): plans of radices 2, 4, 8 inline, any
+  // other through fft_lines_big
+  auto lines = [&](auto dir, auto pad, cplx<T>* buf, cplx<T>* tmp, int n, int ls, const DevPlan& plan, const cplx<T>* tw,
+                   int t, int nthr) -> cplx<T>* {
+    constexpr int DIR = decltype(dir)::value, PADSH = decltype(pad)::value;
+    if constexpr (POW2) {
+      return fft_lines_pp<DIR, T, PADSH, true>(buf, tmp, n, ls, plan, tw, t, nthr);
+    } else {
+      const unsigned char* base = sm;
+      const unsigned o = fft_lines_big<DIR, T, PADSH>((unsigned)(reinterpret_cast<unsigned char*>(buf) - base),
+                                                      (unsigned)(reinterpret_cast<unsigned char*>(tmp) - base), n, ls, &plan,
+                                                      (unsigned)(reinterpret_cast<const unsigned char*>(tw) - base), t, nthr);
+      return reinterpret_cast<cplx<T>*>(sm + o);
+    }
+  };
+
   // ---- row phase: (optional inverse FFT + E update + residual) + stress + forward FFT
   auto row_phase = [&](bool with_inverse, ResAcc<T>& acc_d, ResAcc<T>& acc_n) {
     const int nreal = nrow * NV;
@@ -190,7 +206,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
       __syncthreads();
       bool warp_done = false;   // FP32, power-of-two rows of 32..512 points: one warp per line, in place
       if constexpr (POW2 && sizeof(T) == 4) warp_done = warp_lines_any<+1, PS, T>(W0, npair, Lp, L, tw1, threadIdx.x, blockDim.x);
-      Z = warp_done ? W0 : fft_lines_pp<+1, T, PS, POW2>(W0, W1, npair, Lp, plan1, tw1);
+      Z = warp_done ? W0 : lines(RadixC<+1>{}, RadixC<PS>{}, W0, W1, npair, Lp, plan1, tw1, threadIdx.x, blockDim.x);
       Zo = (Z == W0) ? W1 : W0;
     }
     // E update, residual sums and stress, two points per thread at a time
@@ -252,7 +268,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
     if constexpr (POW2 && sizeof(T) == 4)
       fused = warp_rows_fwd_split_any<PS, T>(Z, npair, Lp, L, Sl, H, nreal, tw1, threadIdx.x, blockDim.x);
     if (!fused) {
-      cplx<T>* Zf = fft_lines_pp<-1, T, PS, POW2>(Z, Zo, npair, Lp, plan1, tw1);
+      cplx<T>* Zf = lines(RadixC<-1>{}, RadixC<PS>{}, Z, Zo, npair, Lp, plan1, tw1, threadIdx.x, blockDim.x);
       for (int idx = threadIdx.x; idx < npair * H; idx += blockDim.x) {
         const int p = fdiv(idx, fH), k = idx - p * H;
         const cplx<T> zk = Zf[p * Lp + padi<PS>(k)];
@@ -286,7 +302,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
     team_sync(nwork);
     bool warp_done = false;   // FP32, power-of-two columns of 32..512 points: one warp per line, in place
     if constexpr (POW2 && sizeof(T) == 4) warp_done = warp_lines_any<-1, 0, T>(X0, nl, N0p, N0, tw0, tid, nwork);
-    cplx<T>* Xf = warp_done ? X0 : fft_lines_pp<-1, T, 0, POW2>(X0, X1, nl, N0p, plan0, tw0, tid, nwork);
+    cplx<T>* Xf = warp_done ? X0 : lines(RadixC<-1>{}, RadixC<0>{}, X0, X1, nl, N0p, plan0, tw0, tid, nwork);
     for (int idx = tid; idx < N0 * ncol; idx += nwork) {
       const int n = fdiv(idx, fnc);
       const int j = idx - n * ncol;
@@ -316,7 +332,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
     }
     team_sync(nwork);
     if constexpr (POW2 && sizeof(T) == 4) warp_done = warp_lines_any<+1, 0, T>(Xf, nl, N0p, N0, tw0, tid, nwork);
-    cplx<T>* Xi = warp_done ? Xf : fft_lines_pp<+1, T, 0, POW2>(Xf, Xf == X0 ? X1 : X0, nl, N0p, plan0, tw0, tid, nwork);
+    cplx<T>* Xi = warp_done ? Xf : lines(RadixC<+1>{}, RadixC<0>{}, Xf, Xf == X0 ? X1 : X0, nl, N0p, plan0, tw0, tid, nwork);
     for (int idx = tid; idx < NV * N0 * ncol; idx += nwork) {
       const int t = fdiv(idx, fnc);
       const int j = idx - t * ncol;
@@ -415,7 +431,7 @@ struct ClusterTask {
 // one atomic and the other CTAs read it from rank 0's shared memory; clusters
 // never wait on one another.  The task is staged in shared memory.
 template <typename T, int NV, int CS, bool POW2>
-__global__ void __launch_bounds__(ClusterThreads<T, POW2>::value, 1)
+__global__ void __launch_bounds__(ClusterThreads<T>::value, 1)
 cluster_solve_2d(const ClusterTask* __restrict__ tasks, int ntasks, unsigned int* next) {
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ int s_task;

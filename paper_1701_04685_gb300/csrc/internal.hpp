@@ -49,6 +49,8 @@ struct FftPlan {
   int r[24] = {};
 };
 bool make_plan(int L, FftPlan* plan);
+// the same with every radix from 2 to 16: the fewest stages, then the smallest radices
+bool make_big_plan(int L, FftPlan* plan);
 
 }  // namespace fh
 

@@ -311,4 +311,40 @@ bool make_plan(int L, FftPlan* plan) {
   return true;
 }
 
+// fewest factors of n (no prime above 13) among 2 .. 16, then the smallest sum
+static bool big_factors(int n, int most, int* r, int* np, int* sum) {
+  if (n == 1) { *np = 0; *sum = 0; return true; }
+  bool found = false;
+  for (int f = std::min(most, n); f >= 2; --f) {   // factors in falling order
+    if (n % f != 0) continue;
+    int sub[24], k = 0, sm = 0;
+    if (!big_factors(n / f, f, sub, &k, &sm) || k + 1 > 24) continue;
+    if (!found || k + 1 < *np || (k + 1 == *np && sm + f < *sum)) {
+      found = true;
+      *np = k + 1;
+      *sum = sm + f;
+      r[0] = f;
+      std::copy(sub, sub + k, r + 1);
+    }
+  }
+  return found;
+}
+
+bool make_big_plan(int L, FftPlan* plan) {
+  FftPlan p, rest;
+  if (!make_plan(L, &rest)) return false;
+  p.L = L;
+  int n = L;
+  for (int q = 0; q < rest.np; ++q)   // larger primes: their direct stages
+    if (rest.r[q] > 13) {
+      p.r[p.np++] = rest.r[q];
+      n /= rest.r[q];
+    }
+  int r[24], np = 0, sum = 0;
+  if (!big_factors(n, 16, r, &np, &sum) || p.np + np > 24) return false;
+  for (int q = 0; q < np; ++q) p.r[p.np++] = r[q];
+  *plan = p;
+  return true;
+}
+
 }  // namespace fh

@@ -71,7 +71,8 @@ int mandel_nv(int d) { return d == 2 ? 3 : 6; }
 
 struct Axis {
   int L = 1;
-  DevPlan plan{};        // radix schedule of the cluster kernel (and the default)
+  DevPlan plan{};        // radix schedule of the cluster kernel for powers of two (and the default)
+  DevPlan big{};         // its schedule for other grids (radices up to 16)
   DevPlan planp[2]{};    // radix schedule of the passes per bulk precision (autotuned)
   double2* tw64 = nullptr;
   float2* tw32 = nullptr;
@@ -1060,6 +1061,10 @@ bool pow2_plans(const fh_solver* s) {
   return true;
 }
 
+// threads per CTA of the cluster kernel
+template <typename T>
+constexpr int cluster_threads() { return fh::ClusterThreads<T>::value; }
+
 // Cluster-resident path (2-axis grids): one cluster of CS CTAs per load case.
 template <typename T, int NV, int CS, bool POW2>
 fh_status cluster_fits_nv(fh_solver* s, bool* ok) {
@@ -1079,7 +1084,7 @@ fh_status cluster_fits_nv(fh_solver* s, bool* ok) {
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(CS);
-  cfg.blockDim = dim3(fh::ClusterThreads<T, POW2>::value);
+  cfg.blockDim = dim3(cluster_threads<T>());
   cfg.dynamicSmemBytes = lay.total;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1110,8 +1115,9 @@ fh::ClusterTask cluster_task(const fh_solver* s, int l) {
   const bool gs = s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0];
   fh::ClusterTask t{};
   t.g = s->g;
-  t.plan0 = s->ax[0].plan;
-  t.plan1 = s->ax[1].plan;
+  const bool pow2 = pow2_plans(s);
+  t.plan0 = pow2 ? s->ax[0].plan : s->ax[0].big;
+  t.plan1 = pow2 ? s->ax[1].plan : s->ax[1].big;
   t.tw0 = twp<T>(s->ax[0]);
   t.tw1 = twp<T>(s->ax[1]);
   t.E = Eptr<T>(const_cast<fh_solver*>(s));
@@ -1132,7 +1138,7 @@ template <typename T, int NV, int CS, bool POW2>
 cudaLaunchConfig_t cluster_config(size_t smem, int nclusters, cudaStream_t stream, cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nclusters * CS);
-  cfg.blockDim = dim3(fh::ClusterThreads<T, POW2>::value);
+  cfg.blockDim = dim3(cluster_threads<T>());
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1645,6 +1651,10 @@ fh_status fh_solver_create(const fh_pattern* p, const fh_generator* gen, int nlo
     s->ax[k].plan.np = fp.np;
     for (int q = 0; q < 24; ++q) s->ax[k].plan.r[q] = fp.r[q];
     s->ax[k].planp[0] = s->ax[k].planp[1] = s->ax[k].plan;
+    if (!fh::make_big_plan(g.dims[k], &fp)) { delete s; fh::set_error("SNF axis length needs more than 24 radix stages"); return FH_ERR_UNSUPPORTED; }
+    s->ax[k].big.L = fp.L;
+    s->ax[k].big.np = fp.np;
+    for (int q = 0; q < 24; ++q) s->ax[k].big.r[q] = fp.r[q];
   }
   choose_shapes(s, FH_PREC_FP64);
   choose_shapes(s, FH_PREC_FP32);
