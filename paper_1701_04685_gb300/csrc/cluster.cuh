@@ -89,6 +89,7 @@ template <typename T> struct ClusterThreads { static constexpr int value = sizeo
 // with a cluster barrier, after which the cluster may start another solve.
 template <typename T, int NV, int CS, bool POW2>
 __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevPlan& plan0, const DevPlan& plan1,
+                                                   const LineSplit& split0, const LineSplit& split1,
                                                    const cplx<T>* __restrict__ tw0g, const cplx<T>* __restrict__ tw1g,
                                                    T* __restrict__ Eg, const uint8_t* __restrict__ phase,
                                                    const T* __restrict__ dC, int nphase, const T* __restrict__ Gt,
@@ -163,11 +164,19 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
   const T scale = (T)g.inv_m;
   __syncthreads();
 
-  // line transform of buf (ping-pong with tmp): plans of radices 2, 4, 8 inline, any
-  // other through fft_lines_big
-  auto lines = [&](auto dir, auto pad, cplx<T>* buf, cplx<T>* tmp, int n, int ls, const DevPlan& plan, const cplx<T>* tw,
-                   int t, int nthr) -> cplx<T>* {
+  // line transform of buf (ping-pong with tmp): plans of radices 2, 4, 8 inline; other
+  // grids by single warps (FP32, where the length splits) or through fft_lines_big
+  auto lines = [&](auto dir, auto pad, cplx<T>* buf, cplx<T>* tmp, int n, int ls, const DevPlan& plan, const LineSplit& split,
+                   const cplx<T>* tw, int t, int nthr) -> cplx<T>* {
     constexpr int DIR = decltype(dir)::value, PADSH = decltype(pad)::value;
+    if constexpr (!POW2 && sizeof(T) == 4) {
+      if (split.R1 > 0) {
+        const unsigned char* base = sm;
+        warp_two_step<T>((unsigned)(reinterpret_cast<unsigned char*>(buf) - base), n, ls, PADSH ? PADSH : 31, DIR > 0, split,
+                         (unsigned)(reinterpret_cast<const unsigned char*>(tw) - base), t, nthr);
+        return buf;
+      }
+    }
     if constexpr (POW2) {
       return fft_lines_pp<DIR, T, PADSH, true>(buf, tmp, n, ls, plan, tw, t, nthr);
     } else {
@@ -206,7 +215,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
       __syncthreads();
       bool warp_done = false;   // FP32, power-of-two rows of 32..512 points: one warp per line, in place
       if constexpr (POW2 && sizeof(T) == 4) warp_done = warp_lines_any<+1, PS, T>(W0, npair, Lp, L, tw1, threadIdx.x, blockDim.x);
-      Z = warp_done ? W0 : lines(RadixC<+1>{}, RadixC<PS>{}, W0, W1, npair, Lp, plan1, tw1, threadIdx.x, blockDim.x);
+      Z = warp_done ? W0 : lines(RadixC<+1>{}, RadixC<PS>{}, W0, W1, npair, Lp, plan1, split1, tw1, threadIdx.x, blockDim.x);
       Zo = (Z == W0) ? W1 : W0;
     }
     // E update, residual sums and stress, two points per thread at a time
@@ -268,7 +277,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
     if constexpr (POW2 && sizeof(T) == 4)
       fused = warp_rows_fwd_split_any<PS, T>(Z, npair, Lp, L, Sl, H, nreal, tw1, threadIdx.x, blockDim.x);
     if (!fused) {
-      cplx<T>* Zf = lines(RadixC<-1>{}, RadixC<PS>{}, Z, Zo, npair, Lp, plan1, tw1, threadIdx.x, blockDim.x);
+      cplx<T>* Zf = lines(RadixC<-1>{}, RadixC<PS>{}, Z, Zo, npair, Lp, plan1, split1, tw1, threadIdx.x, blockDim.x);
       for (int idx = threadIdx.x; idx < npair * H; idx += blockDim.x) {
         const int p = fdiv(idx, fH), k = idx - p * H;
         const cplx<T> zk = Zf[p * Lp + padi<PS>(k)];
@@ -302,7 +311,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
     team_sync(nwork);
     bool warp_done = false;   // FP32, power-of-two columns of 32..512 points: one warp per line, in place
     if constexpr (POW2 && sizeof(T) == 4) warp_done = warp_lines_any<-1, 0, T>(X0, nl, N0p, N0, tw0, tid, nwork);
-    cplx<T>* Xf = warp_done ? X0 : lines(RadixC<-1>{}, RadixC<0>{}, X0, X1, nl, N0p, plan0, tw0, tid, nwork);
+    cplx<T>* Xf = warp_done ? X0 : lines(RadixC<-1>{}, RadixC<0>{}, X0, X1, nl, N0p, plan0, split0, tw0, tid, nwork);
     for (int idx = tid; idx < N0 * ncol; idx += nwork) {
       const int n = fdiv(idx, fnc);
       const int j = idx - n * ncol;
@@ -332,7 +341,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
     }
     team_sync(nwork);
     if constexpr (POW2 && sizeof(T) == 4) warp_done = warp_lines_any<+1, 0, T>(Xf, nl, N0p, N0, tw0, tid, nwork);
-    cplx<T>* Xi = warp_done ? Xf : lines(RadixC<+1>{}, RadixC<0>{}, Xf, Xf == X0 ? X1 : X0, nl, N0p, plan0, tw0, tid, nwork);
+    cplx<T>* Xi = warp_done ? Xf : lines(RadixC<+1>{}, RadixC<0>{}, Xf, Xf == X0 ? X1 : X0, nl, N0p, plan0, split0, tw0, tid, nwork);
     for (int idx = tid; idx < NV * N0 * ncol; idx += nwork) {
       const int t = fdiv(idx, fnc);
       const int j = idx - t * ncol;
@@ -409,6 +418,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
 struct ClusterTask {
   GridInfo g;
   DevPlan plan0, plan1;
+  LineSplit split0, split1;
   const void* tw0;
   const void* tw1;
   void* E;
@@ -447,7 +457,7 @@ cluster_solve_2d(const ClusterTask* __restrict__ tasks, int ntasks, unsigned int
     }
     cluster.sync();   // every CTA holds the index (and the task) before rank 0 draws the next one
     if (task >= ntasks) return;
-    cluster_solve_body<T, NV, CS, POW2>(t.g, t.plan0, t.plan1, static_cast<const cplx<T>*>(t.tw0),
+    cluster_solve_body<T, NV, CS, POW2>(t.g, t.plan0, t.plan1, t.split0, t.split1, static_cast<const cplx<T>*>(t.tw0),
                                         static_cast<const cplx<T>*>(t.tw1), static_cast<T*>(t.E), t.phase,
                                         static_cast<const T*>(t.dC), t.nphase, static_cast<const T*>(t.Gt), t.ctl,
                                         t.st, t.hist, t.g_smem, t.load);

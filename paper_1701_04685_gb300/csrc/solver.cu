@@ -1118,6 +1118,8 @@ fh::ClusterTask cluster_task(const fh_solver* s, int l) {
   const bool pow2 = pow2_plans(s);
   t.plan0 = pow2 ? s->ax[0].plan : s->ax[0].big;
   t.plan1 = pow2 ? s->ax[1].plan : s->ax[1].big;
+  t.split0 = fh::line_split(s->g.dims[0]);
+  t.split1 = fh::line_split(s->g.L);
   t.tw0 = twp<T>(s->ax[0]);
   t.tw1 = twp<T>(s->ax[1]);
   t.E = Eptr<T>(const_cast<fh_solver*>(s));
