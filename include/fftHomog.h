@@ -386,11 +386,14 @@ fh_status fh_fno_set_params(fh_fno* f, const float* params);
 fh_status fh_fno_get_params(const fh_fno* f, float* params);
 fh_status fh_fno_get_grads(const fh_fno* f, float* grads);
 fh_status fh_fno_zero_grad(fh_fno* f);
-/* y = network(x) for `batch` samples (x, y device). */
+/* y = network(x) for `batch` samples (x, y device).  FH_ERR_TIMEOUT when a
+ * tensor-core layer's bounded wait for its MMAs gave up (y not valid). */
 fh_status fh_fno_forward(fh_fno* f, int batch, const float* x, float* y);
-/* Selects the arithmetic unit of the hidden 1 x 1 layers W_l v + w_l (default
- * 1).  Both settings give FP32 accuracy (BF16 weights as above, FP32
- * activations and sums); at present both run the SIMT row kernels. */
+/* The hidden layers (1 x 1 layer and z transforms) run on the tensor cores
+ * (tcgen05: BF16 weights as above, FP32 operands split into three BF16 terms, FP32
+ * accumulation in tensor memory) when width is 32 and n a multiple of 16; enable = 0
+ * selects the SIMT form (default 1).  Not in the paper: the network is this
+ * library's own. */
 fh_status fh_fno_set_tensor_cores(fh_fno* f, int enable);
 /* Forward and backward of the mean squared error against `target`
  * (mean over samples, channels and voxels); the loss goes to *loss (host,

@@ -32,6 +32,7 @@
 #include "internal.hpp"
 #include "fno_rows.cuh"
 #include "fno_spec.cuh"
+#include "fno_tc.cuh"
 
 namespace {
 
@@ -115,7 +116,10 @@ struct fh_fno {
   double* part = nullptr;
   int nparts = 0;
   int sms = 1;
+  // hidden layers on the tensor cores (fno_tc.cuh) where they apply; tc_err is set by
+  // a kernel whose bounded wait gave up
   bool tensor_cores = true;
+  int* tc_err = nullptr;
 };
 
 namespace {
@@ -176,6 +180,51 @@ fh_status launch_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
   if (blocks) *blocks = grid;
   fhrow::k_rows<EPI><<<grid, fhrow::kRowThreads, sm, f->stream>>>(a);
   FCK(cudaGetLastError());
+  return FH_OK;
+}
+
+// The tensor-core form takes the hidden layers (BF16 weights, spectral input, no
+// projection) of 32 channels on rows of 16 .. 128 points, a multiple of 16, whose
+// operands fit a CTA's shared memory.
+bool use_tc(const fh_fno* f, const fhrow::RowArgs& a) {
+  const FnoDims& d = f->d;
+  const int Kp = (2 * d.m + 15) & ~15;
+  return f->tensor_cores && d.W == fhtc::kTcW && a.Cin == fhtc::kTcW && a.a_bf16 && a.Iy && !a.Q && d.N % 16 == 0 &&
+         fhtc::tc_layout(d.N, Kp).total + 1024 <= 227 * 1024;
+}
+
+// a hidden layer's rows, on the tensor cores where that applies
+template <int EPI>
+fh_status hidden_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
+  if (!use_tc(f, a)) return launch_rows<EPI>(f, a, blocks);
+  const FnoDims& d = f->d;
+  fhtc::TcArgs t{};
+  t.N = d.N; t.N3 = d.N3; t.N2 = a.N2; t.m2 = 2 * d.m;
+  t.Kp = (t.m2 + 15) & ~15;
+  t.ntiles = a.nrows / fhtc::kTcRows;   // N^2 rows a sample, N a multiple of 16
+  t.ncols = 32;
+  while (t.ncols < d.N + t.Kp) t.ncols *= 2;
+  t.in = a.in; t.W = reinterpret_cast<const __nv_bfloat16*>(a.A); t.trans = a.a_trans; t.bias = a.bias;
+  t.Iy = a.Iy; t.T = a.T; t.u_in = a.u_in; t.u_out = a.u_out; t.out = a.out; t.Yz = a.Yz; t.err = f->tc_err;
+  const size_t sm = fhtc::tc_layout(d.N, t.Kp).total;
+  FCK(cudaFuncSetAttribute(fhtc::k_rows_tc<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  FCK(cudaFuncSetAttribute(fhtc::k_rows_tc<EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+  // two CTAs share an SM where their shared memory allows (tensor memory has 512 columns)
+  const int res = 2 * (sm + 2048) <= 228 * 1024 && 2 * t.ncols <= 512 ? 2 : 1;
+  fhtc::k_rows_tc<EPI><<<std::min(t.ntiles, res * f->sms), fhtc::kTcThreads, sm, f->stream>>>(t);
+  FCK(cudaGetLastError());
+  return FH_OK;
+}
+
+// a tensor-core layer whose bounded wait gave up leaves an error word
+fh_status tc_status(fh_fno* f) {
+  int h = 0;
+  FCK(cudaMemcpy(&h, f->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
+  if (h != 0) {
+    FCK(cudaMemset(f->tc_err, 0, sizeof(int)));
+    fh::set_error("a tensor-core layer's wait for its MMAs gave up");
+    return FH_ERR_TIMEOUT;
+  }
   return FH_OK;
 }
 
@@ -273,7 +322,7 @@ fh_status forward_all(fh_fno* f, int B, const float* x, float* y, const float* t
         a.y = y;
       }
     }
-    rc = launch_rows<1>(f, a, blocks);
+    rc = hidden_rows<1>(f, a, blocks);
   }
   return rc;
 }
@@ -356,6 +405,8 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
   if ((e = cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return fail(e);
   f->nparts = 8 * f->sms;   // at least the resident blocks of a row kernel
   if ((e = cudaMalloc(&f->part, f->nparts * sizeof(double))) != cudaSuccess) return fail(e);
+  if ((e = cudaMalloc(&f->tc_err, sizeof(int))) != cudaSuccess) return fail(e);
+  if ((e = cudaMemset(f->tc_err, 0, sizeof(int))) != cudaSuccess) return fail(e);
   cudaMemset(f->prm, 0, o * 4);
   cudaMemset(f->grd, 0, o * 4);
   cudaMemset(f->m1, 0, o * 4);
@@ -389,7 +440,7 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
 void fh_fno_destroy(fh_fno* f) {
   if (!f) return;
   void* ptrs[] = {f->prm, f->grd, f->m1, f->m2, f->Wbf, f->Rbf, f->tw, f->zt, f->v, f->u, f->vh,
-                  f->Yz, f->Yy, f->y, f->gy, f->ga, f->gb, f->part, f->flat};
+                  f->Yz, f->Yy, f->y, f->gy, f->ga, f->gb, f->part, f->flat, f->tc_err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete f;
@@ -488,7 +539,7 @@ fh_status fh_fno_forward(fh_fno* f, int batch, const float* x, float* y) {
   if (rc != FH_OK) return rc;
   if (!direct) FCK(cudaMemcpyAsync(y, f->y, (size_t)batch * f->d.cout * f->d.N3 * 4, cudaMemcpyDefault, f->stream));
   FCK(cudaStreamSynchronize(f->stream));
-  return FH_OK;
+  return tc_status(f);
 }
 
 fh_status fh_fno_set_tensor_cores(fh_fno* f, int enable) {
@@ -529,9 +580,9 @@ fh_status fh_fno_loss_grad(fh_fno* f, int batch, const float* x, const float* ta
     if (l > 0) {
       a.u_in = f->u + (size_t)(l - 1) * act;
       a.Yz = f->Yz;
-      rc = launch_rows<2>(f, a);
+      rc = hidden_rows<2>(f, a);
     } else {
-      rc = launch_rows<0>(f, a);
+      rc = hidden_rows<0>(f, a);
     }
     std::swap(gu, next);
   }
@@ -547,7 +598,7 @@ fh_status fh_fno_loss_grad(fh_fno* f, int batch, const float* x, const float* ta
     for (double p : parts) s += p;
     *loss = s / (double)ny;
   }
-  return FH_OK;
+  return tc_status(f);
 }
 
 fh_status fh_fno_adam_step(fh_fno* f, float lr, float beta1, float beta2, float eps, int step) {
