@@ -87,11 +87,12 @@ __device__ __forceinline__ void twiddle_powers(const cplx<T>* tw, int base, cplx
 
 // resident blocks per SM the register budget is set for: three for the
 // single transforms, two for MODE 2 (whose Green step wants more registers;
-// measured faster at two)
-template <int MODE>
-constexpr int col2_minb() { return MODE == 2 ? 2 : 3; }
+// measured faster at two for 128 points; at three for up to 64: 64^3 x 6 loads
+// 35.6 -> 32.8 us)
+template <int MODE, int N = 128>
+constexpr int col2_minb() { return MODE == 2 && N > 64 ? 2 : 3; }
 
-template <int R1, int R2, int MODE, int CT = kColTile, int MINB = col2_minb<MODE>(), typename T = float>
+template <int R1, int R2, int MODE, int CT = kColTile, int MINB = col2_minb<MODE, R1 * R2>(), typename T = float>
 __global__ void __launch_bounds__(Col2<R1, R2, CT, T>::THREADS, MINB)
     line_pass_2s(GridInfo g, const cplx<T>* __restrict__ twg, cplx<T>* __restrict__ S, const T* __restrict__ Gt,
                  const LoadState* st, long long stride, long long ncols, int nload) {

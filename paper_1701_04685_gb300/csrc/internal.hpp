@@ -49,8 +49,9 @@ struct FftPlan {
   int r[24] = {};
 };
 bool make_plan(int L, FftPlan* plan);
-// the same with every radix from 2 to 16: the fewest stages, then the smallest radices
-bool make_big_plan(int L, FftPlan* plan);
+// the same with any radix from 2 to `most` (16 at most; primes to 13 always): the
+// fewest stages, then the smallest radices
+bool make_big_plan(int L, int most, FftPlan* plan);
 
 }  // namespace fh
 

@@ -311,14 +311,17 @@ bool make_plan(int L, FftPlan* plan) {
   return true;
 }
 
-// fewest factors of n (no prime above 13) among 2 .. 16, then the smallest sum
-static bool big_factors(int n, int most, int* r, int* np, int* sum) {
+// fewest factors of n (no prime above 13) among 2 .. most and the primes, then the
+// smallest sum; no factor above `cap` (falling order)
+static bool big_factors(int n, int most, int cap, int* r, int* np, int* sum) {
   if (n == 1) { *np = 0; *sum = 0; return true; }
   bool found = false;
-  for (int f = std::min(most, n); f >= 2; --f) {   // factors in falling order
+  for (int f = std::min(cap, n); f >= 2; --f) {
     if (n % f != 0) continue;
+    const bool prime = f == 2 || f == 3 || f == 5 || f == 7 || f == 11 || f == 13;
+    if (f > most && !prime) continue;
     int sub[24], k = 0, sm = 0;
-    if (!big_factors(n / f, f, sub, &k, &sm) || k + 1 > 24) continue;
+    if (!big_factors(n / f, most, f, sub, &k, &sm) || k + 1 > 24) continue;
     if (!found || k + 1 < *np || (k + 1 == *np && sm + f < *sum)) {
       found = true;
       *np = k + 1;
@@ -330,7 +333,7 @@ static bool big_factors(int n, int most, int* r, int* np, int* sum) {
   return found;
 }
 
-bool make_big_plan(int L, FftPlan* plan) {
+bool make_big_plan(int L, int most, FftPlan* plan) {
   FftPlan p, rest;
   if (!make_plan(L, &rest)) return false;
   p.L = L;
@@ -341,7 +344,7 @@ bool make_big_plan(int L, FftPlan* plan) {
       n /= rest.r[q];
     }
   int r[24], np = 0, sum = 0;
-  if (!big_factors(n, 16, r, &np, &sum) || p.np + np > 24) return false;
+  if (!big_factors(n, most, 16, r, &np, &sum) || p.np + np > 24) return false;
   for (int q = 0; q < np; ++q) p.r[p.np++] = r[q];
   *plan = p;
   return true;

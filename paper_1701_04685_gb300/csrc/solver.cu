@@ -73,6 +73,7 @@ struct Axis {
   int L = 1;
   DevPlan plan{};        // radix schedule of the cluster kernel for powers of two (and the default)
   DevPlan big{};         // its schedule for other grids (radices up to 16)
+  DevPlan tiny{};        // its FP64 schedule for few points a thread (radices up to 4)
   DevPlan planp[2]{};    // radix schedule of the passes per bulk precision (autotuned)
   double2* tw64 = nullptr;
   float2* tw32 = nullptr;
@@ -396,8 +397,8 @@ bool col_gen(const fh_solver* s, int prec, int a) {
 // 8 in FP32, 4 in FP64 (whose tile of 8 would leave one block per SM)
 template <typename T>
 constexpr int col2_ct() { return sizeof(T) == 4 ? fh::kColTile : 4; }
-template <typename T, int MODE>
-constexpr int col2_mb() { return sizeof(T) == 4 ? fh::col2_minb<MODE>() : 3; }
+template <typename T, int MODE, int N>
+constexpr int col2_mb() { return sizeof(T) == 4 ? fh::col2_minb<MODE, N>() : 3; }
 
 template <typename T, int R1, int R2, int MODE>
 void launch_col2(fh_solver* s, int a, int nload) {
@@ -408,7 +409,7 @@ void launch_col2(fh_solver* s, int a, int nload) {
   for (int k = a + 1; k + 1 < g.nd; ++k) stride *= g.dims[k];
   const long long ncols = g.nhalf / g.dims[a];
   const long long tiles = (ncols + CT - 1) / CT;
-  fh::line_pass_2s<R1, R2, MODE, CT, col2_mb<T, MODE>(), T>
+  fh::line_pass_2s<R1, R2, MODE, CT, col2_mb<T, MODE, R1 * R2>(), T>
       <<<(unsigned)(tiles * nload), fh::Col2<R1, R2, CT, T>::THREADS, fh::col2_smem<R1, R2, CT, T>(), s->work>>>(
           g, twp<T>(s->ax[a]), reinterpret_cast<C*>(s->S), Gptr<T>(s), s->st, stride, ncols, nload);
 }
@@ -645,13 +646,13 @@ template <typename T, int R1, int R2>
 cudaError_t set_col2_attrs() {
   constexpr int CT = col2_ct<T>();
   const int sm = (int)fh::col2_smem<R1, R2, CT, T>();
-  cudaError_t e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 0, CT, col2_mb<T, 0>(), T>,
+  cudaError_t e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 0, CT, col2_mb<T, 0, R1 * R2>(), T>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 1, CT, col2_mb<T, 1>(), T>,
+    e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 1, CT, col2_mb<T, 1, R1 * R2>(), T>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 2, CT, col2_mb<T, 2>(), T>,
+    e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 2, CT, col2_mb<T, 2, R1 * R2>(), T>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   return e;
 }
@@ -1118,6 +1119,17 @@ fh::ClusterTask cluster_task(const fh_solver* s, int l) {
   const bool pow2 = pow2_plans(s);
   t.plan0 = pow2 ? s->ax[0].plan : s->ax[0].big;
   t.plan1 = pow2 ? s->ax[1].plan : s->ax[1].big;
+  if (sizeof(T) == 8) {
+    // An FP64 warp instruction takes its quarter of the SM 64 cycles whatever its lanes
+    // do, so a small grid's stage lasts one thread's butterfly: radix 4 where there are
+    // at most two points a thread (32^2: 19.6 -> 17.4 us an iteration; with 3.4 points,
+    // 96^2, 48.7 -> 52.1).  Counted for clusters of 8 in either size, so that a solve's
+    // bits do not depend on the cluster that a batch or the tuner picks (64^2 on 16
+    // CTAs, 29.0 against 24.4, stays with the large radices for that).
+    const fh::ClusterLayout lay = fh::cluster_layout<T>(s->g.dims[0], s->g.L, s->g.nv, 8, true);
+    if (s->g.nv * lay.cols_max * s->g.dims[0] <= 2 * cluster_threads<T>()) t.plan0 = s->ax[0].tiny;
+    if (lay.npair_max * s->g.L <= 2 * cluster_threads<T>()) t.plan1 = s->ax[1].tiny;
+  }
   t.split0 = fh::line_split(s->g.dims[0]);
   t.split1 = fh::line_split(s->g.L);
   t.tw0 = twp<T>(s->ax[0]);
@@ -1653,10 +1665,13 @@ fh_status fh_solver_create(const fh_pattern* p, const fh_generator* gen, int nlo
     s->ax[k].plan.np = fp.np;
     for (int q = 0; q < 24; ++q) s->ax[k].plan.r[q] = fp.r[q];
     s->ax[k].planp[0] = s->ax[k].planp[1] = s->ax[k].plan;
-    if (!fh::make_big_plan(g.dims[k], &fp)) { delete s; fh::set_error("SNF axis length needs more than 24 radix stages"); return FH_ERR_UNSUPPORTED; }
-    s->ax[k].big.L = fp.L;
-    s->ax[k].big.np = fp.np;
-    for (int q = 0; q < 24; ++q) s->ax[k].big.r[q] = fp.r[q];
+    for (int q = 0; q < 2; ++q) {
+      if (!fh::make_big_plan(g.dims[k], q ? 4 : 16, &fp)) { delete s; fh::set_error("SNF axis length needs more than 24 radix stages"); return FH_ERR_UNSUPPORTED; }
+      fh::DevPlan& p = q ? s->ax[k].tiny : s->ax[k].big;
+      p.L = fp.L;
+      p.np = fp.np;
+      std::copy(fp.r, fp.r + 24, p.r);
+    }
   }
   choose_shapes(s, FH_PREC_FP64);
   choose_shapes(s, FH_PREC_FP32);

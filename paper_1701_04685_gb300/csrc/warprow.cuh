@@ -502,8 +502,12 @@ constexpr int kWarpRowThreads = 256;
 // KINV (with FIRST = false): the inverse half of a Krylov operator
 // application, as in row_pass: W = X - y to Wout (X = E, y the inverse
 // transform), block sums of W . Yaux (Yaux = X when null) and W . W.
+// Resident blocks: the loads' latency bounds the pass, so rows of 32 and 64
+// points, whose 6 P values a lane leave room, run three blocks per SM (80
+// registers; with the short tail of finish_row_pass, 64^3 x 6 loads 62.6 -> 48.6 us).  Three spill
+// at P = 4.
 template <typename T, int P, bool FIRST, bool KINV = false>
-__global__ void __launch_bounds__(kWarpRowThreads, (P <= 4 ? 2 : 1)) row_pass_warp6(GridInfo g, const cplx<T>* __restrict__ twg,
+__global__ void __launch_bounds__(kWarpRowThreads, (P <= 2 ? 3 : P <= 4 ? 2 : 1)) row_pass_warp6(GridInfo g, const cplx<T>* __restrict__ twg,
                                                                   T* __restrict__ E, cplx<T>* __restrict__ S,
                                                                   const uint8_t* __restrict__ phase,
                                                                   const T* __restrict__ dC, Control* ctl,
