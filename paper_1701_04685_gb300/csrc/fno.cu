@@ -120,7 +120,6 @@ struct fh_fno {
   // a kernel whose bounded wait gave up
   bool tensor_cores = true;
   int* tc_err = nullptr;
-  double* h_part = nullptr;   // pinned: the error word (slot 0) and the block sums behind it
 };
 
 namespace {
@@ -217,14 +216,11 @@ fh_status hidden_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
   return FH_OK;
 }
 
-// Waits for the stream with the error word that a tensor-core layer leaves when its
-// bounded wait gave up, and the first nparts block sums, read in the same wait.
-fh_status finish(fh_fno* f, int nparts) {
-  int* herr = reinterpret_cast<int*>(f->h_part);
-  FCK(cudaMemcpyAsync(herr, f->tc_err, sizeof(int), cudaMemcpyDeviceToHost, f->stream));
-  if (nparts > 0) FCK(cudaMemcpyAsync(f->h_part + 1, f->part, nparts * sizeof(double), cudaMemcpyDeviceToHost, f->stream));
-  FCK(cudaStreamSynchronize(f->stream));
-  if (*herr != 0) {
+// a tensor-core layer whose bounded wait gave up leaves an error word
+fh_status tc_status(fh_fno* f) {
+  int h = 0;
+  FCK(cudaMemcpy(&h, f->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
+  if (h != 0) {
     FCK(cudaMemset(f->tc_err, 0, sizeof(int)));
     fh::set_error("a tensor-core layer's wait for its MMAs gave up");
     return FH_ERR_TIMEOUT;
@@ -409,7 +405,6 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
   if ((e = cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return fail(e);
   f->nparts = 8 * f->sms;   // at least the resident blocks of a row kernel
   if ((e = cudaMalloc(&f->part, f->nparts * sizeof(double))) != cudaSuccess) return fail(e);
-  if ((e = cudaMallocHost(&f->h_part, (1 + f->nparts) * sizeof(double))) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc(&f->tc_err, sizeof(int))) != cudaSuccess) return fail(e);
   if ((e = cudaMemset(f->tc_err, 0, sizeof(int))) != cudaSuccess) return fail(e);
   cudaMemset(f->prm, 0, o * 4);
@@ -448,7 +443,6 @@ void fh_fno_destroy(fh_fno* f) {
                   f->Yz, f->Yy, f->y, f->gy, f->ga, f->gb, f->part, f->flat, f->tc_err};
   for (void* p : ptrs)
     if (p) cudaFree(p);
-  if (f->h_part) cudaFreeHost(f->h_part);
   delete f;
 }
 
@@ -544,7 +538,8 @@ fh_status fh_fno_forward(fh_fno* f, int batch, const float* x, float* y) {
   fh_status rc = forward_all(f, batch, x, direct ? y : f->y, nullptr, nullptr);
   if (rc != FH_OK) return rc;
   if (!direct) FCK(cudaMemcpyAsync(y, f->y, (size_t)batch * f->d.cout * f->d.N3 * 4, cudaMemcpyDefault, f->stream));
-  return finish(f, 0);
+  FCK(cudaStreamSynchronize(f->stream));
+  return tc_status(f);
 }
 
 fh_status fh_fno_set_tensor_cores(fh_fno* f, int enable) {
@@ -595,14 +590,15 @@ fh_status fh_fno_loss_grad(fh_fno* f, int batch, const float* x, const float* ta
   // lift
   rc = weight_grad(f, batch, d.cin, d.W, gu, x, f->off_P, f->off_p);
   if (rc != FH_OK) return rc;
-  rc = finish(f, gb);
-  if (rc != FH_OK && rc != FH_ERR_TIMEOUT) return rc;
+  std::vector<double> parts(gb);
+  FCK(cudaMemcpyAsync(parts.data(), f->part, gb * sizeof(double), cudaMemcpyDeviceToHost, f->stream));
+  FCK(cudaStreamSynchronize(f->stream));
   if (loss) {
     double s = 0.0;
-    for (int q = 0; q < gb; ++q) s += f->h_part[1 + q];
+    for (double p : parts) s += p;
     *loss = s / (double)ny;
   }
-  return rc;
+  return tc_status(f);
 }
 
 fh_status fh_fno_adam_step(fh_fno* f, float lr, float beta1, float beta2, float eps, int step) {
