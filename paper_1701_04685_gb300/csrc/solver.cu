@@ -232,7 +232,7 @@ void choose_shapes(fh_solver* s, int prec) {
     }
   }
   // FP64 3-D fields whose contiguous axis is 32, 64 or 128 points long: the
-  // two-step row pass (128^3 x 6 loads: 5.4 ms against 7.5 ms for the block
+  // two-step row pass (128^3 x 6 loads: 4.5 ms against 7.5 ms for the block
   // row pass; in FP32 the warp row pass is faster, 0.288 against 0.354 ms)
   s->row2[prec] = 0;
   if (prec == FH_PREC_FP64 && g.nv == 6 && (g.L == 32 || g.L == 64 || g.L == 128)) {
@@ -268,7 +268,7 @@ void choose_shapes(fh_solver* s, int prec) {
     auto blocks = [&](int w) { return (long long)nl * others * ((g.H + w - 1) / w); };
     const int wmin = prec == FH_PREC_FP64 ? 2 : 4;
     // FP64 allows a wider tile (four 128-point columns: 99 KB, two blocks per
-    // SM), measured faster than two (5.07 against 5.38 ms for the axis-0 pass
+    // SM), measured faster than two (5.07 against 5.38 ms for the axis-0 block pass
     // at 128^3 x 6 loads)
     const size_t line_cap = (prec == FH_PREC_FP64 ? 112 : 96) * 1024;
     while (W > wmin && (smem(W) > line_cap || blocks(W) < 2 * sms)) W /= 2;
