@@ -94,7 +94,8 @@ struct fh_fno {
   // parameters (FP32 master): P [W][cin], p [W], Wl [L][W][W], wl [L][W], R [L][NM][W][W] complex, Q [cout][W], q [cout]
   long long off_P, off_p, off_W, off_w, off_R, off_Q, off_q, nparam;
   float* prm = nullptr;
-  float* grd = nullptr;
+  float* grd_mem = nullptr;
+  float* grd = nullptr;   // in grd_mem, placed so that the gradient of R is 16-byte aligned for any channel counts
   float* m1 = nullptr;
   float* m2 = nullptr;
   __nv_bfloat16* Wbf = nullptr;   // [L][W][W]
@@ -384,7 +385,8 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
   cudaError_t e;
   const size_t act = (size_t)max_batch * width * d.N3;
   if ((e = cudaMalloc(&f->prm, o * 4)) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc(&f->grd, o * 4)) != cudaSuccess) return fail(e);
+  if ((e = cudaMalloc(&f->grd_mem, (o + 3) * 4)) != cudaSuccess) return fail(e);
+  f->grd = f->grd_mem + (4 - f->off_R % 4) % 4;
   if ((e = cudaMalloc(&f->m1, o * 4)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc(&f->m2, o * 4)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc(&f->Wbf, (size_t)layers * width * width * 2)) != cudaSuccess) return fail(e);
@@ -439,7 +441,7 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
 
 void fh_fno_destroy(fh_fno* f) {
   if (!f) return;
-  void* ptrs[] = {f->prm, f->grd, f->m1, f->m2, f->Wbf, f->Rbf, f->tw, f->zt, f->v, f->u, f->vh,
+  void* ptrs[] = {f->prm, f->grd_mem, f->m1, f->m2, f->Wbf, f->Rbf, f->tw, f->zt, f->v, f->u, f->vh,
                   f->Yz, f->Yy, f->y, f->gy, f->ga, f->gb, f->part, f->flat, f->tc_err};
   for (void* p : ptrs)
     if (p) cudaFree(p);

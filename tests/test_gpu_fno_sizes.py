@@ -2,7 +2,7 @@
 oracle: rows that are no multiple of four points, channels that fill no group of
 eight or 32, a single channel and mode, modes up to half the axis, batches that
 straddle the voxel chunks of the weight gradient, several blocks of the mixing
-matrices.  Forward within 2e-5 of the largest value, the gradient along a random
+matrices, an odd number of parameters before R.  Forward within 2e-5 of the largest value, the gradient along a random
 direction of every parameter block within 2e-3 of the oracle's central finite
 difference (the bounds of the other network tests)."""
 import numpy as np
@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 
 # n, cin, cout, width, modes, layers, batch
 SIZES = [(4, 1, 1, 1, 1, 1, 1), (5, 2, 3, 2, 2, 2, 3), (8, 7, 6, 33, 4, 1, 2), (15, 3, 5, 5, 7, 2, 2), (20, 1, 36, 12, 10, 1, 3),
-         (22, 9, 41, 17, 5, 1, 2), (16, 1, 4, 56, 2, 1, 1), (40, 1, 2, 8, 3, 1, 1)]
+         (22, 9, 41, 17, 5, 1, 2), (16, 1, 4, 56, 2, 1, 1), (40, 1, 2, 8, 3, 1, 1),
+         (6, 2, 3, 5, 3, 1, 2)]
 
 
 @pytest.mark.parametrize("size", SIZES, ids=["-".join(map(str, s)) for s in SIZES])
