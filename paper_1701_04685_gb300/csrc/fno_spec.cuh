@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kSpecThreads) k_idft_y(int N, int m, int W, in
 // Fusing the three steps leaves one read and one write of the columns and one
 // read of R: bound by R's 4 W^2 bytes per mode (28 MB a layer at W = 32, m = 12).
 // 64^3, one sample: 22 us where the separate x transforms and the mixing took 95;
-// four samples forward and backward: 50 and 144 us (243 and 241).
+// four samples forward and backward: 50 and 87 us (243 and 241).
 template <bool BACK>
 __global__ void __launch_bounds__(kSpecThreads) k_mix_x(int N, int m, int W, int B, int BC, int RS, SpecDiv dv,
                                                         const __nv_bfloat162* __restrict__ R, float2* __restrict__ Yy,
@@ -296,19 +296,60 @@ __global__ void __launch_bounds__(kSpecThreads) k_mix_x(int N, int m, int W, int
           if (b + 1 < bc) cs[((b + 1) * m2 + a0 + a) * W + o] = s1;
         }
       }
-      if (BACK)
-        for (int i = tid; i < na * WW; i += kSpecThreads) {
-          const int a = udiv(i, dv.WW), rem = i - a * WW, o = udiv(rem, dv.W), ii = rem - o * W;
-          float2* t = gR + (size_t)(mode0 + (a0 + a) * mode_ax) * WW + rem;
-          const float2 acc = *t;
-          float2 sum = make_float2(0.f, 0.f);
-          for (int b = 0; b < bc; ++b) {
-            const float2 gg = xs[(b * m2 + a0 + a) * W + o], xx = xv[(b * m2 + a0 + a) * W + ii];
-            sum.x += gg.x * xx.x + gg.y * xx.y;   // g conj(x)
-            sum.y += gg.y * xx.x - gg.x * xx.y;
+      if (BACK) {
+        // an entry's read, sum and write wait for memory: two entries of a row in one
+        // 16-byte access and four accesses in flight a thread (one 8-byte access at a
+        // time: 140 us a layer of 64^3, four samples; 87 us so)
+        constexpr int U = 4;
+        auto outer = [&](int a, int o, int ii, int b) {   // g conj(x)
+          const float2 gg = xs[(b * m2 + a0 + a) * W + o], xx = xv[(b * m2 + a0 + a) * W + ii];
+          return make_float2(gg.x * xx.x + gg.y * xx.y, gg.y * xx.x - gg.x * xx.y);
+        };
+        if ((W & 1) == 0) {
+          const int n2 = (na * WW) >> 1;
+          for (int i0 = tid; i0 < n2; i0 += U * kSpecThreads) {
+            float4 acc[U];
+            float4* t[U];
+            int a[U], o[U], ii[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int i = min(i0 + u * kSpecThreads, n2 - 1);
+              a[u] = udiv(2 * i, dv.WW);
+              const int rem = 2 * i - a[u] * WW;
+              o[u] = udiv(rem, dv.W);
+              ii[u] = rem - o[u] * W;
+              t[u] = reinterpret_cast<float4*>(gR + (size_t)(mode0 + (a0 + a[u]) * mode_ax) * WW + rem);
+              acc[u] = i0 + u * kSpecThreads < n2 ? *t[u] : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+              for (int b = 0; b < bc; ++b) {
+                const float2 p = outer(a[u], o[u], ii[u], b), q = outer(a[u], o[u], ii[u] + 1, b);
+                s0.x += p.x;
+                s0.y += p.y;
+                s1.x += q.x;
+                s1.y += q.y;
+              }
+              if (i0 + u * kSpecThreads < n2)
+                *t[u] = make_float4(acc[u].x + s0.x, acc[u].y + s0.y, acc[u].z + s1.x, acc[u].w + s1.y);
+            }
           }
-          *t = make_float2(acc.x + sum.x, acc.y + sum.y);
+        } else {
+          for (int i = tid; i < na * WW; i += kSpecThreads) {
+            const int a = udiv(i, dv.WW), rem = i - a * WW, o = udiv(rem, dv.W), ii = rem - o * W;
+            float2* t = gR + (size_t)(mode0 + (a0 + a) * mode_ax) * WW + rem;
+            const float2 acc = *t;
+            float2 sum = make_float2(0.f, 0.f);
+            for (int b = 0; b < bc; ++b) {
+              const float2 p = outer(a, o, ii, b);
+              sum.x += p.x;
+              sum.y += p.y;
+            }
+            *t = make_float2(acc.x + sum.x, acc.y + sum.y);
+          }
         }
+      }
     }
     __syncthreads();
     for (int i = tid; i < bc * (m - 1) * W; i += kSpecThreads) {
