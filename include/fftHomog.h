@@ -428,6 +428,10 @@ int fh_checked_build(void);
  * FH_ERR_INTERNAL naming the self test when the check caught the second.
  * Normal build: FH_ERR_UNSUPPORTED, nothing launched. */
 fh_status fh_check_selftest(void);
+/* Checked build: the nth pass along an axis that the library would launch from
+ * now on is not launched and reports an error on the host (nth = 0: none).  Not
+ * for use beside solves on other threads.  Normal build: FH_ERR_UNSUPPORTED. */
+fh_status fh_check_fail_launch(int nth);
 
 #ifdef __cplusplus
 }

@@ -97,6 +97,7 @@ def library():
             "fh_last_error": (C.c_char_p, []),
             "fh_checked_build": (I, []),
             "fh_check_selftest": (I, []),
+            "fh_check_fail_launch": (I, [I]),
         }
         for name, (res, args) in sig.items():
             f = getattr(lib, name)
@@ -113,7 +114,7 @@ def exported_symbols():
             "fh_set_stiffness_phases", "fh_set_stiffness_field", "fh_set_reference", "fh_solve", "fh_get_strain", "fh_set_strain",
             "fh_get_ceff", "fh_get_green", "fh_get_residuals", "fh_profile_passes", "fh_status_string",
             "fh_last_error", "fh_mean_stress_noalloc", "fh_solve_batch",
-            "fh_get_tuning", "fh_checked_build", "fh_check_selftest"]
+            "fh_get_tuning", "fh_checked_build", "fh_check_selftest", "fh_check_fail_launch"]
 
 
 def checked_build():
@@ -127,6 +128,11 @@ def check_selftest():
     FH_ERR_UNSUPPORTED.  Returns (status, message)."""
     rc = library().fh_check_selftest()
     return rc, library().fh_last_error().decode()
+
+
+def check_fail_launch(nth):
+    """Checked build: the nth axis pass from now fails on the host instead of running."""
+    _check(library().fh_check_fail_launch(int(nth)))
 
 
 def _check(rc, ok=(FH_OK,)):

@@ -153,6 +153,7 @@ struct fh_solver {
   int ntiles[2][3] = {};
   size_t line_smem[2][3] = {};
   std::vector<GraphEntry> graphs;
+  cudaError_t launch_err = cudaSuccess;   // first error of a pass's launch not reported yet (launch_status)
   bool cl_gsmem[2][2] = {{true, true}, {true, true}};  // [fp64/fp32][cluster 8/16]: table slice in smem
   LoadState* h_states = nullptr;                       // pinned copies read back after a phase
   double* h_ms = nullptr;
@@ -294,6 +295,26 @@ void save_default_shapes(fh_solver* s) {
   }
 }
 
+// Launch wrappers enqueue and return nothing; an error of theirs waits here for the
+// next launch_status, which every caller asks before it uses what was enqueued (a
+// solve that went on without one of its passes would contract to a wrong field).
+void note(fh_solver* s, cudaError_t e) {
+  if (s->launch_err == cudaSuccess) s->launch_err = e;
+}
+
+fh_status launch_status(fh_solver* s) {
+  const cudaError_t last = cudaGetLastError();
+  const cudaError_t e = s->launch_err != cudaSuccess ? s->launch_err : last;
+  s->launch_err = cudaSuccess;
+  if (e == cudaSuccess) return FH_OK;
+  fh::set_error(std::string("kernel launch: ") + cudaGetErrorString(e));
+  return FH_ERR_CUDA;
+}
+
+#ifdef FH_CHECKED
+int g_fail_launch = 0;   // > 0: that many axis passes from now, one fails on the host (fh_check_fail_launch)
+#endif
+
 void clear_graphs(fh_solver* s) {
   for (auto& e : s->graphs) cudaGraphExecDestroy(e.exec);
   s->graphs.clear();
@@ -426,6 +447,12 @@ void launch_col2_mode(fh_solver* s, int a, int mode, int nload) {
 template <typename T>
 void launch_axis(fh_solver* s, int prec, int a, int mode, int nload) {
   const GridInfo& g = s->g;
+#ifdef FH_CHECKED
+  if (g_fail_launch > 0 && --g_fail_launch == 0) {
+    note(s, cudaErrorLaunchFailure);
+    return;
+  }
+#endif
   switch (col2_len(s, prec, a)) {
     case 32: launch_col2_mode<T, 4, 8>(s, a, mode, nload); return;
     case 64: launch_col2_mode<T, 8, 8>(s, a, mode, nload); return;
@@ -445,8 +472,8 @@ void launch_axis(fh_solver* s, int prec, int a, int mode, int nload) {
   for (int k = 0; k < a; ++k) n_outer *= g.dims[k];
   for (int k = a + 1; k + 1 < g.nd; ++k) n_inner *= g.dims[k];
   if (col_gen(s, prec, a)) {
-    fh::gen_col(mode, g, g.dims[a], twp<T>(s->ax[a]), reinterpret_cast<typename fh::cplx_t<T>::type*>(s->S), Gptr<T>(s), s->st,
-                n_inner * g.H, nload, s->work);
+    note(s, fh::gen_col(mode, g, g.dims[a], twp<T>(s->ax[a]), reinterpret_cast<typename fh::cplx_t<T>::type*>(s->S), Gptr<T>(s),
+                        s->st, n_inner * g.H, nload, s->work));
     return;
   }
   const long long blocks = (long long)nload * n_outer * n_inner * s->ntiles[prec][a];
@@ -529,9 +556,9 @@ void launch_plane(fh_solver* s, int nload) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, fh::plane_pass_warp6<P1, P2, FIRST>, g, (const float2*)s->ax[1].tw32,
-                     (const float2*)s->ax[2].tw32, s->E32, reinterpret_cast<float2*>(s->S), (const uint8_t*)s->phase,
-                     (const float*)dCptr<float>(s), s->ctl, s->st, s->partials, s->hist);
+  note(s, cudaLaunchKernelEx(&cfg, fh::plane_pass_warp6<P1, P2, FIRST>, g, (const float2*)s->ax[1].tw32,
+                             (const float2*)s->ax[2].tw32, s->E32, reinterpret_cast<float2*>(s->S), (const uint8_t*)s->phase,
+                             (const float*)dCptr<float>(s), s->ctl, s->st, s->partials, s->hist));
 }
 
 template <bool FIRST>
@@ -573,8 +600,9 @@ bool use_rowg(const fh_solver* s, int prec) {
 
 template <typename T, bool FIRST, bool KINV>
 int enqueue_rowg(fh_solver* s, int prec, int nload, T* X, const T* dC, Control* ctl, T* Wout, const T* Yaux, int form) {
-  fh::gen_row(FIRST, KINV, s->g, twp<T>(s->ax[s->g.nd - 1]), X, reinterpret_cast<typename fh::cplx_t<T>::type*>(s->S), s->phase,
-              dC, ctl, s->st, s->partials, s->hist, nload, s->rowg_rb[prec], Wout, Yaux, field_ptr<T>(s, form), s->work);
+  note(s, fh::gen_row(FIRST, KINV, s->g, twp<T>(s->ax[s->g.nd - 1]), X, reinterpret_cast<typename fh::cplx_t<T>::type*>(s->S),
+                      s->phase, dC, ctl, s->st, s->partials, s->hist, nload, s->rowg_rb[prec], Wout, Yaux, field_ptr<T>(s, form),
+                      s->work));
   return s->rowg_bpl[prec];
 }
 
@@ -766,31 +794,31 @@ fh_status set_smem_attrs(fh_solver* s, int prec) {
   return s->g.nv == 3 ? set_smem_attrs_nv<T, 3>(s, prec) : set_smem_attrs_nv<T, 6>(s, prec);
 }
 
-template <typename T>
-fh_status get_graph(fh_solver* s, int prec, int nload, int chunk, cudaGraphExec_t* out) {
-  const int variant = s->plane_on ? 2 : 0;   // graphs with and without the plane pass differ
+// The graph of `chunk` iterations that `iterate` enqueues, captured on first use.  A
+// graph is kept only if every launch in it succeeded.
+template <typename Iterate>
+fh_status get_graph(fh_solver* s, int prec, int nload, int chunk, int variant, cudaGraphExec_t* out, Iterate iterate) {
   for (auto& e : s->graphs)
     if (e.prec == prec && e.nload == nload && e.chunk == chunk && e.method == variant) {
       *out = e.exec;
       return FH_OK;
     }
   CK(cudaStreamBeginCapture(s->work, cudaStreamCaptureModeThreadLocal));
-  for (int i = 0; i < chunk; ++i) {
-    enqueue_line_passes<T>(s, prec, nload);
-    enqueue_row_pass<T, false>(s, prec, nload);
+  for (int i = 0; i < chunk; ++i) iterate();
+  cudaGraph_t graph = nullptr;
+  const cudaError_t end = cudaStreamEndCapture(s->work, &graph);
+  fh_status rc = launch_status(s);
+  if (rc == FH_OK) {
+    cudaError_t e = end;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, graph, 0);
+    if (e != cudaSuccess) {
+      fh::set_error(std::string("graph of the iterations: ") + cudaGetErrorString(e));
+      rc = FH_ERR_CUDA;
+    }
   }
-  cudaGraph_t graph;
-  CK(cudaStreamEndCapture(s->work, &graph));
-  cudaGraphExec_t exec;
-  cudaError_t e = cudaGraphInstantiate(&exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) {
-    fh::set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e));
-    return FH_ERR_CUDA;
-  }
-  s->graphs.push_back({prec, nload, chunk, variant, exec});
-  *out = exec;
-  return FH_OK;
+  if (graph) cudaGraphDestroy(graph);
+  if (rc == FH_OK) s->graphs.push_back({prec, nload, chunk, variant, *out});
+  return rc;
 }
 
 // mean stresses of the field X: about four blocks per SM over all loads
@@ -841,7 +869,8 @@ fh_status run_iterations(fh_solver* s, int nload, int chunk, int max_iter, doubl
       CK(cudaGraphLaunch(exec, s->work));
     } else {
       for (int i = 0; i < n; ++i) iterate();
-      CK(cudaGetLastError());
+      fh_status rc = launch_status(s);
+      if (rc != FH_OK) return rc;
     }
     *launched += n;
     ran = n;
@@ -866,7 +895,7 @@ fh_status run_solve(fh_solver* s, int prec, int nload, int chunk, int max_iter, 
   if (rc != FH_OK) return rc;
   CK(cudaEventRecord(s->ev0, s->work));
   enqueue_row_pass<T, true>(s, prec, nload);
-  CK(cudaGetLastError());
+  if ((rc = launch_status(s)) != FH_OK) return rc;
   long long launched = 0, extra = 0;
   bool finished = false;
   if (s->polish && prec == FH_PREC_FP64 && (use_row2(s, prec) || use_rowg(s, prec)) && !s->plane_on) {
@@ -880,7 +909,7 @@ fh_status run_solve(fh_solver* s, int prec, int nload, int chunk, int max_iter, 
     CK(cudaMemsetAsync(&s->ctl->no_forward, 1, sizeof(int), s->work));
     enqueue_row_pass<T, false>(s, prec, nload);
     CK(cudaMemsetAsync(&s->ctl->no_forward, 0, sizeof(int), s->work));
-    CK(cudaGetLastError());
+    if ((rc = launch_status(s)) != FH_OK) return rc;
     launched = 1;
     CK(cudaMemcpyAsync(s->h_states, s->st, sizeof(LoadState) * nload, cudaMemcpyDeviceToHost, s->work));
     CK(cudaStreamSynchronize(s->work));
@@ -888,21 +917,22 @@ fh_status run_solve(fh_solver* s, int prec, int nload, int chunk, int max_iter, 
     for (int l = 0; l < nload; ++l) finished = finished && s->h_states[l].done;
     if (!finished) {
       enqueue_row_pass<T, true>(s, prec, nload);
-      CK(cudaGetLastError());
+      if ((rc = launch_status(s)) != FH_OK) return rc;
       extra = 1;
     }
   }
   if (!finished) {
+    auto iterate = [&] {
+      enqueue_line_passes<T>(s, prec, nload);
+      enqueue_row_pass<T, false>(s, prec, nload);
+    };
+    const int variant = s->plane_on ? 2 : 0;   // graphs with and without the plane pass differ
     rc = run_iterations(s, nload, chunk, max_iter, tol, &launched,
-                        [&](cudaGraphExec_t* exec) { return get_graph<T>(s, prec, nload, chunk, exec); },
-                        [&] {
-                          enqueue_line_passes<T>(s, prec, nload);
-                          enqueue_row_pass<T, false>(s, prec, nload);
-                        });
+                        [&](cudaGraphExec_t* exec) { return get_graph(s, prec, nload, chunk, variant, exec, iterate); }, iterate);
     if (rc != FH_OK) return rc;
   }
   if (!s->skip_mean) enqueue_mean_stress<T>(s, nload, Eptr<T>(s));
-  CK(cudaGetLastError());
+  if ((rc = launch_status(s)) != FH_OK) return rc;
   CK(cudaEventRecord(s->ev1, s->work));
   *launches = (s->skip_mean ? 1 : 2) + extra + launched * (1 + line_launches_per_iter(s, prec));
   return FH_OK;
@@ -1021,31 +1051,14 @@ fh_status run_bicgstab(fh_solver* s, int prec, int nload, int chunk, int max_ite
   fh::kry_init<T><<<nload * kKryBpl, fh::kKryThreads, 0, s->work>>>(r, kry_field<T>(s, prec, KRH), x, s->st, s->ctl,
                                                                      s->g.m, s->g.nv, kKryBpl, s->kpart);
   fh::kry_scalars<0><<<1, fh::kKryThreads, 0, s->work>>>(s->ksc, s->st, s->ctl, s->hist, s->kpart, 3, kKryBpl);
-  CK(cudaGetLastError());
+  if ((rc = launch_status(s)) != FH_OK) return rc;
   long long launched = 0;
-  auto graph = [&](cudaGraphExec_t* out) -> fh_status {
-    for (auto& e : s->graphs)
-      if (e.prec == prec && e.nload == nload && e.chunk == chunk && e.method == 1) {
-        *out = e.exec;
-        return FH_OK;
-      }
-    CK(cudaStreamBeginCapture(s->work, cudaStreamCaptureModeThreadLocal));
-    for (int i = 0; i < chunk; ++i) enqueue_bicgstab_iteration<T>(s, prec, nload);
-    cudaGraph_t graph;
-    CK(cudaStreamEndCapture(s->work, &graph));
-    cudaError_t e = cudaGraphInstantiate(out, graph, 0);
-    cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-      fh::set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e));
-      return FH_ERR_CUDA;
-    }
-    s->graphs.push_back({prec, nload, chunk, 1, *out});
-    return FH_OK;
-  };
-  rc = run_iterations(s, nload, chunk, max_iter, tol, &launched, graph, [&] { enqueue_bicgstab_iteration<T>(s, prec, nload); });
+  auto iterate = [&] { enqueue_bicgstab_iteration<T>(s, prec, nload); };
+  rc = run_iterations(s, nload, chunk, max_iter, tol, &launched,
+                      [&](cudaGraphExec_t* exec) { return get_graph(s, prec, nload, chunk, 1, exec, iterate); }, iterate);
   if (rc != FH_OK) return rc;
   if (!s->skip_mean) enqueue_mean_stress<T>(s, nload, x);
-  CK(cudaGetLastError());
+  if ((rc = launch_status(s)) != FH_OK) return rc;
   CK(cudaEventRecord(s->ev1, s->work));
   *launches = (2 + line_launches_per_iter(s->g)) + 2 + (s->skip_mean ? 0 : 1) + launched * kry_launches_per_iter(s->g);
   return FH_OK;
@@ -1438,10 +1451,10 @@ fh_status profile_passes(fh_solver* s, int prec, int nload, int reps, double* ms
   for (int q = 0; q < 4; ++q) ms[q] = 0.0;
   auto timed = [&](int q, auto&& launch) -> fh_status {
     launch();
-    CK(cudaGetLastError());
     CK(cudaEventRecord(s->ev0, s->work));
     for (int i = 0; i < reps; ++i) launch();
     CK(cudaEventRecord(s->ev1, s->work));
+    if (fh_status e = launch_status(s); e != FH_OK) return e;
     CK(cudaEventSynchronize(s->ev1));
     float t = 0.f;
     CK(cudaEventElapsedTime(&t, s->ev0, s->ev1));
@@ -1530,6 +1543,17 @@ int fh_checked_build(void) {
   return 1;
 #else
   return 0;
+#endif
+}
+
+fh_status fh_check_fail_launch(int nth) {
+#ifdef FH_CHECKED
+  g_fail_launch = nth;
+  return FH_OK;
+#else
+  (void)nth;
+  fh::set_error("not a checked build (compile with FH_CHECKED)");
+  return FH_ERR_UNSUPPORTED;
 #endif
 }
 
