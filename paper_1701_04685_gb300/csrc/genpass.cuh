@@ -13,10 +13,10 @@
 // 0.6 ms an iteration against 2.6 ms (a solve of 20 iterations 13.6 against 53.6 ms).
 //
 // Line layout: row k1 at offset (R2 | 1) k1, so that its stride is odd.  Column
-// tiles: CT = 8 columns a block in FP32 3-D, else 4 (FP64: shared memory; 2-D: a
-// 512^2 grid with 3 loads has only 771 columns), line stride 16 / CT mod 16 (FP64:
-// 2): the lanes of an access phase fall on distinct banks.  Row lines: stride R2
-// mod 16, so that consecutive entries of consecutive lines follow one another.
+// tiles: CT = 8 columns a block in FP32 3-D as far as shared memory goes (N <= 512),
+// else 4 (gen_columns; FP64: shared memory; 2-D: a 512^2 grid with 3 loads has only
+// 771 columns).  Row lines: stride R2 mod 16, so that consecutive entries of
+// consecutive lines follow one another.
 // 512^2 x 3 loads FP32 with point-by-point stiffness: 63 us an iteration against
 // 132 us (block row pass 79, block line pass 53).
 #pragma once
@@ -26,7 +26,6 @@
 
 namespace fh {
 
-template <typename T, int NV> __host__ __device__ constexpr int gen_ct() { return sizeof(T) == 4 && NV == 6 ? 8 : 4; }
 template <typename T, int NV> __host__ __device__ constexpr int gen_threads() { return sizeof(T) == 4 && NV == 6 ? 384 : 256; }
 template <typename T> __host__ __device__ constexpr int gen_rmax() { return sizeof(T) == 4 ? 32 : 16; }
 
@@ -52,12 +51,12 @@ __device__ __forceinline__ C twiddle(const C* tw, int t) {
 }
 
 // MODE 0 forward, 1 inverse, 2 forward + Green step + inverse (axis 0), as line_pass_2s
-template <typename T, int NV, int MODE>
+template <typename T, int NV, int MODE, int CT>
 __global__ void __launch_bounds__(gen_threads<T, NV>(), 2)
     line_pass_gen(GridInfo g, GenShape K, const cplx<T>* __restrict__ twg, cplx<T>* __restrict__ S,
                   const T* __restrict__ Gt, const LoadState* st, long long stride, long long ncols, int nload) {
   using C = cplx<T>;
-  constexpr int NTRI = NV * (NV + 1) / 2, CT = gen_ct<T, NV>(), RM = gen_rmax<T>();
+  constexpr int NTRI = NV * (NV + 1) / 2, RM = gen_rmax<T>();
   constexpr int DIR = MODE == 1 ? 1 : -1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* tw = reinterpret_cast<C*>(smem_raw);   // tw[t] = exp(-2 pi i t / N)
@@ -454,17 +453,20 @@ __global__ void __launch_bounds__(gen_threads<T, NV>(), 2)
   finish_row_pass(ctl, st, partials, hist, blocks_per_load);
 }
 
-inline GenShape gen_shape(int N, bool fp32, bool rows, int ct, int H) {
+inline GenShape gen_shape(int N, bool fp32, int H) {
   GenShape K{};
   K.N = N;
   gen_split(N, fp32, &K.R1, &K.R2);
-  K.RS = K.R2 | 1;
-  const int need = K.R1 * K.RS, mod = rows ? K.R2 % 16 : fp32 ? 16 / ct : 2;
-  K.LS = need + ((mod - need) % 16 + 16) % 16;
+  K.RS = gen_row_stride(K.R2);
   K.dR1 = make_muldiv(K.R1);
   K.dR2 = make_muldiv(K.R2);
   K.dN = make_muldiv(N);
   K.dH = make_muldiv(H);
+  return K;
+}
+inline GenShape gen_row_shape(int N, bool fp32, int H) {
+  GenShape K = gen_shape(N, fp32, H);
+  K.LS = gen_line_stride(K.R1, K.R2, K.R2 % 16);
   return K;
 }
 
@@ -473,7 +475,7 @@ inline GenShape gen_shape(int N, bool fp32, bool rows, int ct, int H) {
 template <typename T, int NV>
 int gen_rb(int L, long long rows_of_all_loads) {
   constexpr bool fp32 = sizeof(T) == 4;
-  const GenShape K = gen_shape(L, fp32, true, 1, 1);
+  const GenShape K = gen_row_shape(L, fp32, 1);
   int rb = std::max(1, 2 * (gen_threads<T, NV>() / K.R2) / NV);
   auto lines = [](int r) { return (r * NV + 1) / 2; };
   while (rb > 1 && (lines(rb) * K.R2 > gen_threads<T, NV>() || (size_t)(L + lines(rb) * K.LS) * 2 * sizeof(T) > 96 * 1024)) --rb;
@@ -481,13 +483,14 @@ int gen_rb(int L, long long rows_of_all_loads) {
   return (int)std::max<long long>(1, std::min<long long>(rb, want));
 }
 
-template <typename T, int NV>
-cudaError_t gen_col_t(int mode, const GridInfo& g, int N, const cplx<T>* tw, cplx<T>* S, const T* G, const LoadState* st,
+template <typename T, int NV, int CT>
+cudaError_t gen_col_ct(int mode, const GridInfo& g, int N, const cplx<T>* tw, cplx<T>* S, const T* G, const LoadState* st,
                       long long stride, int nload, cudaStream_t stream) {
-  constexpr int CT = gen_ct<T, NV>(), TH = gen_threads<T, NV>();
-  const GenShape K = gen_shape(N, sizeof(T) == 4, false, CT, 1);
+  constexpr int TH = gen_threads<T, NV>();
+  GenShape K = gen_shape(N, sizeof(T) == 4, 1);
+  K.LS = gen_col_stride(K.R1, K.R2, sizeof(T) == 4, CT);
   const long long ncols = g.nhalf / N, tiles = (ncols + CT - 1) / CT;
-  const size_t sm = (size_t)(N + NV * CT * K.LS) * 2 * sizeof(T);
+  const size_t sm = gen_col_bytes(N, sizeof(T) == 4, NV, CT);
   // a stage's NV CT R2 tasks in equal rounds
   const int tasks = NV * CT * K.R2, rounds = (tasks + TH - 1) / TH;
   const int threads = ((tasks + rounds - 1) / rounds + 31) / 32 * 32;
@@ -498,17 +501,26 @@ cudaError_t gen_col_t(int mode, const GridInfo& g, int N, const cplx<T>* tw, cpl
     return cudaGetLastError();
   };
   if constexpr (NV == 6) {   // 2-D grids have axis 0 only
-    if (mode == 0) return launch(line_pass_gen<T, NV, 0>);
-    if (mode == 1) return launch(line_pass_gen<T, NV, 1>);
+    if (mode == 0) return launch(line_pass_gen<T, NV, 0, CT>);
+    if (mode == 1) return launch(line_pass_gen<T, NV, 1, CT>);
   }
-  return launch(line_pass_gen<T, NV, 2>);
+  return launch(line_pass_gen<T, NV, 2, CT>);
+}
+
+template <typename T, int NV>
+cudaError_t gen_col_t(int mode, const GridInfo& g, int N, const cplx<T>* tw, cplx<T>* S, const T* G, const LoadState* st,
+                      long long stride, int nload, cudaStream_t stream) {
+  if constexpr (sizeof(T) == 4 && NV == 6) {
+    if (gen_columns(N, true, NV) == 8) return gen_col_ct<T, NV, 8>(mode, g, N, tw, S, G, st, stride, nload, stream);
+  }
+  return gen_col_ct<T, NV, 4>(mode, g, N, tw, S, G, st, stride, nload, stream);
 }
 
 template <typename T, int NV>
 cudaError_t gen_row_t(bool first, bool kinv, const GridInfo& g, const cplx<T>* tw, T* E, cplx<T>* S, const uint8_t* phase,
                       const T* dC, Control* ctl, LoadState* st, double* partials, double* hist, int nload, int rb, T* Wout,
                       const T* Yaux, const T* Cfld, cudaStream_t stream) {
-  const GenShape K = gen_shape(g.L, sizeof(T) == 4, true, 1, g.H);
+  const GenShape K = gen_row_shape(g.L, sizeof(T) == 4, g.H);
   const int bpl = (int)((g.nrows + rb - 1) / rb), lines = (rb * NV + 1) / 2;
   const size_t sm = (size_t)(g.L + lines * K.LS) * 2 * sizeof(T);
   const int threads = (lines * K.R2 + 31) / 32 * 32;

@@ -406,12 +406,11 @@ int col2_len(const fh_solver* s, int prec, int a) {
 }
 
 // The two-step column pass of general lengths (genpass.cuh) applies to the other
-// axes of R1 R2 points that neither the compile-time lengths above nor the warp
-// column pass take.
+// axes of R1 R2 points whose tile fits in a block and that neither the compile-time
+// lengths above nor the warp column pass take.
 bool col_gen(const fh_solver* s, int prec, int a) {
-  int r1, r2;
   return s->col2s && col2_len(s, prec, a) == 0 && col_warp_p(s, prec, a) == 0 &&
-         fh::gen_split(s->g.dims[a], prec == FH_PREC_FP32, &r1, &r2);
+         fh::gen_columns(s->g.dims[a], prec == FH_PREC_FP32, s->g.nv) > 0;
 }
 
 // columns per block and resident blocks per SM of the two-step column pass:
