@@ -25,14 +25,17 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "internal.hpp"
 #include "fno_rows.cuh"
 #include "fno_spec.cuh"
 #include "fno_tc.cuh"
+#include "smem.hpp"
 
 namespace {
 
@@ -117,6 +120,7 @@ struct fh_fno {
   double* part = nullptr;
   int nparts = 0;
   int sms = 1;
+  std::map<std::pair<int, size_t>, int> resident;   // see resident_rows
   // hidden layers on the tensor cores (fno_tc.cuh) where they apply; tc_err is set by
   // a kernel whose bounded wait gave up
   bool tensor_cores = true;
@@ -154,6 +158,19 @@ fhrow::RowArgs row_args(const fh_fno* f, int B, int cin, const float* in, const 
   return a;
 }
 
+// resident blocks per SM of a row kernel, asked for once per kernel and size
+template <int EPI>
+cudaError_t resident_rows(fh_fno* f, size_t sm, int* res) {
+  auto it = f->resident.find({EPI, sm});
+  if (it == f->resident.end()) {
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(res, fhrow::k_rows<EPI>, fhrow::kRowThreads, sm);
+    if (e != cudaSuccess) return e;
+    it = f->resident.insert({{EPI, sm}, *res}).first;
+  }
+  *res = it->second;
+  return cudaSuccess;
+}
+
 template <int EPI>
 fh_status launch_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
   const int nz4 = a.N4 / 4, per_row = (a.WP / 8) * nz4;
@@ -175,8 +192,7 @@ fh_status launch_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
   const size_t sm = fhrow::row_smem_floats(a) * 4;
   const int ntiles = (a.nrows + a.rpb - 1) / a.rpb;
   int res = 1;
-  FCK(cudaFuncSetAttribute(fhrow::k_rows<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  FCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, fhrow::k_rows<EPI>, fhrow::kRowThreads, sm));
+  FCK(resident_rows<EPI>(f, sm, &res));
   const int grid = std::min(ntiles, std::max(1, res) * f->sms);
   if (blocks) *blocks = grid;
   fhrow::k_rows<EPI><<<grid, fhrow::kRowThreads, sm, f->stream>>>(a);
@@ -208,8 +224,6 @@ fh_status hidden_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
   t.in = a.in; t.W = reinterpret_cast<const __nv_bfloat16*>(a.A); t.trans = a.a_trans; t.bias = a.bias;
   t.Iy = a.Iy; t.T = a.T; t.u_in = a.u_in; t.u_out = a.u_out; t.out = a.out; t.Yz = a.Yz; t.err = f->tc_err;
   const size_t sm = fhtc::tc_layout(d.N, t.Kp).total;
-  FCK(cudaFuncSetAttribute(fhtc::k_rows_tc<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  FCK(cudaFuncSetAttribute(fhtc::k_rows_tc<EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   // two CTAs share an SM where their shared memory allows (tensor memory has 512 columns)
   const int res = 2 * (sm + 2048) <= 228 * 1024 && 2 * t.ncols <= 512 ? 2 : 1;
   fhtc::k_rows_tc<EPI><<<std::min(t.ntiles, res * f->sms), fhtc::kTcThreads, sm, f->stream>>>(t);
@@ -248,7 +262,6 @@ fh_status dft_y(fh_fno* f, int B) {
   const size_t per = (size_t)2 * (d.N / 2 + 1) * d.W * sizeof(float2);
   const int kb = y_group(d, (d.m / 4 + 1) * d.W, per);
   const size_t sm = d.N * sizeof(float2) + kb * per;
-  FCK(cudaFuncSetAttribute(fhspec::k_dft_y, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   fhspec::k_dft_y<<<B * d.N * ((d.m + kb - 1) / kb), fhspec::kSpecThreads, sm, f->stream>>>(
       d.N, d.m, d.W, kb, spec_div(d), f->Yz, f->Yy, f->tw);
   FCK(cudaGetLastError());
@@ -260,7 +273,6 @@ fh_status idft_y(fh_fno* f, int B, float scale, int wz) {
   const size_t per = (size_t)2 * d.m * d.W * sizeof(float2);
   const int kb = y_group(d, (d.N / 8 + 1) * d.W, per);
   const size_t sm = d.N * sizeof(float2) + kb * per;
-  FCK(cudaFuncSetAttribute(fhspec::k_idft_y, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   fhspec::k_idft_y<<<B * d.N * ((d.m + kb - 1) / kb), fhspec::kSpecThreads, sm, f->stream>>>(
       d.N, d.m, d.W, kb, spec_div(d), f->Yy, f->Yz, f->tw, scale, wz);
   FCK(cudaGetLastError());
@@ -280,7 +292,6 @@ fh_status mix_x(fh_fno* f, int B, int l, float scale) {
   const size_t base = d.N * sizeof(float2) + bc * per_b;
   const int rs = (int)std::max<size_t>(1, std::min<size_t>(m2, base < half ? (half - base) / per_r : 1));
   const size_t sm = base + rs * per_r;
-  FCK(cudaFuncSetAttribute(fhspec::k_mix_x<BACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   fhspec::k_mix_x<BACK><<<m2 * d.m, fhspec::kSpecThreads, sm, f->stream>>>(
       d.N, d.m, d.W, B, bc, rs, spec_div(d), reinterpret_cast<const __nv_bfloat162*>(f->Rbf) + (size_t)l * d.NM * d.W * d.W, f->Yy,
       f->vh + (size_t)l * B * d.NM * d.W,
@@ -338,6 +349,25 @@ fh_status weight_grad(fh_fno* f, int B, int cin, int cout, const float* g, const
   fhrow::k_weight_grad<<<grid, fhrow::kWgThreads, 0, f->stream>>>(total, d.N3, cin, cout, vec, g, x, f->grd + off_A, f->grd + off_b);
   FCK(cudaGetLastError());
   return FH_OK;
+}
+
+// shared-memory limits of the kernels, once per network
+template <int EPI>
+cudaError_t prepare_rows() {
+  cudaError_t e = fh::allow_smem((const void*)fhrow::k_rows<EPI>);
+  if (e == cudaSuccess) e = fh::allow_smem((const void*)fhtc::k_rows_tc<EPI>);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fhtc::k_rows_tc<EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  return e;
+}
+cudaError_t prepare_kernels() {
+  cudaError_t e = prepare_rows<0>();
+  if (e == cudaSuccess) e = prepare_rows<1>();
+  if (e == cudaSuccess) e = prepare_rows<2>();
+  for (const void* k : {(const void*)fhspec::k_dft_y, (const void*)fhspec::k_idft_y, (const void*)fhspec::k_mix_x<false>,
+                        (const void*)fhspec::k_mix_x<true>})
+    if (e == cudaSuccess) e = fh::allow_smem(k);
+  return e;
 }
 
 fh_status refresh_bf16(fh_fno* f) {
@@ -405,6 +435,7 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return fail(e);
   if ((e = cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return fail(e);
+  if ((e = prepare_kernels()) != cudaSuccess) return fail(e);
   f->nparts = 8 * f->sms;   // at least the resident blocks of a row kernel
   if ((e = cudaMalloc(&f->part, f->nparts * sizeof(double))) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc(&f->tc_err, sizeof(int))) != cudaSuccess) return fail(e);

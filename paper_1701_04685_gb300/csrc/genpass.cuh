@@ -23,6 +23,7 @@
 
 #include "genpass.hpp"
 #include "gendft.cuh"
+#include "smem.hpp"
 
 namespace fh {
 
@@ -484,6 +485,30 @@ int gen_rb(int L, long long rows_of_all_loads) {
 }
 
 template <typename T, int NV, int CT>
+cudaError_t gen_col_prepare_ct() {
+  cudaError_t e = allow_smem((const void*)line_pass_gen<T, NV, 2, CT>);
+  if constexpr (NV == 6) {   // 2-D grids have axis 0 only
+    if (e == cudaSuccess) e = allow_smem((const void*)line_pass_gen<T, NV, 0, CT>);
+    if (e == cudaSuccess) e = allow_smem((const void*)line_pass_gen<T, NV, 1, CT>);
+  }
+  return e;
+}
+template <typename T, int NV>
+cudaError_t gen_col_prepare_t(int N) {
+  if constexpr (sizeof(T) == 4 && NV == 6) {
+    if (gen_columns(N, true, NV) == 8) return gen_col_prepare_ct<T, NV, 8>();
+  }
+  return gen_col_prepare_ct<T, NV, 4>();
+}
+template <typename T, int NV>
+cudaError_t gen_row_prepare_t() {
+  cudaError_t e = allow_smem((const void*)row_pass_gen<T, NV, true, false>);
+  if (e == cudaSuccess) e = allow_smem((const void*)row_pass_gen<T, NV, false, true>);
+  if (e == cudaSuccess) e = allow_smem((const void*)row_pass_gen<T, NV, false, false>);
+  return e;
+}
+
+template <typename T, int NV, int CT>
 cudaError_t gen_col_ct(int mode, const GridInfo& g, int N, const cplx<T>* tw, cplx<T>* S, const T* G, const LoadState* st,
                       long long stride, int nload, cudaStream_t stream) {
   constexpr int TH = gen_threads<T, NV>();
@@ -495,12 +520,10 @@ cudaError_t gen_col_ct(int mode, const GridInfo& g, int N, const cplx<T>* tw, cp
   const int tasks = NV * CT * K.R2, rounds = (tasks + TH - 1) / TH;
   const int threads = ((tasks + rounds - 1) / rounds + 31) / 32 * 32;
   auto launch = [&](auto kern) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     kern<<<(unsigned)(tiles * nload), threads, sm, stream>>>(g, K, tw, S, G, st, stride, ncols, nload);
     return cudaGetLastError();
   };
-  if constexpr (NV == 6) {   // 2-D grids have axis 0 only
+  if constexpr (NV == 6) {
     if (mode == 0) return launch(line_pass_gen<T, NV, 0, CT>);
     if (mode == 1) return launch(line_pass_gen<T, NV, 1, CT>);
   }
@@ -525,8 +548,6 @@ cudaError_t gen_row_t(bool first, bool kinv, const GridInfo& g, const cplx<T>* t
   const size_t sm = (size_t)(g.L + lines * K.LS) * 2 * sizeof(T);
   const int threads = (lines * K.R2 + 31) / 32 * 32;
   auto launch = [&](auto kern) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
     kern<<<(unsigned)(nload * bpl), threads, sm, stream>>>(g, K, rb, tw, E, S, phase, dC, ctl, st, partials, hist, bpl, Wout, Yaux,
                                                            Cfld);
     return cudaGetLastError();

@@ -9,11 +9,16 @@
 
 namespace fh {
 
-
 // rows per block of the row pass for rows of L points (gen_split), n_v components
 // and the given number of rows over all loads
 int gen_rows_per_block(double, int nv, int L, long long rows);
 int gen_rows_per_block(float, int nv, int L, long long rows);
+
+// once per solve, before the launches: the kernels' shared-memory limits (allow_smem)
+cudaError_t gen_col_prepare(double, int nv, int N);
+cudaError_t gen_col_prepare(float, int nv, int N);
+cudaError_t gen_row_prepare(double, int nv);
+cudaError_t gen_row_prepare(float, int nv);
 
 // pass along an axis of N points with element stride `stride` (modes as line_pass)
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const double2* tw, double2* S, const double* G,

@@ -9,6 +9,11 @@ int gen_rows_per_block(float, int nv, int L, long long rows) {
   return nv == 3 ? gen_rb<float, 3>(L, rows) : gen_rb<float, 6>(L, rows);
 }
 
+cudaError_t gen_col_prepare(float, int nv, int N) {
+  return nv == 3 ? gen_col_prepare_t<float, 3>(N) : gen_col_prepare_t<float, 6>(N);
+}
+cudaError_t gen_row_prepare(float, int nv) { return nv == 3 ? gen_row_prepare_t<float, 3>() : gen_row_prepare_t<float, 6>(); }
+
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const float2* tw, float2* S, const float* G, const LoadState* st,
                     long long stride, int nload, cudaStream_t stream) {
   return g.nv == 3 ? gen_col_t<float, 3>(mode, g, N, tw, S, G, st, stride, nload, stream)

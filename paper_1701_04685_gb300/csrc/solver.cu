@@ -14,6 +14,8 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -28,6 +30,7 @@
 #include "genpass.hpp"
 #include "gensplit.hpp"
 #include "clusterkern.hpp"
+#include "smem.hpp"
 #include "planewarp.cuh"
 
 namespace fh {
@@ -48,6 +51,27 @@ using fh::LoadState;
       return FH_ERR_CUDA;                                                            \
     }                                                                                \
   } while (0)
+
+namespace fh {
+cudaError_t allow_smem(const void* kernel) {
+  static std::mutex mutex;
+  static std::map<std::pair<int, const void*>, int> limits;   // per device and kernel
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mutex);
+  auto it = limits.find({dev, kernel});
+  if (it == limits.end()) {
+    cudaFuncAttributes attr{};
+    int most = 0;
+    if ((e = cudaFuncGetAttributes(&attr, kernel)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    it = limits.insert({{dev, kernel}, most - (int)attr.sharedSizeBytes}).first;
+  }
+  // set every time: a device reset forgets it
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, it->second);
+}
+}  // namespace fh
 
 namespace {
 
@@ -650,11 +674,11 @@ void enqueue_row_pass(fh_solver* s, int prec, int nload) {
 
 template <typename T, int P>
 cudaError_t set_warp_attrs(fh_solver* s, int prec, size_t rs) {
-  cudaError_t e = cudaFuncSetAttribute(fh::row_pass_warp6<T, P, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+  cudaError_t e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, true>);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fh::row_pass_warp6<T, P, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+  e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, false>);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(fh::row_pass_warp6<T, P, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+  e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, false, true>);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s->warp_res[prec], fh::row_pass_warp6<T, P, false>,
                                                        fh::kWarpRowThreads, rs);
@@ -662,34 +686,28 @@ cudaError_t set_warp_attrs(fh_solver* s, int prec, size_t rs) {
 
 template <int P>
 cudaError_t set_col_attrs() {
-  const int sm = (int)fh::colpass_smem<P>();
-  cudaError_t e = cudaFuncSetAttribute(fh::line_pass_warp6<P, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(fh::line_pass_warp6<P, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(fh::line_pass_warp6<P, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  cudaError_t e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 0>);
+  if (e == cudaSuccess) e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 1>);
+  if (e == cudaSuccess) e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 2>);
   return e;
 }
 
 template <typename T, int R1, int R2>
 cudaError_t set_col2_attrs() {
   constexpr int CT = col2_ct<T>();
-  const int sm = (int)fh::col2_smem<R1, R2, CT, T>();
-  cudaError_t e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 0, CT, col2_mb<T, 0, R1 * R2>(), T>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  cudaError_t e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 0, CT, col2_mb<T, 0, R1 * R2>(), T>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 1, CT, col2_mb<T, 1, R1 * R2>(), T>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 1, CT, col2_mb<T, 1, R1 * R2>(), T>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fh::line_pass_2s<R1, R2, 2, CT, col2_mb<T, 2, R1 * R2>(), T>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 2, CT, col2_mb<T, 2, R1 * R2>(), T>);
   return e;
 }
 
 template <int P1, int P2>
 cudaError_t set_plane_attrs() {
-  const int sm = (int)fh::plane_smem<P1, P2>();
-  cudaError_t e = cudaFuncSetAttribute(fh::plane_pass_warp6<P1, P2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  cudaError_t e = fh::allow_smem((const void*)fh::plane_pass_warp6<P1, P2, true>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fh::plane_pass_warp6<P1, P2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    e = fh::allow_smem((const void*)fh::plane_pass_warp6<P1, P2, false>);
   return e;
 }
 
@@ -710,12 +728,11 @@ cudaError_t set_plane_attrs_of(int code) {
 
 template <typename T, int R1, int R2>
 cudaError_t set_row2_attrs() {
-  const int sm = (int)fh::row2_smem<T, R1, R2>();
-  cudaError_t e = cudaFuncSetAttribute(fh::row_pass_2s<T, R1, R2, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  cudaError_t e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, true, false>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fh::row_pass_2s<T, R1, R2, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, false, false>);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fh::row_pass_2s<T, R1, R2, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, false, true>);
   return e;
 }
 
@@ -739,11 +756,11 @@ fh_status set_smem_attrs_nv(fh_solver* s, int prec) {
     fh::set_error("contiguous axis too long for the point-by-point stiffness in this precision (shared memory)");
     return FH_ERR_UNSUPPORTED;
   }
+  if (s->rowg_rb[prec] > 0) CK(fh::gen_row_prepare(T(0), NV));
   if (s->row_smem_gen[prec] <= kMaxSmem) {   // the block row pass (also taken by point-by-point stiffness)
-    const int rg = (int)s->row_smem_gen[prec];
-    CK(cudaFuncSetAttribute(fh::row_pass<T, NV, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, rg));
-    CK(cudaFuncSetAttribute(fh::row_pass<T, NV, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, rg));
-    CK(cudaFuncSetAttribute(fh::row_pass<T, NV, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, rg));
+    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, true>));
+    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, false>));
+    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, false, true>));
   }
   if (s->row_warp[prec] != 0) {
     if constexpr (sizeof(T) == 4) {
@@ -764,7 +781,10 @@ fh_status set_smem_attrs_nv(fh_solver* s, int prec) {
       case 128: CK((set_col2_attrs<T, 8, 16>())); continue;
       default: break;
     }
-    if (col_gen(s, prec, a)) continue;   // sets its own attributes
+    if (col_gen(s, prec, a)) {
+      CK(fh::gen_col_prepare(T(0), NV, s->g.dims[a]));
+      continue;
+    }
     if constexpr (sizeof(T) == 4) {
       switch (col_warp_p(s, prec, a)) {
         case 1: CK((set_col_attrs<1>())); continue;
@@ -781,9 +801,9 @@ fh_status set_smem_attrs_nv(fh_solver* s, int prec) {
     return FH_ERR_UNSUPPORTED;
   }
   if (lm > 0) {
-    CK(cudaFuncSetAttribute(fh::line_pass<T, NV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lm));
-    CK(cudaFuncSetAttribute(fh::line_pass<T, NV, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lm));
-    CK(cudaFuncSetAttribute(fh::line_pass<T, NV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lm));
+    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 0>));
+    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 1>));
+    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 2>));
   }
   return FH_OK;
 }
@@ -1093,7 +1113,7 @@ fh_status cluster_fits_nv(fh_solver* s, bool* ok) {
   if (lay.total + 1024 > kMaxSmem) return FH_OK;
   s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0] = gs;
   const void* kern = fh::cluster_kernel(T(0), NV, CS, POW2);
-  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.total));
+  CK(fh::allow_smem(kern));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(CS);
@@ -2405,7 +2425,7 @@ fh_status launch_queue(fh_solver* const* solvers, const std::vector<int>& member
   std::stable_sort(tasks.begin(), tasks.end(),
                    [](const fh::ClusterTask& a, const fh::ClusterTask& b) { return a.g.m > b.g.m; });
   const void* kern = fh::cluster_kernel(T(0), NV, CS, POW2);
-  CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  CK(fh::allow_smem(kern));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = cluster_config<T, NV, CS, POW2>(smem, 1, stream, attr);
