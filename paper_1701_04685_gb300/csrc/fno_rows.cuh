@@ -120,6 +120,21 @@ __device__ __forceinline__ void outer84(float (&acc)[8][4], const float4 a0, con
   }
 }
 
+// e^2 to the float pair (hi, lo) of at most 32 squares (TwoSum / TwoProduct: an FP64
+// multiply-add per element is a large part of the last layer's time), or in FP64 where
+// the square or its rounding error leaves FP32's range
+__device__ __forceinline__ void add_square(float e, float& hi, float& lo, double& sum) {
+  const float m = fabsf(e);
+  if (m < 0x1p61f && (m >= 0x1p-51f || m == 0.f)) {
+    const float pr = e * e, er = fmaf(e, e, -pr);
+    const float hs = hi + pr, bp = hs - hi;
+    lo += ((hi - (hs - bp)) + (pr - bp)) + er;
+    hi = hs;
+  } else {
+    sum += (double)e * e;
+  }
+}
+
 template <int EPI>
 __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
   extern __shared__ __align__(16) float smf[];
@@ -148,8 +163,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
       const int c = i / a.QP, q = i - c * a.QP;
       sQ[i] = q < a.cout ? a.Q[q * a.W + c] : 0.f;
     }
-  // the block sum of squared errors as a float pair (TwoSum / TwoProduct)
-  float ehi = 0.f, elo = 0.f;
+  double esum = 0.0;   // this thread's squared errors
   const int ntiles = (a.nrows + a.rpb - 1) / a.rpb;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int row0 = tile * a.rpb;
@@ -286,6 +300,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
           outer84(s, *reinterpret_cast<const float4*>(w), *reinterpret_cast<const float4*>(w + 4),
                   *reinterpret_cast<const float4*>(v));
         const size_t base = (size_t)b2 * a.cout * a.N3 + (size_t)(row2 - b2 * a.N2) * a.N + z2;
+        float ehi = 0.f, elo = 0.f;   // the task's squared errors as a float pair
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const int q = 8 * qg + i;
@@ -302,21 +317,17 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
           for (int j = 0; j < 4; ++j) {
             const float e = s[i][j] - tq[j];
             g[j] = 2.f * e * a.inv_count;
-            if (j < zn2) {
-              const float pr = e * e, er = fmaf(e, e, -pr);
-              const float hs = ehi + pr, bp = hs - ehi;
-              elo += ((ehi - (hs - bp)) + (pr - bp)) + er;
-              ehi = hs;
-            }
+            if (j < zn2) add_square(e, ehi, elo, esum);
           }
           store4(a.gy + p, make_float4(g[0], g[1], g[2], g[3]), zn2, a.vec);
         }
+        esum += (double)ehi + (double)elo;
       }
     }
   }
   if (a.Q && a.target) {
     __shared__ double red[kRowThreads / 32];
-    double v = (double)ehi + (double)elo;
+    double v = esum;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if ((tid & 31) == 0) red[tid >> 5] = v;
     __syncthreads();
