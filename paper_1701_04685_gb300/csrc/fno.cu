@@ -501,11 +501,24 @@ void flat_to_device(const fh_fno* f, const float* flat, std::vector<float>& dev)
 // A parameter-shaped device vector in the public order: the complex weights are
 // taken apart on the device (an HBM pass, 0.1 ms for 57 M parameters) and the copy
 // goes straight to the caller's buffer, where a host loop over a second copy took
-// five times as long as the copy itself.
+// five times as long as the copy itself.  Where the device has no room for the second
+// vector the host takes them apart.
 fh_status copy_out(const fh_fno* fc, const float* src, float* flat) {
   fh_fno* f = const_cast<fh_fno*>(fc);
   std::lock_guard<std::mutex> lock(f->flat_mutex);   // read-outs from several threads share the buffer
-  if (!f->flat) FCK(cudaMalloc(&f->flat, f->nparam * 4));
+  if (!f->flat && cudaMalloc(&f->flat, f->nparam * 4) != cudaSuccess) {
+    cudaGetLastError();
+    f->flat = nullptr;
+    FCK(cudaMemcpyAsync(flat, src, f->nparam * 4, cudaMemcpyDeviceToHost, f->stream));
+    FCK(cudaStreamSynchronize(f->stream));
+    const long long nR = (f->off_Q - f->off_R) / 2;
+    const std::vector<float> R(flat + f->off_R, flat + f->off_Q);
+    for (long long i = 0; i < nR; ++i) {
+      flat[f->off_R + i] = R[2 * i];
+      flat[f->off_R + nR + i] = R[2 * i + 1];
+    }
+    return FH_OK;
+  }
   k_to_flat<<<grid_for(f->nparam), kT, 0, f->stream>>>(f->nparam, f->off_R, (f->off_Q - f->off_R) / 2, src, f->flat);
   FCK(cudaGetLastError());
   FCK(cudaMemcpyAsync(flat, f->flat, f->nparam * 4, cudaMemcpyDeviceToHost, f->stream));
