@@ -34,6 +34,7 @@
 #include "internal.hpp"
 #include "fno_rows.cuh"
 #include "fno_spec.cuh"
+#include "fno_out.hpp"
 #include "fno_tc.cuh"
 #include "smem.hpp"
 
@@ -119,6 +120,7 @@ struct fh_fno {
   float* gb = nullptr;      // [B][W][N3]
   double* part = nullptr;
   int nparts = 0;
+  int device = 0;
   int sms = 1;
   std::map<std::pair<int, size_t>, int> resident;   // see resident_rows
   // hidden layers on the tensor cores (fno_tc.cuh) where they apply; tc_err is set by
@@ -432,9 +434,8 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
   if ((e = cudaMalloc(&f->gy, (size_t)max_batch * cout * d.N3 * 4)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc(&f->ga, act * 4)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc(&f->gb, act * 4)) != cudaSuccess) return fail(e);
-  int dev = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return fail(e);
-  if ((e = cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return fail(e);
+  if ((e = cudaGetDevice(&f->device)) != cudaSuccess) return fail(e);
+  if ((e = cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, f->device)) != cudaSuccess) return fail(e);
   if ((e = prepare_kernels()) != cudaSuccess) return fail(e);
   f->nparts = 8 * f->sms;   // at least the resident blocks of a row kernel
   if ((e = cudaMalloc(&f->part, f->nparts * sizeof(double))) != cudaSuccess) return fail(e);
@@ -577,9 +578,9 @@ fh_status fh_fno_zero_grad(fh_fno* f) {
 fh_status fh_fno_forward(fh_fno* f, int batch, const float* x, float* y) {
   if (!f || !x || !y) { fh::set_error("null argument"); return FH_ERR_ARG; }
   if (batch < 1 || batch > f->max_batch) { fh::set_error("batch out of range"); return FH_ERR_ARG; }
-  // the last kernel writes a device output directly (anything else goes through a copy)
   cudaPointerAttributes attr{};
-  const bool direct = cudaPointerGetAttributes(&attr, y) == cudaSuccess && attr.type == cudaMemoryTypeDevice;
+  const bool known = cudaPointerGetAttributes(&attr, y) == cudaSuccess;
+  const bool direct = fh::writes_directly(known && attr.type == cudaMemoryTypeDevice, attr.device, f->device);
   cudaGetLastError();   // a host pointer may leave an error behind on some drivers
   fh_status rc = forward_all(f, batch, x, direct ? y : f->y, nullptr, nullptr);
   if (rc != FH_OK) return rc;
