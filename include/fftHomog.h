@@ -423,9 +423,9 @@ const char* fh_last_error(void);
  * normal build. */
 /* 1 in the checked build, else 0. */
 int fh_checked_build(void);
-/* Checked build: launches a one-thread kernel that tests one index inside and
- * one outside a declared extent (inside its buffer either way) and returns
- * FH_ERR_INTERNAL naming the self test when the check caught the second.
+/* Checked build: launches a one-thread kernel of each compiled unit that tests one
+ * index inside and one outside a declared extent (inside its buffer either way) and
+ * returns FH_ERR_INTERNAL naming the self test when a check caught the second.
  * Normal build: FH_ERR_UNSUPPORTED, nothing launched. */
 fh_status fh_check_selftest(void);
 /* Checked build: the nth pass along an axis that the library would launch from

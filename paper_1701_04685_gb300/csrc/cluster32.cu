@@ -13,18 +13,6 @@ static const void* variant(int cs, bool pow2) {
 
 const void* cluster_kernel(float, int nv, int cs, bool pow2) { return nv == 3 ? variant<3>(cs, pow2) : variant<6>(cs, pow2); }
 
-cudaError_t cluster_take_check32(CheckRecord* rec) {
-  *rec = CheckRecord{};
-#ifdef FH_CHECKED
-  cudaError_t e = cudaMemcpyFromSymbol(rec, g_check, sizeof(*rec));
-  if (e == cudaSuccess && rec->count != 0ull) {
-    const CheckRecord zero{};
-    e = cudaMemcpyToSymbol(g_check, &zero, sizeof(zero));
-  }
-  return e;
-#else
-  return cudaSuccess;
-#endif
-}
+CheckUnit check_unit_cluster32() { return {check_take, check_selftest}; }
 
 }  // namespace fh

@@ -14,8 +14,4 @@ namespace fh {
 const void* cluster_kernel(double, int nv, int cs, bool pow2);
 const void* cluster_kernel(float, int nv, int cs, bool pow2);
 
-// checked build: the units' violation records (cleared when taken)
-cudaError_t cluster_take_check64(CheckRecord* rec);
-cudaError_t cluster_take_check32(CheckRecord* rec);
-
 }  // namespace fh

@@ -35,8 +35,4 @@ cudaError_t gen_row(bool first, bool kinv, const GridInfo& g, const float2* tw, 
                     const uint8_t* phase, const float* dC, Control* ctl, LoadState* st, double* partials, double* hist,
                     int nload, int rb, float* Wout, const float* Yaux, const float* Cfld, cudaStream_t stream);
 
-// checked build: the units' violation records (cleared when taken)
-cudaError_t gen_take_check64(CheckRecord* rec);
-cudaError_t gen_take_check32(CheckRecord* rec);
-
 }  // namespace fh

@@ -29,18 +29,6 @@ cudaError_t gen_row(bool first, bool kinv, const GridInfo& g, const float2* tw, 
                                        Cfld, stream);
 }
 
-cudaError_t gen_take_check32(CheckRecord* rec) {
-  *rec = CheckRecord{};
-#ifdef FH_CHECKED
-  cudaError_t e = cudaMemcpyFromSymbol(rec, g_check, sizeof(*rec));
-  if (e == cudaSuccess && rec->count != 0ull) {
-    const CheckRecord zero{};
-    e = cudaMemcpyToSymbol(g_check, &zero, sizeof(zero));
-  }
-  return e;
-#else
-  return cudaSuccess;
-#endif
-}
+CheckUnit check_unit_gen32() { return {check_take, check_selftest}; }
 
 }  // namespace fh

@@ -64,9 +64,43 @@ static __device__ __noinline__ bool check_fail(int site, long long i, long long 
 #define FH_IN(site, i, n) \
   (((unsigned long long)(long long)(i) < (unsigned long long)(long long)(n)) || \
    ::fh::check_fail((site), (long long)(i), (long long)(n)))
+// one index inside and one outside a declared extent of 4 (the buffer holds
+// 64 entries, so even a failed check would stay inside it)
+static __global__ void check_selftest_kernel(int* buf) {
+  for (int i = 3; i <= 5; i += 2)
+    if (FH_IN(CK_SELFTEST, i, 4)) buf[i] = 1;
+}
+static inline cudaError_t check_selftest(int* buf) {
+  check_selftest_kernel<<<1, 1>>>(buf);
+  return cudaGetLastError();
+}
+// this unit's record, cleared when taken
+static inline cudaError_t check_take(CheckRecord* rec) {
+  cudaError_t e = cudaMemcpyFromSymbol(rec, g_check, sizeof(*rec));
+  if (e == cudaSuccess && rec->count != 0ull) {
+    const CheckRecord zero{};
+    e = cudaMemcpyToSymbol(g_check, &zero, sizeof(zero));
+  }
+  return e;
+}
 #else
 #define FH_IN(site, i, n) true
+static inline cudaError_t check_selftest(int*) { return cudaSuccess; }
+static inline cudaError_t check_take(CheckRecord* rec) {
+  *rec = CheckRecord{};
+  return cudaSuccess;
+}
 #endif
+
+// The units whose kernels carry checks, each with a record of its own.
+struct CheckUnit {
+  cudaError_t (*take)(CheckRecord*);
+  cudaError_t (*selftest)(int*);
+};
+CheckUnit check_unit_cluster64();
+CheckUnit check_unit_cluster32();
+CheckUnit check_unit_gen64();
+CheckUnit check_unit_gen32();
 
 struct GridInfo {
   int d, nv, ntri, nd;

@@ -1519,21 +1519,26 @@ const char* check_site_name(int site) {
   return (site > 0 && site < fh::CK_NSITES) ? names[site] : "?";
 }
 
+#ifdef FH_CHECKED
+std::vector<fh::CheckUnit> check_units() {
+  return {{fh::check_take, fh::check_selftest}, fh::check_unit_cluster64(), fh::check_unit_cluster32(), fh::check_unit_gen64(),
+          fh::check_unit_gen32()};
+}
+#endif
+
 // Checked build: after an entry point's work, the record of the first index
 // found outside its array turns the call's status into FH_ERR_INTERNAL (the
 // record is cleared).  Without FH_CHECKED the status passes through.
 fh_status checked(fh_status rc) {
 #ifdef FH_CHECKED
   CK(cudaDeviceSynchronize());
+  // every unit's record is taken, so that none is left for a later call; the first is named
   fh::CheckRecord rec{};
-  CK(cudaMemcpyFromSymbol(&rec, fh::g_check, sizeof(rec)));
-  if (rec.count != 0ull) {
-    const fh::CheckRecord zero{};
-    CK(cudaMemcpyToSymbol(fh::g_check, &zero, sizeof(zero)));
+  for (const fh::CheckUnit& u : check_units()) {
+    fh::CheckRecord r{};
+    CK(u.take(&r));
+    if (rec.count == 0ull) rec = r;
   }
-  // the units of the cluster kernel and of the general two-step passes keep records of their own
-  for (auto take : {fh::cluster_take_check64, fh::cluster_take_check32, fh::gen_take_check64, fh::gen_take_check32})
-    if (rec.count == 0ull) CK(take(&rec));
   if (rec.count != 0ull) {
     fh::set_error(std::string("index check failed (") + std::to_string(rec.count) + " accesses): " +
                   check_site_name(rec.site) + ", index " + std::to_string(rec.index) + " outside [0, " +
@@ -1543,15 +1548,6 @@ fh_status checked(fh_status rc) {
 #endif
   return rc;
 }
-
-#ifdef FH_CHECKED
-// one index inside and one outside a declared extent of 4 (the buffer holds
-// 64 entries, so even a failed check would stay inside it)
-__global__ void check_selftest_kernel(int* buf) {
-  for (int i = 3; i <= 5; i += 2)
-    if (FH_IN(fh::CK_SELFTEST, i, 4)) buf[i] = 1;
-}
-#endif
 
 }  // namespace
 
@@ -1582,8 +1578,9 @@ fh_status fh_check_selftest(void) {
   if (rc != FH_OK) return rc;
   int* buf = nullptr;
   CK(cudaMalloc(&buf, 64 * sizeof(int)));
-  check_selftest_kernel<<<1, 1>>>(buf);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  for (const fh::CheckUnit& u : check_units())
+    if (e == cudaSuccess) e = u.selftest(buf);
   rc = checked(FH_OK);
   cudaFree(buf);
   if (e != cudaSuccess) {
