@@ -21,9 +21,10 @@ LIB = os.path.join(OUT_DIR, "libffthomog.so")
 LIB_CHECKED = os.path.join(OUT_DIR, "libffthomog_checked.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-SOURCES = ["solver.cu", "cluster64.cu", "cluster32.cu", "genpass64.cu", "genpass32.cu", "lattice.cpp", "noalloc.cu", "fno.cu"]
+SOURCES = ["solver.cu", "cluster64.cu", "cluster32.cu", "clusterst64.cu", "clusterst32.cu", "genpass64.cu", "genpass32.cu",
+           "clusterplan.cpp", "lattice.cpp", "noalloc.cu", "fno.cu"]
 # the units whose kernels carry the index checks of the checked build
-CHECKED = ["solver.cu", "cluster64.cu", "cluster32.cu", "genpass64.cu", "genpass32.cu"]
+CHECKED = ["solver.cu", "cluster64.cu", "cluster32.cu", "clusterst64.cu", "clusterst32.cu", "genpass64.cu", "genpass32.cu"]
 HEADERS = ["internal.hpp", "kernels.cuh", "fft.cuh", "cluster.cuh", "warprow.cuh", "linewarp.cuh", "colpass2.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -24,29 +24,10 @@
 // is addressed by byte offsets so that the accesses stay shared-memory instructions.
 #pragma once
 
+#include "bigsplit.hpp"
 #include "gendft.cuh"
-#include "gensplit.hpp"
 
 namespace fh {
-
-// the split of an axis for warp_two_step: R1 = 0 none, R1 = 1 a line per lane
-struct LineSplit {
-  int R1, R2;
-  unsigned m1, m2;   // lane / R = umulhi(lane, m)
-};
-inline LineSplit line_split(int N) {
-  LineSplit s{};
-  if (N >= 2 && N <= 16) {
-    s.R1 = 1;
-    s.R2 = N;
-  } else if (!gen_split(N, false, &s.R1, &s.R2)) {   // radices to 16: 16 warps' registers hold them
-    s.R1 = s.R2 = 0;
-    return s;
-  }
-  s.m1 = s.R1 > 1 ? (unsigned)((0x100000000ull + s.R1 - 1) / s.R1) : 0u;
-  s.m2 = (unsigned)((0x100000000ull + s.R2 - 1) / s.R2);
-  return s;
-}
 
 // f(RadixC<R>) for a run-time R from 2 to 16
 template <typename F>
@@ -186,7 +167,9 @@ __device__ __noinline__ unsigned fft_lines_big(unsigned a, unsigned b, int nline
       FH_BIG_STAGE(9) FH_BIG_STAGE(10) FH_BIG_STAGE(11) FH_BIG_STAGE(12) FH_BIG_STAGE(13) FH_BIG_STAGE(14)
       FH_BIG_STAGE(15) FH_BIG_STAGE(16)
 #undef FH_BIG_STAGE
-      default: stockham_stage_prime<DIR, T, PADSH>(in, out, nlines, ls, L, Ns, r, tw, tid, nthr); break;
+      default:   // reached in FP64 only (cluster_choice); without it ptxas spills more of the FP32 kernel
+        stockham_stage_prime<DIR, T, PADSH>(in, out, nlines, ls, L, Ns, r, tw, tid, nthr);
+        break;
     }
     team_sync(nthr);
     const unsigned t = a;

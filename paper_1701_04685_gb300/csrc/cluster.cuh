@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 
 #include "bigfft.cuh"
+#include "clusterkern.hpp"
 #include "kernels.cuh"
 #include "warprow.cuh"
 
@@ -82,12 +83,15 @@ __host__ __device__ inline ClusterLayout cluster_layout(int N0, int L, int nv, i
 }
 
 // threads per CTA: 16 warps in FP32, 8 in FP64 (whose pipe they fill, and whose
-// larger line transforms need the registers)
-template <typename T> struct ClusterThreads { static constexpr int value = sizeof(T) == 4 ? 512 : 256; };
+// larger line transforms need the registers) and in the staged kernel, whose inlined
+// stages need them too
+template <typename T, int KIND> struct ClusterThreads {
+  static constexpr int value = sizeof(T) == 4 && KIND != kClusterStaged ? 512 : 256;
+};
 
 // The whole solve of load `load` by the cluster this CTA belongs to.  Ends
 // with a cluster barrier, after which the cluster may start another solve.
-template <typename T, int NV, int CS, bool POW2>
+template <typename T, int NV, int CS, int KIND>
 __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevPlan& plan0, const DevPlan& plan1,
                                                    const LineSplit& split0, const LineSplit& split1,
                                                    const cplx<T>* __restrict__ tw0g, const cplx<T>* __restrict__ tw1g,
@@ -95,6 +99,7 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
                                                    const T* __restrict__ dC, int nphase, const T* __restrict__ Gt,
                                                    Control* ctl, LoadState* st, double* __restrict__ hist, int g_smem,
                                                    int load) {
+  constexpr bool POW2 = KIND == kClusterPow2;
   constexpr int NTRI = NV * (NV + 1) / 2;
   extern __shared__ __align__(128) unsigned char sm[];
   cg::cluster_group cluster = cg::this_cluster();
@@ -164,12 +169,13 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
   const T scale = (T)g.inv_m;
   __syncthreads();
 
-  // line transform of buf (ping-pong with tmp): plans of radices 2, 4, 8 inline; other
-  // grids by single warps (FP32, where the length splits) or through fft_lines_big
+  // line transform of buf (ping-pong with tmp): inlined stages (powers of two and the
+  // staged kernel); in the general kernel by single warps (FP32, where the length splits)
+  // or through fft_lines_big
   auto lines = [&](auto dir, auto pad, cplx<T>* buf, cplx<T>* tmp, int n, int ls, const DevPlan& plan, const LineSplit& split,
                    const cplx<T>* tw, int t, int nthr) -> cplx<T>* {
     constexpr int DIR = decltype(dir)::value, PADSH = decltype(pad)::value;
-    if constexpr (!POW2 && sizeof(T) == 4) {
+    if constexpr (KIND == kClusterGeneral && sizeof(T) == 4) {
       if (split.R1 > 0) {
         const unsigned char* base = sm;
         warp_two_step<T>((unsigned)(reinterpret_cast<unsigned char*>(buf) - base), n, ls, PADSH ? PADSH : 31, DIR > 0, split,
@@ -177,8 +183,8 @@ __device__ __forceinline__ void cluster_solve_body(const GridInfo& g, const DevP
         return buf;
       }
     }
-    if constexpr (POW2) {
-      return fft_lines_pp<DIR, T, PADSH, true>(buf, tmp, n, ls, plan, tw, t, nthr);
+    if constexpr (KIND != kClusterGeneral) {
+      return fft_lines_pp<DIR, T, PADSH, POW2>(buf, tmp, n, ls, plan, tw, t, nthr);
     } else {
       const unsigned char* base = sm;
       const unsigned o = fft_lines_big<DIR, T, PADSH>((unsigned)(reinterpret_cast<unsigned char*>(buf) - base),
@@ -440,8 +446,8 @@ struct ClusterTask {
 // on as many clusters as fit.  Rank 0 of a cluster draws the next index with
 // one atomic and the other CTAs read it from rank 0's shared memory; clusters
 // never wait on one another.  The task is staged in shared memory.
-template <typename T, int NV, int CS, bool POW2>
-__global__ void __launch_bounds__(ClusterThreads<T>::value, 1)
+template <typename T, int NV, int CS, int KIND>
+__global__ void __launch_bounds__(ClusterThreads<T, KIND>::value, 1)
 cluster_solve_2d(const ClusterTask* __restrict__ tasks, int ntasks, unsigned int* next) {
   cg::cluster_group cluster = cg::this_cluster();
   __shared__ int s_task;
@@ -457,7 +463,7 @@ cluster_solve_2d(const ClusterTask* __restrict__ tasks, int ntasks, unsigned int
     }
     cluster.sync();   // every CTA holds the index (and the task) before rank 0 draws the next one
     if (task >= ntasks) return;
-    cluster_solve_body<T, NV, CS, POW2>(t.g, t.plan0, t.plan1, t.split0, t.split1, static_cast<const cplx<T>*>(t.tw0),
+    cluster_solve_body<T, NV, CS, KIND>(t.g, t.plan0, t.plan1, t.split0, t.split1, static_cast<const cplx<T>*>(t.tw0),
                                         static_cast<const cplx<T>*>(t.tw1), static_cast<T*>(t.E), t.phase,
                                         static_cast<const T*>(t.dC), t.nphase, static_cast<const T*>(t.Gt), t.ctl,
                                         t.st, t.hist, t.g_smem, t.load);

@@ -279,9 +279,13 @@ __device__ __forceinline__ void stockham_stage_prime(const cplx<T>* in, cplx<T>*
     const int j = jq * Ns + k;
     const cplx<T>* li = in + line * ls;
     cplx<T> acc = li[padi<PADSH>(j)];
+    const int d1 = k * stride, d2 = t_out * step;   // both exponents by additions: a remainder per term is half the loop
+    int e1 = 0, e2 = 0;
     for (int t = 1; t < R; ++t) {
-      int e = t * k * stride + ((t_out * t) % R) * step;
-      if (e >= L) e -= L;
+      e1 += d1;   // t k stride < L
+      e2 += d2;
+      if (e2 >= L) e2 -= L;
+      const int e = e1 + e2 >= L ? e1 + e2 - L : e1 + e2;
       cplx<T> w = tw[e];
       if (DIR > 0) w.y = -w.y;
       acc = cadd(acc, cmul(li[padi<PADSH>(j + t * nb)], w));

@@ -99,6 +99,8 @@ struct CheckUnit {
 };
 CheckUnit check_unit_cluster64();
 CheckUnit check_unit_cluster32();
+CheckUnit check_unit_clusterst64();
+CheckUnit check_unit_clusterst32();
 CheckUnit check_unit_gen64();
 CheckUnit check_unit_gen32();
 

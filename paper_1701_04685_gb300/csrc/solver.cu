@@ -95,9 +95,6 @@ int mandel_nv(int d) { return d == 2 ? 3 : 6; }
 
 struct Axis {
   int L = 1;
-  DevPlan plan{};        // radix schedule of the cluster kernel for powers of two (and the default)
-  DevPlan big{};         // its schedule for other grids (radices up to 16)
-  DevPlan tiny{};        // its FP64 schedule for few points a thread (radices up to 4)
   DevPlan planp[2]{};    // radix schedule of the passes per bulk precision (autotuned)
   double2* tw64 = nullptr;
   float2* tw32 = nullptr;
@@ -176,6 +173,7 @@ struct fh_solver {
   int lineW[2][3] = {};
   int ntiles[2][3] = {};
   size_t line_smem[2][3] = {};
+  fh::ClusterChoice cl_choice[2];         // kernel and radix schedules of the cluster path per precision (2-axis grids)
   std::vector<GraphEntry> graphs;
   cudaError_t launch_err = cudaSuccess;   // first error of a pass's launch not reported yet (launch_status)
   bool cl_gsmem[2][2] = {{true, true}, {true, true}};  // [fp64/fp32][cluster 8/16]: table slice in smem
@@ -1083,24 +1081,37 @@ fh_status run_bicgstab(fh_solver* s, int prec, int nload, int chunk, int max_ite
   return FH_OK;
 }
 
-// both axis plans use radices 2, 4, 8 only: the cluster kernel variant
-// without the other stages (fewer registers, 16 warps per CTA)
-bool pow2_plans(const fh_solver* s) {
-  for (int a = 0; a < 2; ++a)
-    for (int q = 0; q < s->ax[a].plan.np; ++q) {
-      const int r = s->ax[a].plan.r[q];
-      if (r != 2 && r != 4 && r != 8) return false;
-    }
-  return true;
+template <typename T>
+const fh::ClusterChoice& cluster_of(const fh_solver* s) { return s->cl_choice[sizeof(T) == 8 ? 0 : 1]; }
+
+DevPlan dev_plan(const fh::FftPlan& p) {
+  DevPlan d{};
+  d.L = p.L;
+  d.np = p.np;
+  std::copy(p.r, p.r + 24, d.r);
+  return d;
 }
 
-// threads per CTA of the cluster kernel
+// Launch configuration of the cluster kernel with `nclusters` clusters.
 template <typename T>
-constexpr int cluster_threads() { return fh::ClusterThreads<T>::value; }
+cudaLaunchConfig_t cluster_config(int kind, int CS, size_t smem, int nclusters, cudaStream_t stream, cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nclusters * CS);
+  cfg.blockDim = dim3(fh::cluster_kernel_threads(sizeof(T) == 4, kind));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CS;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
 
 // Cluster-resident path (2-axis grids): one cluster of CS CTAs per load case.
-template <typename T, int NV, int CS, bool POW2>
-fh_status cluster_fits_nv(fh_solver* s, bool* ok) {
+template <typename T, int CS>
+fh_status cluster_fits(fh_solver* s, bool* ok) {
   *ok = false;
   const GridInfo& g = s->g;
   if (g.nd != 2) return FH_OK;
@@ -1112,20 +1123,12 @@ fh_status cluster_fits_nv(fh_solver* s, bool* ok) {
   }
   if (lay.total + 1024 > kMaxSmem) return FH_OK;
   s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0] = gs;
-  const void* kern = fh::cluster_kernel(T(0), NV, CS, POW2);
+  const int kind = cluster_of<T>(s).kind;
+  const void* kern = fh::cluster_kernel(T(0), g.nv, CS, kind);
   CK(fh::allow_smem(kern));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CS);
-  cfg.blockDim = dim3(cluster_threads<T>());
-  cfg.dynamicSmemBytes = lay.total;
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  const cudaLaunchConfig_t cfg = cluster_config<T>(kind, CS, lay.total, 1, nullptr, attr);
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
     cudaGetLastError();
@@ -1135,33 +1138,14 @@ fh_status cluster_fits_nv(fh_solver* s, bool* ok) {
   return FH_OK;
 }
 
-template <typename T, int CS>
-fh_status cluster_fits(fh_solver* s, bool* ok) {
-  if (pow2_plans(s))
-    return s->g.nv == 3 ? cluster_fits_nv<T, 3, CS, true>(s, ok) : cluster_fits_nv<T, 6, CS, true>(s, ok);
-  return s->g.nv == 3 ? cluster_fits_nv<T, 3, CS, false>(s, ok) : cluster_fits_nv<T, 6, CS, false>(s, ok);
-}
-
 // Task of the cluster kernel for load l of solver s.
 template <typename T, int CS>
 fh::ClusterTask cluster_task(const fh_solver* s, int l) {
   const bool gs = s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0];
   fh::ClusterTask t{};
   t.g = s->g;
-  const bool pow2 = pow2_plans(s);
-  t.plan0 = pow2 ? s->ax[0].plan : s->ax[0].big;
-  t.plan1 = pow2 ? s->ax[1].plan : s->ax[1].big;
-  if (sizeof(T) == 8) {
-    // An FP64 warp instruction takes its quarter of the SM 64 cycles whatever its lanes
-    // do, so a small grid's stage lasts one thread's butterfly: radix 4 where there are
-    // at most two points a thread (32^2: 19.6 -> 17.4 us an iteration; with 3.4 points,
-    // 96^2, 48.7 -> 52.1).  Counted for clusters of 8 in either size, so that a solve's
-    // bits do not depend on the cluster that a batch or the tuner picks (64^2 on 16
-    // CTAs, 29.0 against 24.4, stays with the large radices for that).
-    const fh::ClusterLayout lay = fh::cluster_layout<T>(s->g.dims[0], s->g.L, s->g.nv, 8, true);
-    if (s->g.nv * lay.cols_max * s->g.dims[0] <= 2 * cluster_threads<T>()) t.plan0 = s->ax[0].tiny;
-    if (lay.npair_max * s->g.L <= 2 * cluster_threads<T>()) t.plan1 = s->ax[1].tiny;
-  }
+  t.plan0 = dev_plan(cluster_of<T>(s).plan0);
+  t.plan1 = dev_plan(cluster_of<T>(s).plan1);
   t.split0 = fh::line_split(s->g.dims[0]);
   t.split1 = fh::line_split(s->g.L);
   t.tw0 = twp<T>(s->ax[0]);
@@ -1179,26 +1163,9 @@ fh::ClusterTask cluster_task(const fh_solver* s, int l) {
   return t;
 }
 
-// Launch configuration of the cluster kernel with `nclusters` clusters.
-template <typename T, int NV, int CS, bool POW2>
-cudaLaunchConfig_t cluster_config(size_t smem, int nclusters, cudaStream_t stream, cudaLaunchAttribute* attr) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nclusters * CS);
-  cfg.blockDim = dim3(cluster_threads<T>());
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cfg;
-}
-
 // A single solve: one cluster per load, each taking its own load's task.
-template <typename T, int NV, int CS, bool POW2>
-fh_status launch_cluster_nv(fh_solver* s, int nload) {
+template <typename T, int CS>
+fh_status launch_cluster(fh_solver* s, int nload) {
   const GridInfo& g = s->g;
   const bool gs = s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0];
   const fh::ClusterLayout lay = fh::cluster_layout<T>(g.dims[0], g.L, g.nv, CS, gs);
@@ -1206,19 +1173,13 @@ fh_status launch_cluster_nv(fh_solver* s, int nload) {
   CK(cudaMemcpyAsync(s->qtasks, s->h_tasks, nload * sizeof(fh::ClusterTask), cudaMemcpyHostToDevice, s->work));
   CK(cudaMemsetAsync(s->qnext, 0, sizeof(unsigned int), s->work));
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = cluster_config<T, NV, CS, POW2>(lay.total, nload, s->work, attr);
+  const int kind = cluster_of<T>(s).kind;
+  cudaLaunchConfig_t cfg = cluster_config<T>(kind, CS, lay.total, nload, s->work, attr);
   const fh::ClusterTask* tp = s->qtasks;
   unsigned int* np = s->qnext;
   void* args[] = {&tp, &nload, &np};
-  CK(cudaLaunchKernelExC(&cfg, fh::cluster_kernel(T(0), NV, CS, POW2), args));
+  CK(cudaLaunchKernelExC(&cfg, fh::cluster_kernel(T(0), g.nv, CS, kind), args));
   return FH_OK;
-}
-
-template <typename T, int CS>
-fh_status launch_cluster(fh_solver* s, int nload) {
-  if (pow2_plans(s))
-    return s->g.nv == 3 ? launch_cluster_nv<T, 3, CS, true>(s, nload) : launch_cluster_nv<T, 6, CS, true>(s, nload);
-  return s->g.nv == 3 ? launch_cluster_nv<T, 3, CS, false>(s, nload) : launch_cluster_nv<T, 6, CS, false>(s, nload);
 }
 
 // Pick path and cluster size; returns 1 (passes) or 2 (cluster) in *path.
@@ -1521,8 +1482,8 @@ const char* check_site_name(int site) {
 
 #ifdef FH_CHECKED
 std::vector<fh::CheckUnit> check_units() {
-  return {{fh::check_take, fh::check_selftest}, fh::check_unit_cluster64(), fh::check_unit_cluster32(), fh::check_unit_gen64(),
-          fh::check_unit_gen32()};
+  return {{fh::check_take, fh::check_selftest}, fh::check_unit_cluster64(), fh::check_unit_cluster32(),
+          fh::check_unit_clusterst64(), fh::check_unit_clusterst32(), fh::check_unit_gen64(), fh::check_unit_gen32()};
 }
 #endif
 
@@ -1701,18 +1662,15 @@ fh_status fh_solver_create(const fh_pattern* p, const fh_generator* gen, int nlo
     fh::FftPlan fp;
     if (!fh::make_plan(g.dims[k], &fp)) { delete s; fh::set_error("SNF axis length needs more than 24 radix stages"); return FH_ERR_UNSUPPORTED; }
     s->ax[k].L = fp.L;
-    s->ax[k].plan.L = fp.L;
-    s->ax[k].plan.np = fp.np;
-    for (int q = 0; q < 24; ++q) s->ax[k].plan.r[q] = fp.r[q];
-    s->ax[k].planp[0] = s->ax[k].planp[1] = s->ax[k].plan;
-    for (int q = 0; q < 2; ++q) {
-      if (!fh::make_big_plan(g.dims[k], q ? 4 : 16, &fp)) { delete s; fh::set_error("SNF axis length needs more than 24 radix stages"); return FH_ERR_UNSUPPORTED; }
-      fh::DevPlan& p = q ? s->ax[k].tiny : s->ax[k].big;
-      p.L = fp.L;
-      p.np = fp.np;
-      std::copy(fp.r, fp.r + 24, p.r);
-    }
+    s->ax[k].planp[0] = s->ax[k].planp[1] = dev_plan(fp);
   }
+  if (g.nd == 2)
+    for (int prec = 0; prec < 2; ++prec)
+      if (!fh::cluster_choice(g.dims[0], g.dims[1], g.nv, prec == FH_PREC_FP32, &s->cl_choice[prec])) {
+        delete s;
+        fh::set_error("SNF axis length needs more than 24 radix stages");
+        return FH_ERR_UNSUPPORTED;
+      }
   choose_shapes(s, FH_PREC_FP64);
   choose_shapes(s, FH_PREC_FP32);
   save_default_shapes(s);
@@ -2404,16 +2362,16 @@ fh_status finish_deferred(fh_solver* s, int nload, PhaseOut* out) {
 // ordered largest pattern first, and as many clusters as fit stay resident.
 struct QueueGroup {
   int prec, nv, cs;
-  bool pow2;
+  int kind;                   // ClusterKind
   std::vector<int> members;   // indices into the batch
 };
 
-template <typename T, int NV, int CS, bool POW2>
-fh_status launch_queue(fh_solver* const* solvers, const std::vector<int>& members, const int* nload,
-                       cudaStream_t stream, fh::ClusterTask** dtasks, unsigned int** dnext) {
+template <typename T, int CS>
+fh_status launch_queue(const QueueGroup& q, fh_solver* const* solvers, const int* nload, cudaStream_t stream,
+                       fh::ClusterTask** dtasks, unsigned int** dnext) {
   std::vector<fh::ClusterTask> tasks;
   size_t smem = 0;
-  for (int i : members) {
+  for (int i : q.members) {
     fh_solver* s = solvers[i];
     const bool gs = s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0];
     smem = std::max(smem, fh::cluster_layout<T>(s->g.dims[0], s->g.L, s->g.nv, CS, gs).total);
@@ -2421,11 +2379,11 @@ fh_status launch_queue(fh_solver* const* solvers, const std::vector<int>& member
   }
   std::stable_sort(tasks.begin(), tasks.end(),
                    [](const fh::ClusterTask& a, const fh::ClusterTask& b) { return a.g.m > b.g.m; });
-  const void* kern = fh::cluster_kernel(T(0), NV, CS, POW2);
+  const void* kern = fh::cluster_kernel(T(0), q.nv, CS, q.kind);
   CK(fh::allow_smem(kern));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = cluster_config<T, NV, CS, POW2>(smem, 1, stream, attr);
+  cudaLaunchConfig_t cfg = cluster_config<T>(q.kind, CS, smem, 1, stream, attr);
   int resident = 0;
   CK(cudaOccupancyMaxActiveClusters(&resident, kern, &cfg));
   const int nclusters = std::max(1, std::min<int>((int)tasks.size(), resident));
@@ -2442,14 +2400,10 @@ fh_status launch_queue(fh_solver* const* solvers, const std::vector<int>& member
   return FH_OK;
 }
 
-template <typename T, int NV>
-fh_status launch_queue_nv(const QueueGroup& q, fh_solver* const* solvers, const int* nload, cudaStream_t stream,
+template <typename T>
+fh_status launch_queue_cs(const QueueGroup& q, fh_solver* const* solvers, const int* nload, cudaStream_t stream,
                           fh::ClusterTask** dt, unsigned int** dn) {
-  if (q.cs == 16)
-    return q.pow2 ? launch_queue<T, NV, 16, true>(solvers, q.members, nload, stream, dt, dn)
-                  : launch_queue<T, NV, 16, false>(solvers, q.members, nload, stream, dt, dn);
-  return q.pow2 ? launch_queue<T, NV, 8, true>(solvers, q.members, nload, stream, dt, dn)
-                : launch_queue<T, NV, 8, false>(solvers, q.members, nload, stream, dt, dn);
+  return q.cs == 16 ? launch_queue<T, 16>(q, solvers, nload, stream, dt, dn) : launch_queue<T, 8>(q, solvers, nload, stream, dt, dn);
 }
 
 // Queue the deferred cluster solves of a phase: group them, let one stream
@@ -2461,9 +2415,9 @@ fh_status run_queued(fh_solver* const* solvers, const int* nload, const std::vec
   if (deferred.empty()) return FH_OK;
   std::vector<QueueGroup> groups;
   for (int i : deferred) {
-    const QueueGroup key{prec, solvers[i]->g.nv, out[i].cs, pow2_plans(solvers[i]), {}};
+    const QueueGroup key{prec, solvers[i]->g.nv, out[i].cs, solvers[i]->cl_choice[prec == FH_PREC_FP64 ? 0 : 1].kind, {}};
     auto it = std::find_if(groups.begin(), groups.end(), [&](const QueueGroup& q) {
-      return q.nv == key.nv && q.cs == key.cs && q.pow2 == key.pow2;
+      return q.nv == key.nv && q.cs == key.cs && q.kind == key.kind;
     });
     if (it == groups.end()) { groups.push_back(key); it = groups.end() - 1; }
     it->members.push_back(i);
@@ -2497,12 +2451,8 @@ fh_status run_queued(fh_solver* const* solvers, const int* nload, const std::vec
     fh::ClusterTask* dt = nullptr;
     unsigned int* dn = nullptr;
     fh_status rc;
-    if (prec == FH_PREC_FP64)
-      rc = q.nv == 3 ? launch_queue_nv<double, 3>(q, solvers, nload, qs, &dt, &dn)
-                     : launch_queue_nv<double, 6>(q, solvers, nload, qs, &dt, &dn);
-    else
-      rc = q.nv == 3 ? launch_queue_nv<float, 3>(q, solvers, nload, qs, &dt, &dn)
-                     : launch_queue_nv<float, 6>(q, solvers, nload, qs, &dt, &dn);
+    rc = prec == FH_PREC_FP64 ? launch_queue_cs<double>(q, solvers, nload, qs, &dt, &dn)
+                              : launch_queue_cs<float>(q, solvers, nload, qs, &dt, &dn);
     if (dt) bufs.push_back(dt);
     if (dn) bufs.push_back(dn);
     if (rc != FH_OK) { cleanup(); return rc; }
