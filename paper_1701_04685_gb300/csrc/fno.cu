@@ -122,7 +122,7 @@ struct fh_fno {
   int nparts = 0;
   int device = 0;
   int sms = 1;
-  std::map<std::pair<int, size_t>, int> resident;   // see resident_rows
+  std::map<std::pair<const void*, size_t>, int> prepared;   // see prepare
   // hidden layers on the tensor cores (fno_tc.cuh) where they apply; tc_err is set by
   // a kernel whose bounded wait gave up
   bool tensor_cores = true;
@@ -160,16 +160,18 @@ fhrow::RowArgs row_args(const fh_fno* f, int B, int cin, const float* in, const 
   return a;
 }
 
-// resident blocks per SM of a row kernel, asked for once per kernel and size
-template <int EPI>
-cudaError_t resident_rows(fh_fno* f, size_t sm, int* res) {
-  auto it = f->resident.find({EPI, sm});
-  if (it == f->resident.end()) {
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(res, fhrow::k_rows<EPI>, fhrow::kRowThreads, sm);
+// A kernel's shared-memory limit, once per kernel and size; *resident (where asked for)
+// its resident blocks per SM.
+cudaError_t prepare(fh_fno* f, const void* kernel, int threads, size_t sm, int* resident = nullptr) {
+  auto it = f->prepared.find({kernel, sm});
+  if (it == f->prepared.end()) {
+    cudaError_t e = fh::allow_smem(kernel, sm);
+    int res = 1;
+    if (e == cudaSuccess && resident) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&res, kernel, threads, sm);
     if (e != cudaSuccess) return e;
-    it = f->resident.insert({{EPI, sm}, *res}).first;
+    it = f->prepared.insert({{kernel, sm}, res}).first;
   }
-  *res = it->second;
+  if (resident) *resident = it->second;
   return cudaSuccess;
 }
 
@@ -194,7 +196,7 @@ fh_status launch_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
   const size_t sm = fhrow::row_smem_floats(a) * 4;
   const int ntiles = (a.nrows + a.rpb - 1) / a.rpb;
   int res = 1;
-  FCK(resident_rows<EPI>(f, sm, &res));
+  FCK(prepare(f, (const void*)fhrow::k_rows<EPI>, fhrow::kRowThreads, sm, &res));
   const int grid = std::min(ntiles, std::max(1, res) * f->sms);
   if (blocks) *blocks = grid;
   fhrow::k_rows<EPI><<<grid, fhrow::kRowThreads, sm, f->stream>>>(a);
@@ -226,6 +228,7 @@ fh_status hidden_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
   t.in = a.in; t.W = reinterpret_cast<const __nv_bfloat16*>(a.A); t.trans = a.a_trans; t.bias = a.bias;
   t.Iy = a.Iy; t.T = a.T; t.u_in = a.u_in; t.u_out = a.u_out; t.out = a.out; t.Yz = a.Yz; t.err = f->tc_err;
   const size_t sm = fhtc::tc_layout(d.N, t.Kp).total;
+  FCK(prepare(f, (const void*)fhtc::k_rows_tc<EPI>, fhtc::kTcThreads, sm));
   // two CTAs share an SM where their shared memory allows (tensor memory has 512 columns)
   const int res = 2 * (sm + 2048) <= 228 * 1024 && 2 * t.ncols <= 512 ? 2 : 1;
   fhtc::k_rows_tc<EPI><<<std::min(t.ntiles, res * f->sms), fhtc::kTcThreads, sm, f->stream>>>(t);
@@ -264,6 +267,7 @@ fh_status dft_y(fh_fno* f, int B) {
   const size_t per = (size_t)2 * (d.N / 2 + 1) * d.W * sizeof(float2);
   const int kb = y_group(d, (d.m / 4 + 1) * d.W, per);
   const size_t sm = d.N * sizeof(float2) + kb * per;
+  FCK(prepare(f, (const void*)fhspec::k_dft_y, fhspec::kSpecThreads, sm));
   fhspec::k_dft_y<<<B * d.N * ((d.m + kb - 1) / kb), fhspec::kSpecThreads, sm, f->stream>>>(
       d.N, d.m, d.W, kb, spec_div(d), f->Yz, f->Yy, f->tw);
   FCK(cudaGetLastError());
@@ -275,6 +279,7 @@ fh_status idft_y(fh_fno* f, int B, float scale, int wz) {
   const size_t per = (size_t)2 * d.m * d.W * sizeof(float2);
   const int kb = y_group(d, (d.N / 8 + 1) * d.W, per);
   const size_t sm = d.N * sizeof(float2) + kb * per;
+  FCK(prepare(f, (const void*)fhspec::k_idft_y, fhspec::kSpecThreads, sm));
   fhspec::k_idft_y<<<B * d.N * ((d.m + kb - 1) / kb), fhspec::kSpecThreads, sm, f->stream>>>(
       d.N, d.m, d.W, kb, spec_div(d), f->Yy, f->Yz, f->tw, scale, wz);
   FCK(cudaGetLastError());
@@ -294,6 +299,7 @@ fh_status mix_x(fh_fno* f, int B, int l, float scale) {
   const size_t base = d.N * sizeof(float2) + bc * per_b;
   const int rs = (int)std::max<size_t>(1, std::min<size_t>(m2, base < half ? (half - base) / per_r : 1));
   const size_t sm = base + rs * per_r;
+  FCK(prepare(f, (const void*)fhspec::k_mix_x<BACK>, fhspec::kSpecThreads, sm));
   fhspec::k_mix_x<BACK><<<m2 * d.m, fhspec::kSpecThreads, sm, f->stream>>>(
       d.N, d.m, d.W, B, bc, rs, spec_div(d), reinterpret_cast<const __nv_bfloat162*>(f->Rbf) + (size_t)l * d.NM * d.W * d.W, f->Yy,
       f->vh + (size_t)l * B * d.NM * d.W,
@@ -353,23 +359,13 @@ fh_status weight_grad(fh_fno* f, int B, int cin, int cout, const float* g, const
   return FH_OK;
 }
 
-// shared-memory limits of the kernels, once per network
-template <int EPI>
-cudaError_t prepare_rows() {
-  cudaError_t e = fh::allow_smem((const void*)fhrow::k_rows<EPI>);
-  if (e == cudaSuccess) e = fh::allow_smem((const void*)fhtc::k_rows_tc<EPI>);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fhtc::k_rows_tc<EPI>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  return e;
-}
-cudaError_t prepare_kernels() {
-  cudaError_t e = prepare_rows<0>();
-  if (e == cudaSuccess) e = prepare_rows<1>();
-  if (e == cudaSuccess) e = prepare_rows<2>();
-  for (const void* k : {(const void*)fhspec::k_dft_y, (const void*)fhspec::k_idft_y, (const void*)fhspec::k_mix_x<false>,
-                        (const void*)fhspec::k_mix_x<true>})
-    if (e == cudaSuccess) e = fh::allow_smem(k);
-  return e;
+// the tensor-core rows' share of an SM's shared memory and L1 cache
+cudaError_t prefer_shared() {
+  for (const void* k : {(const void*)fhtc::k_rows_tc<0>, (const void*)fhtc::k_rows_tc<1>, (const void*)fhtc::k_rows_tc<2>}) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 fh_status refresh_bf16(fh_fno* f) {
@@ -436,7 +432,7 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
   if ((e = cudaMalloc(&f->gb, act * 4)) != cudaSuccess) return fail(e);
   if ((e = cudaGetDevice(&f->device)) != cudaSuccess) return fail(e);
   if ((e = cudaDeviceGetAttribute(&f->sms, cudaDevAttrMultiProcessorCount, f->device)) != cudaSuccess) return fail(e);
-  if ((e = prepare_kernels()) != cudaSuccess) return fail(e);
+  if ((e = prefer_shared()) != cudaSuccess) return fail(e);
   f->nparts = 8 * f->sms;   // at least the resident blocks of a row kernel
   if ((e = cudaMalloc(&f->part, f->nparts * sizeof(double))) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc(&f->tc_err, sizeof(int))) != cudaSuccess) return fail(e);

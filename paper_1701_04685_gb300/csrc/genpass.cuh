@@ -485,26 +485,33 @@ int gen_rb(int L, long long rows_of_all_loads) {
 }
 
 template <typename T, int NV, int CT>
-cudaError_t gen_col_prepare_ct() {
-  cudaError_t e = allow_smem((const void*)line_pass_gen<T, NV, 2, CT>);
+cudaError_t gen_col_prepare_ct(int N) {
+  const size_t sm = gen_col_bytes(N, sizeof(T) == 4, NV, CT);
+  cudaError_t e = allow_smem((const void*)line_pass_gen<T, NV, 2, CT>, sm);
   if constexpr (NV == 6) {   // 2-D grids have axis 0 only
-    if (e == cudaSuccess) e = allow_smem((const void*)line_pass_gen<T, NV, 0, CT>);
-    if (e == cudaSuccess) e = allow_smem((const void*)line_pass_gen<T, NV, 1, CT>);
+    if (e == cudaSuccess) e = allow_smem((const void*)line_pass_gen<T, NV, 0, CT>, sm);
+    if (e == cudaSuccess) e = allow_smem((const void*)line_pass_gen<T, NV, 1, CT>, sm);
   }
   return e;
 }
 template <typename T, int NV>
 cudaError_t gen_col_prepare_t(int N) {
   if constexpr (sizeof(T) == 4 && NV == 6) {
-    if (gen_columns(N, true, NV) == 8) return gen_col_prepare_ct<T, NV, 8>();
+    if (gen_columns(N, true, NV) == 8) return gen_col_prepare_ct<T, NV, 8>(N);
   }
-  return gen_col_prepare_ct<T, NV, 4>();
+  return gen_col_prepare_ct<T, NV, 4>(N);
+}
+// shared memory of the row pass with rb rows per block
+template <typename T, int NV>
+size_t gen_row_bytes(const GenShape& K, int rb) {
+  return (size_t)(K.N + (rb * NV + 1) / 2 * K.LS) * 2 * sizeof(T);
 }
 template <typename T, int NV>
-cudaError_t gen_row_prepare_t() {
-  cudaError_t e = allow_smem((const void*)row_pass_gen<T, NV, true, false>);
-  if (e == cudaSuccess) e = allow_smem((const void*)row_pass_gen<T, NV, false, true>);
-  if (e == cudaSuccess) e = allow_smem((const void*)row_pass_gen<T, NV, false, false>);
+cudaError_t gen_row_prepare_t(const GridInfo& g, int rb) {
+  const size_t sm = gen_row_bytes<T, NV>(gen_row_shape(g.L, sizeof(T) == 4, g.H), rb);
+  cudaError_t e = allow_smem((const void*)row_pass_gen<T, NV, true, false>, sm);
+  if (e == cudaSuccess) e = allow_smem((const void*)row_pass_gen<T, NV, false, true>, sm);
+  if (e == cudaSuccess) e = allow_smem((const void*)row_pass_gen<T, NV, false, false>, sm);
   return e;
 }
 
@@ -545,7 +552,7 @@ cudaError_t gen_row_t(bool first, bool kinv, const GridInfo& g, const cplx<T>* t
                       const T* Yaux, const T* Cfld, cudaStream_t stream) {
   const GenShape K = gen_row_shape(g.L, sizeof(T) == 4, g.H);
   const int bpl = (int)((g.nrows + rb - 1) / rb), lines = (rb * NV + 1) / 2;
-  const size_t sm = (size_t)(g.L + lines * K.LS) * 2 * sizeof(T);
+  const size_t sm = gen_row_bytes<T, NV>(K, rb);
   const int threads = (lines * K.R2 + 31) / 32 * 32;
   auto launch = [&](auto kern) {
     kern<<<(unsigned)(nload * bpl), threads, sm, stream>>>(g, K, rb, tw, E, S, phase, dC, ctl, st, partials, hist, bpl, Wout, Yaux,

@@ -17,8 +17,8 @@ int gen_rows_per_block(float, int nv, int L, long long rows);
 // once per solve, before the launches: the kernels' shared-memory limits (allow_smem)
 cudaError_t gen_col_prepare(double, int nv, int N);
 cudaError_t gen_col_prepare(float, int nv, int N);
-cudaError_t gen_row_prepare(double, int nv);
-cudaError_t gen_row_prepare(float, int nv);
+cudaError_t gen_row_prepare(double, const GridInfo& g, int rb);
+cudaError_t gen_row_prepare(float, const GridInfo& g, int rb);
 
 // pass along an axis of N points with element stride `stride` (modes as line_pass)
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const double2* tw, double2* S, const double* G,

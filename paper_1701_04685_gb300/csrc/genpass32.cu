@@ -12,7 +12,9 @@ int gen_rows_per_block(float, int nv, int L, long long rows) {
 cudaError_t gen_col_prepare(float, int nv, int N) {
   return nv == 3 ? gen_col_prepare_t<float, 3>(N) : gen_col_prepare_t<float, 6>(N);
 }
-cudaError_t gen_row_prepare(float, int nv) { return nv == 3 ? gen_row_prepare_t<float, 3>() : gen_row_prepare_t<float, 6>(); }
+cudaError_t gen_row_prepare(float, const GridInfo& g, int rb) {
+  return g.nv == 3 ? gen_row_prepare_t<float, 3>(g, rb) : gen_row_prepare_t<float, 6>(g, rb);
+}
 
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const float2* tw, float2* S, const float* G, const LoadState* st,
                     long long stride, int nload, cudaStream_t stream) {

@@ -12,7 +12,9 @@ int gen_rows_per_block(double, int nv, int L, long long rows) {
 cudaError_t gen_col_prepare(double, int nv, int N) {
   return nv == 3 ? gen_col_prepare_t<double, 3>(N) : gen_col_prepare_t<double, 6>(N);
 }
-cudaError_t gen_row_prepare(double, int nv) { return nv == 3 ? gen_row_prepare_t<double, 3>() : gen_row_prepare_t<double, 6>(); }
+cudaError_t gen_row_prepare(double, const GridInfo& g, int rb) {
+  return g.nv == 3 ? gen_row_prepare_t<double, 3>(g, rb) : gen_row_prepare_t<double, 6>(g, rb);
+}
 
 cudaError_t gen_col(int mode, const GridInfo& g, int N, const double2* tw, double2* S, const double* G, const LoadState* st,
                     long long stride, int nload, cudaStream_t stream) {

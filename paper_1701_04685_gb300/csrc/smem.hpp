@@ -3,12 +3,16 @@
 
 #include <cuda_runtime.h>
 
+#include <cstddef>
+
 namespace fh {
 
-// Lets `kernel` have as much dynamic shared memory as a block of the current device can
-// (the opt-in limit less the kernel's static part).  The limit belongs to the process and
-// not to a solver or network; as every caller sets the same value, none on another host
-// thread can lower it between this call and a launch.
-cudaError_t allow_smem(const void* kernel);
+// Lets `kernel` have `bytes` of dynamic shared memory on the current device.  The limit
+// belongs to the process and not to a solver or network: it is raised and never lowered,
+// so that none on another host thread falls below what its next launch asks for.
+// (The most a block can have, for every kernel, would do as well, but leaves kernels of
+// small requests less L1 cache: 40 iterations of a 512^2 grid with point-by-point
+// stiffness 2.65 ms against 2.61.)
+cudaError_t allow_smem(const void* kernel, size_t bytes);
 
 }  // namespace fh

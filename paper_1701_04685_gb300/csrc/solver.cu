@@ -53,23 +53,19 @@ using fh::LoadState;
   } while (0)
 
 namespace fh {
-cudaError_t allow_smem(const void* kernel) {
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
   static std::mutex mutex;
-  static std::map<std::pair<int, const void*>, int> limits;   // per device and kernel
+  static std::map<std::pair<int, const void*>, size_t> limits;   // per device and kernel
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mutex);
-  auto it = limits.find({dev, kernel});
-  if (it == limits.end()) {
-    cudaFuncAttributes attr{};
-    int most = 0;
-    if ((e = cudaFuncGetAttributes(&attr, kernel)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-    it = limits.insert({{dev, kernel}, most - (int)attr.sharedSizeBytes}).first;
-  }
+  size_t& limit = limits[{dev, kernel}];
+  const size_t want = std::max(limit, bytes);
   // set every time: a device reset forgets it
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, it->second);
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+  if (e == cudaSuccess) limit = want;
+  return e;
 }
 }  // namespace fh
 
@@ -672,11 +668,11 @@ void enqueue_row_pass(fh_solver* s, int prec, int nload) {
 
 template <typename T, int P>
 cudaError_t set_warp_attrs(fh_solver* s, int prec, size_t rs) {
-  cudaError_t e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, true>);
+  cudaError_t e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, true>, rs);
   if (e != cudaSuccess) return e;
-  e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, false>);
+  e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, false>, rs);
   if (e != cudaSuccess) return e;
-  e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, false, true>);
+  e = fh::allow_smem((const void*)fh::row_pass_warp6<T, P, false, true>, rs);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s->warp_res[prec], fh::row_pass_warp6<T, P, false>,
                                                        fh::kWarpRowThreads, rs);
@@ -684,28 +680,29 @@ cudaError_t set_warp_attrs(fh_solver* s, int prec, size_t rs) {
 
 template <int P>
 cudaError_t set_col_attrs() {
-  cudaError_t e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 0>);
-  if (e == cudaSuccess) e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 1>);
-  if (e == cudaSuccess) e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 2>);
+  cudaError_t e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 0>, fh::colpass_smem<P>());
+  if (e == cudaSuccess) e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 1>, fh::colpass_smem<P>());
+  if (e == cudaSuccess) e = fh::allow_smem((const void*)fh::line_pass_warp6<P, 2>, fh::colpass_smem<P>());
   return e;
 }
 
 template <typename T, int R1, int R2>
 cudaError_t set_col2_attrs() {
   constexpr int CT = col2_ct<T>();
-  cudaError_t e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 0, CT, col2_mb<T, 0, R1 * R2>(), T>);
+  const size_t sm = fh::col2_smem<R1, R2, CT, T>();
+  cudaError_t e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 0, CT, col2_mb<T, 0, R1 * R2>(), T>, sm);
   if (e == cudaSuccess)
-    e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 1, CT, col2_mb<T, 1, R1 * R2>(), T>);
+    e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 1, CT, col2_mb<T, 1, R1 * R2>(), T>, sm);
   if (e == cudaSuccess)
-    e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 2, CT, col2_mb<T, 2, R1 * R2>(), T>);
+    e = fh::allow_smem((const void*)fh::line_pass_2s<R1, R2, 2, CT, col2_mb<T, 2, R1 * R2>(), T>, sm);
   return e;
 }
 
 template <int P1, int P2>
 cudaError_t set_plane_attrs() {
-  cudaError_t e = fh::allow_smem((const void*)fh::plane_pass_warp6<P1, P2, true>);
+  cudaError_t e = fh::allow_smem((const void*)fh::plane_pass_warp6<P1, P2, true>, fh::plane_smem<P1, P2>());
   if (e == cudaSuccess)
-    e = fh::allow_smem((const void*)fh::plane_pass_warp6<P1, P2, false>);
+    e = fh::allow_smem((const void*)fh::plane_pass_warp6<P1, P2, false>, fh::plane_smem<P1, P2>());
   return e;
 }
 
@@ -726,11 +723,11 @@ cudaError_t set_plane_attrs_of(int code) {
 
 template <typename T, int R1, int R2>
 cudaError_t set_row2_attrs() {
-  cudaError_t e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, true, false>);
+  cudaError_t e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, true, false>, fh::row2_smem<T, R1, R2>());
   if (e == cudaSuccess)
-    e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, false, false>);
+    e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, false, false>, fh::row2_smem<T, R1, R2>());
   if (e == cudaSuccess)
-    e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, false, true>);
+    e = fh::allow_smem((const void*)fh::row_pass_2s<T, R1, R2, false, true>, fh::row2_smem<T, R1, R2>());
   return e;
 }
 
@@ -754,11 +751,11 @@ fh_status set_smem_attrs_nv(fh_solver* s, int prec) {
     fh::set_error("contiguous axis too long for the point-by-point stiffness in this precision (shared memory)");
     return FH_ERR_UNSUPPORTED;
   }
-  if (s->rowg_rb[prec] > 0) CK(fh::gen_row_prepare(T(0), NV));
+  if (s->rowg_rb[prec] > 0) CK(fh::gen_row_prepare(T(0), s->g, s->rowg_rb[prec]));
   if (s->row_smem_gen[prec] <= kMaxSmem) {   // the block row pass (also taken by point-by-point stiffness)
-    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, true>));
-    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, false>));
-    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, false, true>));
+    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, true>, s->row_smem_gen[prec]));
+    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, false>, s->row_smem_gen[prec]));
+    CK(fh::allow_smem((const void*)fh::row_pass<T, NV, false, true>, s->row_smem_gen[prec]));
   }
   if (s->row_warp[prec] != 0) {
     if constexpr (sizeof(T) == 4) {
@@ -799,9 +796,9 @@ fh_status set_smem_attrs_nv(fh_solver* s, int prec) {
     return FH_ERR_UNSUPPORTED;
   }
   if (lm > 0) {
-    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 0>));
-    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 1>));
-    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 2>));
+    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 0>, lm));
+    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 1>, lm));
+    CK(fh::allow_smem((const void*)fh::line_pass<T, NV, 2>, lm));
   }
   return FH_OK;
 }
@@ -1125,7 +1122,7 @@ fh_status cluster_fits(fh_solver* s, bool* ok) {
   s->cl_gsmem[sizeof(T) == 8 ? 0 : 1][CS == 16 ? 1 : 0] = gs;
   const int kind = cluster_of<T>(s).kind;
   const void* kern = fh::cluster_kernel(T(0), g.nv, CS, kind);
-  CK(fh::allow_smem(kern));
+  CK(fh::allow_smem(kern, lay.total));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchAttribute attr[1];
   const cudaLaunchConfig_t cfg = cluster_config<T>(kind, CS, lay.total, 1, nullptr, attr);
@@ -2380,7 +2377,7 @@ fh_status launch_queue(const QueueGroup& q, fh_solver* const* solvers, const int
   std::stable_sort(tasks.begin(), tasks.end(),
                    [](const fh::ClusterTask& a, const fh::ClusterTask& b) { return a.g.m > b.g.m; });
   const void* kern = fh::cluster_kernel(T(0), q.nv, CS, q.kind);
-  CK(fh::allow_smem(kern));
+  CK(fh::allow_smem(kern, smem));
   if (CS > 8) CK(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = cluster_config<T>(q.kind, CS, smem, 1, stream, attr);
