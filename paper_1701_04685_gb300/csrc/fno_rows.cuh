@@ -120,20 +120,18 @@ __device__ __forceinline__ void outer84(float (&acc)[8][4], const float4 a0, con
   }
 }
 
-// e^2 to the float pair (hi, lo) of at most 32 squares (TwoSum / TwoProduct: an FP64
-// multiply-add per element is a large part of the last layer's time), or in FP64 where
-// the square or its rounding error leaves FP32's range
-__device__ __forceinline__ void add_square(float e, float& hi, float& lo, double& sum) {
-  const float m = fabsf(e);
-  if (m < 0x1p61f && (m >= 0x1p-51f || m == 0.f)) {
-    const float pr = e * e, er = fmaf(e, e, -pr);
-    const float hs = hi + pr, bp = hs - hi;
-    lo += ((hi - (hs - bp)) + (pr - bp)) + er;
-    hi = hs;
-  } else {
-    sum += (double)e * e;
-  }
+// e^2 to the float pair (hi, lo) (TwoSum / TwoProduct: an FP64 multiply-add per element
+// is a large part of the last layer's time)
+__device__ __forceinline__ void add_square(float e, float& hi, float& lo) {
+  const float pr = e * e, er = fmaf(e, e, -pr);
+  const float hs = hi + pr, bp = hs - hi;
+  lo += ((hi - (hs - bp)) + (pr - bp)) + er;
+  hi = hs;
 }
+// the pair of at most 32 squares holds their sum: no square has left FP32's range (the
+// sum would be infinite or NaN), and those whose rounding errors have (below 2^-102) are
+// less than 2^-37 of it
+__device__ __forceinline__ bool pair_holds(float hi) { return hi >= 0x1p-60f && hi < 0x1p126f; }
 
 template <int EPI>
 __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
@@ -281,7 +279,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
         }
       }
     }
-    if (a.Q) {
+    if (EPI == 1 && a.Q) {   // the projection follows a hidden layer only
       const int nqg = a.QP >> 3;
       for (int t = tid; t < nr * nqg * nz4; t += kRowThreads) {
         const int rr = udiv(t, a.dQt), rm = t - rr * a.dQt.d;
@@ -317,15 +315,24 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
           for (int j = 0; j < 4; ++j) {
             const float e = s[i][j] - tq[j];
             g[j] = 2.f * e * a.inv_count;
-            if (j < zn2) add_square(e, ehi, elo, esum);
+            s[i][j] = e;
+            if (j < zn2) add_square(e, ehi, elo);
           }
           store4(a.gy + p, make_float4(g[0], g[1], g[2], g[3]), zn2, a.vec);
         }
-        esum += (double)ehi + (double)elo;
+        if (pair_holds(ehi)) {
+          esum += (double)ehi + (double)elo;
+        } else if (a.target) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (8 * qg + i < a.cout && j < zn2) esum += (double)s[i][j] * s[i][j];
+        }
       }
     }
   }
-  if (a.Q && a.target) {
+  if (EPI == 1 && a.Q && a.target) {
     __shared__ double red[kRowThreads / 32];
     double v = esum;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
