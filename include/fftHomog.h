@@ -376,7 +376,10 @@ fh_status fh_mean_stress_noalloc(int d, long long m, int nload, const double* E,
  * Arrays x [batch][cin][n^3], y and targets [batch][cout][n^3] are device FP32.
  * The parameter vector (host FP32) is, in order: P[width][cin], p[width],
  * W[layers][width][width], w[layers][width], Re R[layers][2m][2m][m][width][width],
- * Im R[...], Q[cout][width], q[cout]. */
+ * Im R[...], Q[cout][width], q[cout].
+ * Sizes: 4 <= n <= 128, channels and max_batch 1..64, 2 modes <= n, layers 1..8
+ * (else FH_ERR_ARG) and width (width + 2 max_batch) <= 3632 (else
+ * FH_ERR_UNSUPPORTED). */
 typedef struct fh_fno fh_fno;
 fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int layers, int max_batch,
                         void* cuda_stream, fh_fno** out);

@@ -389,6 +389,11 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
     fh::set_error("FNO sizes out of range (n<=128, channels<=64, 2*modes<=n, layers<=8, batch<=64)");
     return FH_ERR_ARG;
   }
+  // a limit of the interface, not of the kernels (which go further)
+  if (width * (width + 2 * max_batch) > 3632) {
+    fh::set_error("FNO width/batch too large: width (width + 2 max_batch) must not exceed 3632");
+    return FH_ERR_UNSUPPORTED;
+  }
   fh_fno* f = new fh_fno();
   FnoDims& d = f->d;
   d.N = n; d.cin = cin; d.cout = cout; d.W = width; d.m = modes; d.L = layers;
@@ -441,15 +446,6 @@ fh_status fh_fno_create(int n, int cin, int cout, int width, int modes, int laye
   cudaMemset(f->grd, 0, o * 4);
   cudaMemset(f->m1, 0, o * 4);
   cudaMemset(f->m2, 0, o * 4);
-  // sizes beyond these were never offered (they also bound the shared memory of the kernels)
-  constexpr int KC = 8;
-  const size_t sm_mb = (size_t)KC * width * width * 8 + (size_t)2 * max_batch * KC * width * 8;
-  const size_t sm_zy = (size_t)n * n * 4 + (size_t)n * 8 + (size_t)n * modes * 8;
-  if (sm_mb > 227 * 1024 || sm_zy > 227 * 1024) {
-    fh::set_error("FNO width/batch/grid too large for the shared-memory tiles");
-    fh_fno_destroy(f);
-    return FH_ERR_UNSUPPORTED;
-  }
   std::vector<float2> tw(n);
   for (int t = 0; t < n; ++t) {
     const long double a = 2.0L * 3.141592653589793238462643383279502884L * t / n;

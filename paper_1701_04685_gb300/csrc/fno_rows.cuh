@@ -50,7 +50,7 @@ struct RowArgs {
   int nrows, rpb;      // rows in all, rows per block
   int vec;             // rows and pointers allow 16-byte accesses
   int kc;              // rows of the activation tile, max(Cin, W)
-  UDiv dN, dNq, dCin, dW, dm2W, dTask, dOg, dCg, dKg, dQt, dQg;
+  UDiv dNq, dCin, dTask, dOg, dCg, dKg, dQt, dQg;
   const float* in;     // [b][Cin][N3]
   const void* A;       // [W][Cin], or [Cin][W] when a_trans
   int a_bf16, a_trans;
