@@ -350,11 +350,16 @@ fh_status forward_all(fh_fno* f, int B, const float* x, float* y, const float* t
 fh_status weight_grad(fh_fno* f, int B, int cin, int cout, const float* g, const float* x, long long off_A, long long off_b) {
   const FnoDims& d = f->d;
   const int total = B * d.N3;   // at most 64 * 128^3
-  const int tiles = ((cout + 31) / 32) * ((cin + 31) / 32);
+  const int to = cout <= 8 ? 8 : 32, tc = cin <= 8 ? 8 : 32;
+  const int tiles = ((cout + to - 1) / to) * ((cin + tc - 1) / tc);
   const int chunks = (total + fhrow::kWgVox - 1) / fhrow::kWgVox;
   const int vec = d.N3 % 4 == 0 && aligned16(g) && aligned16(x);
   const dim3 grid(std::min(chunks, 2 * f->sms), tiles);
-  fhrow::k_weight_grad<<<grid, fhrow::kWgThreads, 0, f->stream>>>(total, d.N3, cin, cout, vec, g, x, f->grd + off_A, f->grd + off_b);
+  auto launch = [&](auto kernel) {
+    kernel<<<grid, fhrow::kWgThreads, 0, f->stream>>>(total, d.N3, cin, cout, vec, g, x, f->grd + off_A, f->grd + off_b);
+  };
+  if (to == 8) launch(tc == 8 ? fhrow::k_weight_grad<8, 8> : fhrow::k_weight_grad<8, 32>);
+  else launch(tc == 8 ? fhrow::k_weight_grad<32, 8> : fhrow::k_weight_grad<32, 32>);
   FCK(cudaGetLastError());
   return FH_OK;
 }
