@@ -206,7 +206,11 @@ fh_status launch_rows(fh_fno* f, fhrow::RowArgs& a, int* blocks = nullptr) {
 
 // The tensor-core form takes the hidden layers (BF16 weights, spectral input, no
 // projection) of 32 channels on rows of 16 .. 128 points, a multiple of 16, whose
-// operands fit a CTA's shared memory.
+// operands fit a CTA's shared memory.  Its tile is written for that width, the learned
+// start's: four rows of 32 channels are the 128 lines of an MMA.  16 channels would take
+// eight rows a tile (and twice the spectral operand), which is not written: their SIMT
+// rows halve the time of the former layers, whose 1 x 1 products alone ran on the tensor
+// cores (64^3, 12 modes, four samples: forward 2.35 -> 0.96 ms).
 bool use_tc(const fh_fno* f, const fhrow::RowArgs& a) {
   const FnoDims& d = f->d;
   const int Kp = (2 * d.m + 15) & ~15;
@@ -342,7 +346,7 @@ fh_status forward_all(fh_fno* f, int B, const float* x, float* y, const float* t
         a.y = y;
       }
     }
-    rc = hidden_rows<1>(f, a, blocks);
+    rc = a.target ? launch_rows<3>(f, a, blocks) : hidden_rows<1>(f, a, blocks);
   }
   return rc;
 }

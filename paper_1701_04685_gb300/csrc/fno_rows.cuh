@@ -58,17 +58,17 @@ struct RowArgs {
   const float* Iy;     // [row][m2][W] or null
   const float* T;      // [m2][N]
   const float* u_in;   // gelu' argument [b][W][N3] (EPI 2)
-  float* u_out;        // pre-activation (EPI 1) or null
+  float* u_out;        // pre-activation (EPI 1, 3) or null
   float* out;          // [b][W][N3] or null
   float* Yz;           // [row][m2][W] or null
   // projection
   const float* Q;      // [cout][W] or null
   const float* qb;
   int cout, QP;
-  float* y;            // [b][cout][N3], or with target: null
-  const float* target; // [b][cout][N3] or null
-  float* gy;           // 2 (y - target) inv_count
-  double* part;        // one block sum of (y - target)^2 per block
+  float* y;            // [b][cout][N3] (EPI 1)
+  const float* target; // [b][cout][N3] (EPI 3)
+  float* gy;           // 2 (y - target) inv_count (EPI 3)
+  double* part;        // one block sum of (y - target)^2 per block (EPI 3)
   float inv_count;
 };
 
@@ -133,6 +133,9 @@ __device__ __forceinline__ void add_square(float e, float& hi, float& lo) {
 // less than 2^-37 of it
 __device__ __forceinline__ bool pair_holds(float hi) { return hi >= 0x1p-60f && hi < 0x1p126f; }
 
+// EPI 0: the identity, 1: the GELU (with the projection y where Q is given), 2: the
+// product with gelu'(u), 3: the GELU with the projection, the squared errors and their
+// gradient (training's last layer)
 template <int EPI>
 __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
   extern __shared__ __align__(16) float smf[];
@@ -161,6 +164,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
       const int c = i / a.QP, q = i - c * a.QP;
       sQ[i] = q < a.cout ? a.Q[q * a.W + c] : 0.f;
     }
+  constexpr bool PROJ = EPI == 1 || EPI == 3, LOSS = EPI == 3;
   double esum = 0.0;   // this thread's squared errors
   const int ntiles = (a.nrows + a.rpb - 1) / a.rpb;
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -215,7 +219,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
         const int o = 8 * og + i;
         if (o >= a.W) break;
         const size_t p = base + (size_t)o * a.N3;
-        if (EPI == 1) {
+        if (EPI == 1 || EPI == 3) {
           if (a.u_out) store4(a.u_out + p, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]), zn, a.vec);
 #pragma unroll
           for (int j = 0; j < 4; ++j) acc[i][j] = row_gelu(acc[i][j]);
@@ -279,7 +283,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
         }
       }
     }
-    if (EPI == 1 && a.Q) {   // the projection follows a hidden layer only
+    if (PROJ && a.Q) {
       const int nqg = a.QP >> 3;
       for (int t = tid; t < nr * nqg * nz4; t += kRowThreads) {
         const int rr = udiv(t, a.dQt), rm = t - rr * a.dQt.d;
@@ -304,7 +308,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
           const int q = 8 * qg + i;
           if (q >= a.cout) break;
           const size_t p = base + (size_t)q * a.N3;
-          if (!a.target) {
+          if (!LOSS) {
             store4(a.y + p, make_float4(s[i][0], s[i][1], s[i][2], s[i][3]), zn2, a.vec);
             continue;
           }
@@ -320,9 +324,10 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
           }
           store4(a.gy + p, make_float4(g[0], g[1], g[2], g[3]), zn2, a.vec);
         }
+        if (!LOSS) continue;
         if (pair_holds(ehi)) {
           esum += (double)ehi + (double)elo;
-        } else if (a.target) {
+        } else {
 #pragma unroll
           for (int i = 0; i < 8; ++i)
 #pragma unroll
@@ -332,7 +337,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
       }
     }
   }
-  if (EPI == 1 && a.Q && a.target) {
+  if (LOSS) {
     __shared__ double red[kRowThreads / 32];
     double v = esum;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
