@@ -212,9 +212,8 @@ fh_status fh_pattern_half_freqs(const fh_pattern* p, int64_t* h, int64_t* nh);
 /* Solver for one pattern and generator on one CUDA stream (cudaStream_t,
  * NULL = legacy default stream).  Allocates device work memory for up to
  * nload_max load cases (1..FH_MAX_LOADS).  The pattern may be destroyed
- * afterwards.  Every axis length up to 4096 is supported: radices 2, 3, 4,
- * 5, 8 are written out, 7, 11, 13 and any larger prime factor run as direct
- * DFT stages (slower for large primes).  Errors: FH_ERR_ARG,
+ * afterwards.  Every axis length up to 4096 is supported; prime factors above 13
+ * run as direct DFT stages (slower for large primes).  Errors: FH_ERR_ARG,
  * FH_ERR_UNSUPPORTED (an SNF axis longer than 4096, or |det M| = 1: a single point has
  * no fluctuation, E = 0 and C_eff = C there), FH_ERR_CUDA. */
 fh_status fh_solver_create(const fh_pattern* p, const fh_generator* gen,

@@ -11,10 +11,12 @@
 // quarter of the SM 64 cycles, and one warp's two steps use one quarter only (96^2
 // 48.7 against 53.6 us).
 //
-// fft_lines_big, for the other lengths: the Stockham stages of fft.cuh with every radix from 2 to 16 (gendft.cuh),
-// so that most lengths need two stages and none below 4096 more than four (96 = 8 x
-// 12, 192 = 12 x 16, 768 = 8 x 8 x 12, where the schedule of 8, 4, 2, 3, ... has
-// three to five), plus the direct stage for larger primes.
+// fft_lines_big, for the other lengths of the general variant: the Stockham stages of
+// fft.cuh with every radix from 2 to 16 (gendft.cuh), so that most lengths need two
+// stages and none below 4096 more than four (96 = 8 x 12, 192 = 12 x 16, 768 = 8 x 8 x
+// 12, where the schedule of 8, 4, 2, 3, ... has three to five), plus the direct stage
+// for larger primes.  A called stage costs about 700 cycles more than an inlined one, so
+// that clusterplan.cpp sends the lengths that gain less to the staged variant.
 //
 // A stage deals its butterflies line by line across the lanes: with the odd line
 // strides of the cluster layout every access is free of bank conflicts and a warp's

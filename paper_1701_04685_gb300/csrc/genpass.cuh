@@ -10,7 +10,7 @@
 // times (rows), where the general block passes run three or more Stockham stages
 // with all index arithmetic, twiddle reads from global memory and a barrier each.
 // Index divisions are one multiplication per R points.  100^3 x 6 loads in FP32:
-// 0.6 ms an iteration against 2.6 ms (a solve of 20 iterations 13.6 against 53.6 ms).
+// 0.55 ms an iteration against 2.6 ms (a solve of 20 iterations 12.4 against 53.5 ms).
 //
 // Line layout: row k1 at offset (R2 | 1) k1, so that its stride is odd.  Column
 // tiles: CT = 8 columns a block in FP32 3-D as far as shared memory goes (N <= 512),
@@ -18,7 +18,8 @@
 // 771 columns).  Row lines: stride R2 mod 16, so that consecutive entries of
 // consecutive lines follow one another.
 // 512^2 x 3 loads FP32 with point-by-point stiffness: 63 us an iteration against
-// 132 us (block row pass 79, block line pass 53).
+// 132 us (block row pass 79, block line pass 53).  Four columns at 640 points (2 x 640 x
+// 640 x 6 loads, axis-1 pass): 85 us against 303 us for the block line pass.
 #pragma once
 
 #include "genpass.hpp"

@@ -2355,7 +2355,7 @@ fh_status finish_deferred(fh_solver* s, int nload, PhaseOut* out) {
 }
 
 // One queue launch for every (solver, load) of a group of deferred cluster
-// solves that share precision, n_v, cluster size and radix variant; tasks are
+// solves that share precision, n_v, cluster size and kind; tasks are
 // ordered largest pattern first, and as many clusters as fit stay resident.
 struct QueueGroup {
   int prec, nv, cs;
