@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) k_rows(const RowArgs a) {
         int vo[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) vo[j] = cg + j * ncg < a.W ? j * ncg * a.NS : 0;
-#pragma unroll 2
+#pragma unroll 1   // unrolled twice, every instance but EPI 2 spills (64^3, width 16, two samples: 530 against 522 us)
         for (int q = 0; q < a.N4; q += 4) {
           float4 x[4], y[4];
 #pragma unroll
